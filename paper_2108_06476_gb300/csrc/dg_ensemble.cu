@@ -16,8 +16,8 @@
 //      u_out <- u_in + B k.
 // Phase B reads only its own elements' states (the faces were read in phase
 // A), so u_out may be u_in: a step updates the state in place. The arithmetic
-// is that of dg_rhs: the same device functions (face_flux, volume_batch,
-// and their FP32 perturbation forms), with each member's own split-form
+// is that of dg_rhs: the same device functions (face_flux, fx_batch, and the
+// FP32 perturbation forms), with each member's own split-form
 // tables. The barrier's wait is bounded (about one second); if it runs out,
 // the launch sets the timeout bit of the error word and skips phase B, and
 // dg_ensemble_check reports DG_ERR_TIMEOUT.
@@ -43,7 +43,7 @@ namespace {
 using namespace dg;
 
 constexpr int kEnsMinN = 3, kEnsMaxN = 5;
-constexpr int kEnsMaxItem = 32;          // elements per work item
+constexpr int kEnsMaxItem = 8;           // elements per work item (128 threads / 16 lines)
 constexpr unsigned kErrTimeout = 8u;     // error-word bit: a bounded wait gave up
 
 struct SimDesc {
@@ -76,7 +76,7 @@ struct EnsArgs {
   const void* tables;  // per member Tables<R>
   unsigned* err;
   unsigned* bar;       // barrier counter, zero at launch
-  int pair;            // FP64: phase B pair-parallel (see ens_volume_pp)
+  int pair;            // FP64: phase B one element at a time (see ens_volume_pp)
 };
 
 int fail(int code, const char* msg) { return dg::set_last_error(code, msg); }
@@ -163,7 +163,8 @@ __device__ void ens_faces(const EnsArgs& a, const SimDesc& sd, const WorkItem& w
 // phase B of one item: volume term, lifting and the stage update
 template <typename R, int N>
 __device__ void ens_volume(const EnsArgs& a, const SimDesc& sd, const WorkItem& w,
-                           const Tables<R>& tb, unsigned char* smem) {
+                           const Tables<R>& tb, unsigned char* smem,
+                           FxShared<3, sizeof(R) == 8 ? kEnsMaxItem : 1>& sh) {
   const Geom g = member_geom(sd, a);
   StageFuse fz;
   fz.k = a.k + sd.off;
@@ -178,17 +179,16 @@ __device__ void ens_volume(const EnsArgs& a, const SimDesc& sd, const WorkItem& 
     volume_batch32<3, N, kVRanocha, kEnsMaxItem>(u, nullptr, static_cast<const float*>(a.fs) + sd.fsoff,
                                                  g, tb, a.err, fz, w.e0, w.count, smem);
   else
-    volume_batch<3, N, R, kVRanocha, kEnsMaxItem>(u, nullptr, static_cast<const R*>(a.fs) + sd.fsoff,
-                                                  g, tb, a.err, fz, w.e0, w.count, smem);
+    fx_batch<3, N, kEnsMaxItem>(u, nullptr, static_cast<const R*>(a.fs) + sd.fsoff, g, tb, a.err,
+                                fz, w.e0, w.count, smem, sh);
 }
 
-// phase B of one item, pair-parallel (FP64): the item's elements one after
-// another, each with the whole CTA: one thread per (line, node pair) of a
-// direction evaluates the pair flux into shared memory, then one thread per
-// node sums its line in the line-owning order (bitwise the same result)
+// phase B of one item with the whole CTA on one element after another (FP64;
+// bitwise the same result)
 template <int N>
 __device__ void ens_volume_pp(const EnsArgs& a, const SimDesc& sd, const WorkItem& w,
-                              const Tables<double>& tb, unsigned char* smem) {
+                              const Tables<double>& tb, unsigned char* smem,
+                              FxShared<3, kEnsMaxItem>& sh) {
   const Geom g = member_geom(sd, a);
   StageFuse fz;
   fz.k = a.k + sd.off;
@@ -198,19 +198,23 @@ __device__ void ens_volume_pp(const EnsArgs& a, const SimDesc& sd, const WorkIte
   fz.u_out = a.uout + sd.off;
   double* u = const_cast<double*>(a.uin) + sd.off;
   const double* fs = static_cast<const double*>(a.fs) + sd.fsoff;
-  for (int el = 0; el < w.count; ++el)
-    pp_elements<3, N, kVRanocha, false, 1, 1, true>(u, nullptr, fs, g, tb, a.err, fz, 0, w.e0 + el, 1,
-                                              smem);
+  for (int el = 0; el < w.count; ++el) {
+    fx_batch<3, N, kEnsMaxItem, true>(u, nullptr, fs, g, tb, a.err, fz, w.e0 + el, 1, smem, sh);
+    __syncthreads();
+  }
 }
 
 // one cooperative launch per stage: blocks walk the work list (largest
-// degrees first) in each phase; CTAs of at most 128 threads, at least three
-// resident per SM (at most 168 registers a thread)
+// degrees first) in each phase; CTAs of at most 128 threads. FP64: 80 registers
+// a thread, so that six CTAs fit an SM (48 members: 154 ms per step with one
+// thread per line in FP64 at 168 registers, 71 ms in fixed point); FP32: at
+// most 168, three CTAs.
 constexpr int kEnsMaxThreads = 128;
 template <typename R>
-__global__ void __launch_bounds__(kEnsMaxThreads, 3) ensemble_stage_kernel(EnsArgs a) {
+__global__ void __launch_bounds__(kEnsMaxThreads, sizeof(R) == 8 ? 6 : 3) ensemble_stage_kernel(EnsArgs a) {
   extern __shared__ __align__(16) unsigned char dg_smem[];
   __shared__ Tables<R> s_tb;
+  __shared__ FxShared<3, sizeof(R) == 8 ? kEnsMaxItem : 1> s_fx;
   for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
     const WorkItem w = a.items[it];
     const SimDesc sd = a.sims[w.sim];
@@ -235,15 +239,15 @@ __global__ void __launch_bounds__(kEnsMaxThreads, 3) ensemble_stage_kernel(EnsAr
     __syncthreads();
     if constexpr (sizeof(R) == 8) {
       if (a.pair) {
-        if (sd.N == 3) ens_volume_pp<3>(a, sd, w, s_tb, dg_smem);
-        else if (sd.N == 4) ens_volume_pp<4>(a, sd, w, s_tb, dg_smem);
-        else ens_volume_pp<5>(a, sd, w, s_tb, dg_smem);
+        if (sd.N == 3) ens_volume_pp<3>(a, sd, w, s_tb, dg_smem, s_fx);
+        else if (sd.N == 4) ens_volume_pp<4>(a, sd, w, s_tb, dg_smem, s_fx);
+        else ens_volume_pp<5>(a, sd, w, s_tb, dg_smem, s_fx);
         continue;
       }
     }
-    if (sd.N == 3) ens_volume<R, 3>(a, sd, w, s_tb, dg_smem);
-    else if (sd.N == 4) ens_volume<R, 4>(a, sd, w, s_tb, dg_smem);
-    else ens_volume<R, 5>(a, sd, w, s_tb, dg_smem);
+    if (sd.N == 3) ens_volume<R, 3>(a, sd, w, s_tb, dg_smem, s_fx);
+    else if (sd.N == 4) ens_volume<R, 4>(a, sd, w, s_tb, dg_smem, s_fx);
+    else ens_volume<R, 5>(a, sd, w, s_tb, dg_smem, s_fx);
     __syncthreads();
   }
 }
@@ -317,7 +321,7 @@ struct dg_ensemble {
   long long nvalues, nnodes, nfs, nref;
   int block;  // threads per CTA (tunable)
   int per_sm; // requested resident CTAs per SM (tunable)
-  int pair;   // FP64: pair-parallel volume phase (tunable; 0: one thread per line)
+  int pair;   // FP64: volume phase one element at a time (tunable)
   int grid;   // persistent CTAs (cooperative launch)
   int nitems;
   SimDesc* d_sims;
@@ -347,17 +351,13 @@ int items_epb(int N, int block) {
 }
 
 // dynamic shared memory of a work item: FP64, node slots + accumulators;
-// FP32, the same in FP32 plus the staged RK register (volume32_smem);
-// pair-parallel, one element's slots, accumulators and pair fluxes of one
-// direction
+// FP32, the same in FP32 plus the staged RK register (volume32_smem); one
+// element's when the item's elements are taken in turn
 int smem_for(int precision, int block, int pair) {
-  if (pair)
-    return std::max(PairPar<3, 3, 1>::SMEM,
-                    std::max(PairPar<3, 4, 1>::SMEM, PairPar<3, 5, 1>::SMEM));
   int m = 0;
   for (int N = kEnsMinN; N <= kEnsMaxN; ++N) {
-    const int P = (N + 1) * (N + 1) * (N + 1), epb = items_epb(N, block);
-    const int b = precision == DG_FP64 ? epb * (9 + 5) * P * 8
+    const int P = (N + 1) * (N + 1) * (N + 1), epb = pair ? 1 : items_epb(N, block);
+    const int b = precision == DG_FP64 ? epb * (8 + 5) * P * 8
                                        : ((4 * epb * 14 * P + 15) & ~15) + 8 * epb * 5 * P;
     if (b > m) m = b;
   }
@@ -761,7 +761,7 @@ int dg_ensemble_get_block(const dg_ensemble* E, int* threads, int* ctas_per_sm, 
 }
 
 // Autotuner: times one stage for every candidate (threads per CTA, CTAs per
-// SM and, for FP64, one thread per line or pair-parallel) from u into u_tmp
+// SM and, for FP64, elements of an item at once or in turn) from u into u_tmp
 // (u is not changed) and keeps the fastest; the RK register is saved and
 // restored around the trials.
 int dg_ensemble_tune(dg_ensemble* E, const double* u, double* u_tmp, int* best_threads,

@@ -5,7 +5,12 @@
 //    the right element) of every interface and stores it in the face buffer
 //    fs[dir][v][e_left][l] (l = face-node index, see line_node).
 //
-//  volume_kernel: one CTA per EPB elements, one thread per element line.
+//  volume_fx_kernel (dg_fixed_volume.cuh): Ranocha's volume flux on FP64
+//    meshes, the pair fluxes in 64-bit fixed point with the threads of a line
+//    taking disjoint node pairs in turn.
+//
+//  volume_kernel (Chandrashekar's and the central flux): one CTA per EPB
+//    elements, one thread per element line.
 //    Prologue: conserved -> primitive at every node into shared memory.
 //    Per direction (a runtime loop; the flux is written with the direction's
 //    normal component first, so one code body serves every direction): each
@@ -18,15 +23,18 @@
 //    coalesced store of du, or the fused stage update k <- A k + dt du,
 //    u <- u + B k.
 //
-//  volume_pp_kernel (FP64 meshes under kPairParallelElems elements): one
-//    thread per node pair instead of per line; with FACES it also evaluates
-//    its elements' face fluxes, so that a whole rhs or stage is one launch.
+//  volume_fx_pp_kernel, volume_pp_kernel (FP64 meshes under
+//    kPairParallelElems elements; the first for Ranocha's flux from N = 2):
+//    one thread per node pair instead of per line; with FACES they also
+//    evaluate their elements' face fluxes, so that a whole rhs or stage is one
+//    launch.
 //
 // These templates are instantiated for FP64 meshes; FP32 meshes run the
 // perturbation-form kernels of dg_rhs32.cuh.
 #pragma once
 #include "dg_device.cuh"
 #include "dg_f32.cuh"
+#include "dg_fixed.cuh"
 
 namespace dg {
 
@@ -108,6 +116,22 @@ __device__ __forceinline__ void generic_nf(const LinePrim<R, D>& L, const LinePr
   volume_flux<VF, R, D, 0>(a, b, gm1inv, f);
 }
 
+// line l and position i of a node along direction dir (inverse of line_node)
+template <int D, int N>
+__device__ __forceinline__ void pp_line_of(int dir, int node, int& l, int& i) {
+  constexpr int NP = N + 1;
+  if (dir == 0) {
+    l = node / NP;
+    i = node % NP;
+  } else if (dir == 1) {
+    i = (node / NP) % NP;
+    l = (D == 2) ? node % NP : node % NP + NP * (node / (NP * NP));
+  } else {
+    i = node / (NP * NP);
+    l = node % (NP * NP);
+  }
+}
+
 template <int D, int N, typename R, int VF, int EPB>
 __device__ __forceinline__ void volume_direction(int dir, R (*sp)[3 + 2 * D][Shape<D, N>::P],
                                                  R (*sa)[D + 2][Shape<D, N>::P], int el, int l,
@@ -154,9 +178,8 @@ __device__ __forceinline__ void volume_direction(int dir, R (*sp)[3 + 2 * D][Sha
   for (int a = 0; a < NP; ++a) {
 #pragma unroll
     for (int b = a + 1; b < NP; ++b) {
-      R f[NV], an = R(0);
-      if (VF == kVRanocha) ranocha_nf<R, D>(q[a], q[b], f, an);
-      else generic_nf<VF, R, D>(q[a], q[b], gm1inv, f);
+      R f[NV];
+      generic_nf<VF, R, D>(q[a], q[b], gm1inv, f);
       const R dab = tb.Ds[dir][a][b], dba = tb.Ds[dir][b][a];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
@@ -254,9 +277,8 @@ __device__ __forceinline__ void volume_direction_rows(int dir, R (*sp)[3 + 2 * D
     for (int b = 1; b < NP; ++b) {
       if (b > a) {
         const LinePrim<R, D> qb = stage(b);
-        R f[NV], an = R(0);
-        if (VF == kVRanocha) ranocha_nf<R, D>(qa, qb, f, an);
-        else generic_nf<VF, R, D>(qa, qb, gm1inv, f);
+        R f[NV];
+        generic_nf<VF, R, D>(qa, qb, gm1inv, f);
         const R dab = tb.Ds[dir][a][b], dba = tb.Ds[dir][b][a];
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
@@ -620,15 +642,15 @@ __global__ void surface_kernel(const double* __restrict__ u, R* __restrict__ fs,
 // evaluated by both of its elements, with the face kernel's arithmetic, so the
 // result is the same as with the face kernel.
 //
-// G: directions per phase (0: all of them when one element's pair fluxes fit
-// in 96 KB, else one); EPB: elements per CTA.
-template <int D, int N, int G = 0, int EPB = 1>
+// EPB: elements per CTA. GROUP directions per phase: all of them when one
+// element's pair fluxes fit in 96 KB, else one.
+template <int D, int N, int EPB = 1>
 struct PairPar {
   static constexpr int NP = N + 1, P = Shape<D, N>::P, LINES = Shape<D, N>::LINES,
                        NV = D + 2, NC = 3 + 2 * D;
   static constexpr int NPAIRS = N * (N + 1) / 2;
   static constexpr bool ALLDIRS = D * LINES * NPAIRS * NV * 8 <= 98304;
-  static constexpr int GROUP = G > 0 ? G : (ALLDIRS ? D : 1);
+  static constexpr int GROUP = ALLDIRS ? D : 1;
   static constexpr int WORK = GROUP * LINES * NPAIRS;  // pair items per element and phase
   // volume threads: the pair items of the CTA's elements, at most 512
   static constexpr int THREADS = EPB * WORK < 512 ? ((EPB * WORK + 31) / 32) * 32 : 512;
@@ -674,37 +696,25 @@ __device__ __forceinline__ int pp_pair_index(int a, int b) {  // a < b
   return a * N - a * (a - 1) / 2 + (b - a - 1);
 }
 
-// line l and position i of a node along direction dir (inverse of line_node)
-template <int D, int N>
-__device__ __forceinline__ void pp_line_of(int dir, int node, int& l, int& i) {
-  constexpr int NP = N + 1;
-  if (dir == 0) {
-    l = node / NP;
-    i = node % NP;
-  } else if (dir == 1) {
-    i = (node / NP) % NP;
-    l = (D == 2) ? node % NP : node % NP + NP * (node / (NP * NP));
-  } else {
-    i = node / (NP * NP);
-    l = node % (NP * NP);
-  }
-}
+}  // namespace dg
+#include "dg_fixed_volume.cuh"
+namespace dg {
 
 // The body for the `count` (<= EPB) elements from e0 (every thread of the
 // block calls it; it ends with a barrier after its last shared-memory read,
 // so a block may run it for one batch after another). smem: C::SMEM bytes
 // (C::SMEM_F with FACES).
-template <int D, int N, int VF, bool FACES, int G, int EPB, bool CHAIN = false>
+template <int D, int N, int VF, bool FACES, int EPB>
 __device__ __forceinline__ void pp_elements(double* u, double* __restrict__ du,
                                             const double* __restrict__ fs, const Geom& g,
                                             const Tables<double>& tb, unsigned* __restrict__ err,
                                             const StageFuse& fz, int sfk, int e0, int count,
                                             unsigned char* dg_smem) {
-  using C = PairPar<D, N, G, EPB>;
+  using C = PairPar<D, N, EPB>;
   constexpr int NP = C::NP, P = C::P, NV = C::NV, NC = C::NC, LINES = C::LINES,
                 NPAIRS = C::NPAIRS, GROUP = C::GROUP, WORK = C::WORK;
   // per element el: slots sp[NC][P], accumulators sa[NV][P], direction
-  // parts sd[GROUP][NV][P] (unless CHAIN), pair fluxes sf[WORK][NV]; FACES: sfc[el] =
+  // parts sd[GROUP][NV][P], pair fluxes sf[WORK][NV]; FACES: sfc[el] =
   // [side][dir][c][l], side 0 the element's right face, 1 its left face, c in
   // normal-first order
   auto sp = [&](int el) {
@@ -818,45 +828,8 @@ __device__ __forceinline__ void pp_elements(double* u, double* __restrict__ du,
       for (int v = 0; v < NV; ++v) sfe[w * NV + v] = f[v];
     }
     __syncthreads();
-    if constexpr (CHAIN) {
-      // CHAIN: per (element, variable, node), the line sums of the group's
-      // directions in the line-owning kernel's order, each continuing the
-      // running total of the earlier directions, with the lifting at the line
-      // ends (face values in normal-first order)
-      for (int t = threadIdx.x; t < EPB * NV * P; t += blockDim.x) {
-        const int el = t / (NV * P), r = t % (NV * P);
-        if (el >= count) continue;
-        const int v = r / P, node = r % P;
-        const int e = e0 + el;
-        const double* sfe = sf(el);
-        const double* fce = sfc + (long long)el * 2 * D * LINES * NV;
-        double acc = d0 == 0 ? 0.0 : sa(el)[v][node];
-        for (int gd = 0; gd < GROUP; ++gd) {
-          const int dir = d0 + gd, c = nf_component<D>(v, dir);
-          int l, i;
-          pp_line_of<D, N>(dir, node, l, i);
-          for (int j = 0; j < NP; ++j) {
-            if (j == i) continue;
-            const int p = j < i ? pp_pair_index<N>(j, i) : pp_pair_index<N>(i, j);
-            acc = fma(tb.Ds[dir][i][j], sfe[((gd * LINES + l) * NPAIRS + p) * NV + c], acc);
-          }
-          if (i == N)
-            acc = fma(tb.liftR[dir],
-                      FACES ? fce[((0 * D + dir) * NV + c) * LINES + l]
-                            : fs[(long long)(dir * NV + v) * base + (long long)e * LINES + l],
-                      acc);
-          if (i == 0)
-            acc = fma(tb.liftL[dir],
-                      FACES ? fce[((1 * D + dir) * NV + c) * LINES + l]
-                            : fs[(long long)(dir * NV + v) * base +
-                                 (long long)s_left[el][dir] * LINES + l],
-                      acc);
-        }
-        sa(el)[v][node] = acc;
-      }
-      __syncthreads();
-    } else {
-      // otherwise per (element, direction, node): the line sum on its own
+    {
+      // per (element, direction, node): the line sum on its own
       // (in the same order of pairs), then the lifting (normal-first
       // components back to variables); a direction whose terms cancel exactly
       // keeps its exact zero
@@ -924,9 +897,7 @@ __device__ __forceinline__ void pp_elements(double* u, double* __restrict__ du,
     }
   }
   // epilogue: the CTA's elements are contiguous in the state
-  // (CHAIN: tb holds the coefficients times dt, as volume_batch's does, so
-  // the sums are already dt du)
-  const double dtv = fz.k ? (CHAIN ? 1.0 : *fz.dt) : 0.0;
+  const double dtv = fz.k ? *fz.dt : 0.0;
   double* const uo = fz.u_out ? fz.u_out : u;
   for (int t = threadIdx.x; t < count * NV * P; t += blockDim.x) {
     const int el = t / (NV * P), r = t % (NV * P);
@@ -934,7 +905,7 @@ __device__ __forceinline__ void pp_elements(double* u, double* __restrict__ du,
     const double val = sa(el)[v][node];
     const long long i = (long long)e0 * NV * P + t;
     if (fz.k) {
-      double kk = CHAIN ? val : dtv * val;
+      double kk = dtv * val;
       if (fz.a != 0.0) kk = fma(fz.a, fz.k[i], kk);
       fz.k[i] = kk;
       uo[i] = u[i] + fz.b * kk;
@@ -946,14 +917,14 @@ __device__ __forceinline__ void pp_elements(double* u, double* __restrict__ du,
 }
 
 template <int D, int N, int VF, bool FACES, int EPB>
-__global__ void __launch_bounds__(FACES ? PairPar<D, N, 0, EPB>::THREADS_F
-                                        : PairPar<D, N, 0, EPB>::THREADS)
+__global__ void __launch_bounds__(FACES ? PairPar<D, N, EPB>::THREADS_F
+                                        : PairPar<D, N, EPB>::THREADS)
     volume_pp_kernel(double* u, double* __restrict__ du, const double* __restrict__ fs, Geom g,
                      Tables<double> tb, unsigned* __restrict__ err, StageFuse fz, int sfk) {
   extern __shared__ __align__(16) unsigned char dg_smem[];
   const int e0 = blockIdx.x * EPB;
   const int left = (int)g.nelem - e0;
-  pp_elements<D, N, VF, FACES, 0, EPB>(u, du, fs, g, tb, err, fz, sfk, e0,
+  pp_elements<D, N, VF, FACES, EPB>(u, du, fs, g, tb, err, fz, sfk, e0,
                                        left < EPB ? left : EPB, dg_smem);
 }
 
@@ -999,11 +970,7 @@ cudaError_t launch_volume_epb(const double* u, R* du, R* fs, const Geom& g, cons
   const int threads = EPB * L::LINES;
   constexpr int SM = EPB * L::PER_ELEM;
   cudaError_t e;
-  if (vf == kVRanocha) {
-    if ((e = allow_smem(volume_kernel<D, N, R, kVRanocha, EPB>, SM)) != cudaSuccess) return e;
-    volume_kernel<D, N, R, kVRanocha, EPB><<<(unsigned)grid, threads, SM, st>>>(
-        const_cast<double*>(u), du, fs, g, tb, err, fz);
-  } else if (vf == kVChandrashekar) {
+  if (vf == kVChandrashekar) {
     if ((e = allow_smem(volume_kernel<D, N, R, kVChandrashekar, EPB>, SM)) != cudaSuccess) return e;
     volume_kernel<D, N, R, kVChandrashekar, EPB><<<(unsigned)grid, threads, SM, st>>>(
         const_cast<double*>(u), du, fs, g, tb, err, fz);
@@ -1015,13 +982,44 @@ cudaError_t launch_volume_epb(const double* u, R* du, R* fs, const Geom& g, cons
   return cudaGetLastError();
 }
 
+template <int D, int N, int EPB>
+cudaError_t launch_volume_fx(const double* u, double* du, const double* fs, const Geom& g,
+                             const Tables<double>& tb, unsigned* err, cudaStream_t st,
+                             const StageFuse& fz) {
+  using L = FxLaunch<D, N>;
+  const long long grid = (g.nelem + EPB - 1) / EPB;
+  cudaError_t e;
+  if ((e = allow_smem(volume_fx_kernel<D, N, EPB>, EPB * L::ELEM)) != cudaSuccess ||
+      (e = prefer_shared(volume_fx_kernel<D, N, EPB>)) != cudaSuccess)
+    return e;
+  volume_fx_kernel<D, N, EPB><<<(unsigned)grid, L::threads(EPB), EPB * L::ELEM, st>>>(
+      const_cast<double*>(u), du, fs, g, tb, err, fz);
+  return cudaGetLastError();
+}
+
 // meshes of fewer elements than this run the pair-parallel FP64 volume kernel
+template <int D, int N, bool FACES>
+cudaError_t launch_volume_fx_pp(const double* u, double* du, double* fs, const Geom& g,
+                                const Tables<double>& tb, int sf, unsigned* err, cudaStream_t st,
+                                const StageFuse& fz) {
+  constexpr int EPB = FACES ? pp_epb<D, N>() : 1;
+  using C = FxPairPar<D, N, EPB>;
+  constexpr int threads = FACES ? C::THREADS_F : C::THREADS;
+  constexpr int smem = FACES ? C::SMEM_F : C::SMEM;
+  cudaError_t e;
+  if ((e = allow_smem(volume_fx_pp_kernel<D, N, FACES, EPB>, smem)) != cudaSuccess) return e;
+  const unsigned grid = (unsigned)((g.nelem + EPB - 1) / EPB);
+  volume_fx_pp_kernel<D, N, FACES, EPB><<<grid, threads, smem, st>>>(
+      const_cast<double*>(u), du, fs, g, tb, err, fz, sf);
+  return cudaGetLastError();
+}
+
 template <int D, int N, int VF, bool FACES>
 cudaError_t launch_volume_pp_vf(const double* u, double* du, double* fs, const Geom& g,
                                 const Tables<double>& tb, int sf, unsigned* err, cudaStream_t st,
                                 const StageFuse& fz) {
   constexpr int EPB = FACES ? pp_epb<D, N>() : 1;
-  using C = PairPar<D, N, 0, EPB>;
+  using C = PairPar<D, N, EPB>;
   constexpr int threads = FACES ? C::THREADS_F : C::THREADS;
   constexpr int smem = FACES ? C::SMEM_F : C::SMEM;
   cudaError_t e;
@@ -1039,14 +1037,24 @@ cudaError_t launch_volume_pp(const double* u, double* du, double* fs, const Geom
                              const Tables<double>& tb, int vf, int sf, unsigned* err,
                              cudaStream_t st, const StageFuse& fz, bool faces) {
   if (faces) {
-    if (vf == kVRanocha)
-      return launch_volume_pp_vf<D, N, kVRanocha, true>(u, du, fs, g, tb, sf, err, st, fz);
+    // N = 1 has one pair per line, too few to pay for the fixed-point form's
+    // extra phases (2D 16^2: 8.7 us per rhs in FP64, 9.4 in fixed point)
+    if (vf == kVRanocha) {
+      if constexpr (N == 1)
+        return launch_volume_pp_vf<D, N, kVRanocha, true>(u, du, fs, g, tb, sf, err, st, fz);
+      else
+        return launch_volume_fx_pp<D, N, true>(u, du, fs, g, tb, sf, err, st, fz);
+    }
     if (vf == kVChandrashekar)
       return launch_volume_pp_vf<D, N, kVChandrashekar, true>(u, du, fs, g, tb, sf, err, st, fz);
     return launch_volume_pp_vf<D, N, kVCentral, true>(u, du, fs, g, tb, sf, err, st, fz);
   }
-  if (vf == kVRanocha)
-    return launch_volume_pp_vf<D, N, kVRanocha, false>(u, du, fs, g, tb, sf, err, st, fz);
+  if (vf == kVRanocha) {
+    if constexpr (N == 1)
+      return launch_volume_pp_vf<D, N, kVRanocha, false>(u, du, fs, g, tb, sf, err, st, fz);
+    else
+      return launch_volume_fx_pp<D, N, false>(u, du, fs, g, tb, sf, err, st, fz);
+  }
   if (vf == kVChandrashekar)
     return launch_volume_pp_vf<D, N, kVChandrashekar, false>(u, du, fs, g, tb, sf, err, st, fz);
   return launch_volume_pp_vf<D, N, kVCentral, false>(u, du, fs, g, tb, sf, err, st, fz);
@@ -1144,6 +1152,12 @@ cudaError_t launch_rhs_dn(const double* u, R* du, R* fs, const Geom& g, const Ta
     constexpr int EPB = L::EPB;
     if (g.nelem < kPairParallelElems)
       return launch_volume_pp<D, N>(u, du, fs, g, tb, vf, sf, err, st, fz, false);
+    if (vf == kVRanocha) {
+      constexpr int FEPB = FxLaunch<D, N>::EPB;
+      if (FEPB > 1 && g.nelem < 2LL * 152 * FEPB)
+        return launch_volume_fx<D, N, 1>(u, du, fs, g, tb, err, st, fz);
+      return launch_volume_fx<D, N, FEPB>(u, du, fs, g, tb, err, st, fz);
+    }
     if (EPB > 1 && g.nelem < 2LL * 152 * EPB)
       return launch_volume_epb<D, N, R, 1>(u, du, fs, g, tb, vf, err, st, fz);
     return launch_volume_epb<D, N, R, EPB>(u, du, fs, g, tb, vf, err, st, fz);

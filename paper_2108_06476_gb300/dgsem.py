@@ -540,8 +540,9 @@ class Ensemble:
 
     @property
     def pair_parallel(self):
-        """Threads per line of the volume phase: False, one thread per line;
-        True (FP64 only), one thread per node pair (the same result)."""
+        """The volume phase takes the elements of a work item at once (False)
+        or one after another with the whole CTA (True, FP64 only); the same
+        result."""
         on = ctypes.c_int()
         _check(load().dg_ensemble_get_pair_parallel(self._h, ctypes.byref(on)),
                "dg_ensemble_get_pair_parallel")
@@ -553,9 +554,8 @@ class Ensemble:
                "dg_ensemble_set_pair_parallel")
 
     def tune(self, u, u_tmp):
-        """Autotune the CTA shape and (FP64) the threads per line; returns
-        (threads, ctas_per_sm, ms_per_stage); the chosen threads per line:
-        pair_parallel."""
+        """Autotune the CTA shape and (FP64) pair_parallel; returns (threads,
+        ctas_per_sm, ms_per_stage)."""
         self._chk(u)
         self._chk(u_tmp)
         t, b, ms = ctypes.c_int(), ctypes.c_int(), ctypes.c_float()

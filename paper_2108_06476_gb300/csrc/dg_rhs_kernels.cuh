@@ -698,6 +698,7 @@ __device__ __forceinline__ int pp_pair_index(int a, int b) {  // a < b
 
 }  // namespace dg
 #include "dg_fixed_volume.cuh"
+#include "dg_weak.cuh"
 namespace dg {
 
 // The body for the `count` (<= EPB) elements from e0 (every thread of the
@@ -964,21 +965,15 @@ cudaError_t prefer_shared(K kernel) {
 // parts: bit 0 = surface kernel, bit 1 = volume kernel (both for an rhs)
 template <int D, int N, typename R, int EPB>
 cudaError_t launch_volume_epb(const double* u, R* du, R* fs, const Geom& g, const Tables<R>& tb,
-                              int vf, unsigned* err, cudaStream_t st, const StageFuse& fz) {
+                              unsigned* err, cudaStream_t st, const StageFuse& fz) {
   using L = Launch<D, N, R>;
   const long long grid = (g.nelem + EPB - 1) / EPB;
   const int threads = EPB * L::LINES;
   constexpr int SM = EPB * L::PER_ELEM;
   cudaError_t e;
-  if (vf == kVChandrashekar) {
-    if ((e = allow_smem(volume_kernel<D, N, R, kVChandrashekar, EPB>, SM)) != cudaSuccess) return e;
-    volume_kernel<D, N, R, kVChandrashekar, EPB><<<(unsigned)grid, threads, SM, st>>>(
-        const_cast<double*>(u), du, fs, g, tb, err, fz);
-  } else {
-    if ((e = allow_smem(volume_kernel<D, N, R, kVCentral, EPB>, SM)) != cudaSuccess) return e;
-    volume_kernel<D, N, R, kVCentral, EPB><<<(unsigned)grid, threads, SM, st>>>(
-        const_cast<double*>(u), du, fs, g, tb, err, fz);
-  }
+  if ((e = allow_smem(volume_kernel<D, N, R, kVChandrashekar, EPB>, SM)) != cudaSuccess) return e;
+  volume_kernel<D, N, R, kVChandrashekar, EPB><<<(unsigned)grid, threads, SM, st>>>(
+      const_cast<double*>(u), du, fs, g, tb, err, fz);
   return cudaGetLastError();
 }
 
@@ -998,6 +993,19 @@ cudaError_t launch_volume_fx(const double* u, double* du, const double* fs, cons
 }
 
 // meshes of fewer elements than this run the pair-parallel FP64 volume kernel
+template <int D, int N, int EPB>
+cudaError_t launch_volume_weak(const double* u, double* du, const double* fs, const Geom& g,
+                               const Tables<double>& tb, unsigned* err, cudaStream_t st,
+                               const StageFuse& fz) {
+  constexpr int P = Shape<D, N>::P, threads = 32 * ((EPB * P + 31) / 32),
+                smem = EPB * (D + 2) * P * 8;
+  cudaError_t e;
+  if ((e = allow_smem(volume_weak_kernel<D, N, EPB>, smem)) != cudaSuccess) return e;
+  volume_weak_kernel<D, N, EPB><<<(unsigned)((g.nelem + EPB - 1) / EPB), threads, smem, st>>>(
+      const_cast<double*>(u), du, fs, g, tb, err, fz);
+  return cudaGetLastError();
+}
+
 template <int D, int N, bool FACES>
 cudaError_t launch_volume_fx_pp(const double* u, double* du, double* fs, const Geom& g,
                                 const Tables<double>& tb, int sf, unsigned* err, cudaStream_t st,
@@ -1158,9 +1166,15 @@ cudaError_t launch_rhs_dn(const double* u, R* du, R* fs, const Geom& g, const Ta
         return launch_volume_fx<D, N, 1>(u, du, fs, g, tb, err, st, fz);
       return launch_volume_fx<D, N, FEPB>(u, du, fs, g, tb, err, st, fz);
     }
+    if (vf == kVCentral) {
+      constexpr int WEPB = WeakLaunch<D, N>::EPB;
+      if (WEPB > 1 && g.nelem < 2LL * 152 * WEPB)
+        return launch_volume_weak<D, N, 1>(u, du, fs, g, tb, err, st, fz);
+      return launch_volume_weak<D, N, WEPB>(u, du, fs, g, tb, err, st, fz);
+    }
     if (EPB > 1 && g.nelem < 2LL * 152 * EPB)
-      return launch_volume_epb<D, N, R, 1>(u, du, fs, g, tb, vf, err, st, fz);
-    return launch_volume_epb<D, N, R, EPB>(u, du, fs, g, tb, vf, err, st, fz);
+      return launch_volume_epb<D, N, R, 1>(u, du, fs, g, tb, err, st, fz);
+    return launch_volume_epb<D, N, R, EPB>(u, du, fs, g, tb, err, st, fz);
   }
 }
 

@@ -236,3 +236,42 @@ def test_a_state_at_rest_keeps_its_density_and_energy(d, N, n):
     du = Mesh(d, N, n, surface_flux="ranocha").rhs(torch.from_numpy(u).cuda())
     du = du.cpu().numpy().reshape(ne, d + 2, P)
     assert not du[:, 0].any() and not du[:, d + 1].any()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,N,n", [(2, 1, (27, 25)), (2, 3, (26, 25)), (2, 6, (25, 27)),
+                                   (3, 1, (9, 9, 9)), (3, 2, (40, 13, 17)), (3, 3, (10, 9, 7)),
+                                   (3, 4, (9, 10, 7)), (3, 5, (9, 9, 8)), (3, 6, (9, 9, 8)),
+                                   (3, 7, (8, 9, 9))])
+@pytest.mark.parametrize("kind", ["random", "fast", "still", "units", "huge"])
+def test_weak_form_against_the_oracle(d, N, n, kind):
+    # the nodal-flux form of the central volume flux, in fixed point and (an
+    # element with a value beyond its exponents) in FP64
+    torch = _gpu()
+    import oracle
+    from paper_2108_06476_gb300 import Mesh, workloads as W
+    oracle.build()
+    rng = np.random.default_rng([d, N, 6])
+    ne, P = int(np.prod(n)), (N + 1) ** d
+    rho = np.exp(rng.uniform(-1, 1, (ne, P)))
+    p = 2.0 * np.exp(rng.uniform(-1, 1, (ne, P)))
+    v = [rng.uniform(-0.5, 0.5, (ne, P)) for _ in range(d)]
+    if kind == "fast":
+        v = [30.0 + 2.0 * x for x in v]
+    if kind == "still":
+        v = [0.0 * x for x in v]
+    if kind == "units":
+        rho, p, v = rho * 1e-20, p * 1e-8, [x * 1e6 for x in v]
+    if kind == "huge":  # every other element beyond the accepted exponents
+        rho[::2] *= 1e50
+        p[::2] *= 1e50
+    u = np.ascontiguousarray(W.prim_to_cons(rho, v, p).reshape(-1))
+    dom = W.box(d)
+    m = Mesh(d, N, n, volume_flux="central", surface_flux="hll")
+    got = m.rhs(torch.from_numpy(u).cuda()).cpu().numpy().reshape(ne, d + 2, P)
+    assert m.check() == 0
+    elems = np.unique(np.linspace(0, ne - 1, 40).astype(np.int64))
+    ref = oracle.rhs(d, N, n, dom, u, vflux=2, sflux=2, elems=elems).reshape(ne, d + 2, P)
+    for e in elems:
+        err = np.linalg.norm(got[e] - ref[e]) / np.linalg.norm(ref[e])
+        assert err <= 1e-12, (kind, int(e), err)

@@ -158,10 +158,25 @@ DG_FX_FN Scale element_scale(const unsigned* key, const int* c) {
          (int)((emax - emin) >> 20) + s.ee - ee <= 8 && s.s < 16 && s.kv < 63 && s.km < 63;
   return s;
 }
-// c with p (f/(gamma-1) + 1) < 2^c p, f = 1.1 and 2.2
+// c with p (f/(gamma-1) + 1) < 2^c p, f = 1.1 and 2.2, in FP32 (an FP64
+// division in every warp would cost as much as a node's primitives; f has 2%
+// to spare)
 DG_FX_FN void scale_bits(double gm1, int* c) {
-  c[0] = ilogb(1.1 / gm1 + 1.0) + 1;
-  c[1] = ilogb(2.2 / gm1 + 1.0) + 1;
+#ifdef DG_FX_HOST
+  const float g = (float)gm1;
+#else
+  const float g = d2f(gm1);
+#endif
+  const float x[2] = {1.1f / g + 1.0f, 2.2f / g + 1.0f};
+  for (int i = 0; i < 2; ++i) {
+#ifdef DG_FX_HOST
+    unsigned b;
+    __builtin_memcpy(&b, &x[i], 4);
+#else
+    const unsigned b = __float_as_uint(x[i]);
+#endif
+    c[i] = (int)(b >> 23) - 127 + 1;
+  }
 }
 
 // x/2 in format 63 - E (|x| < 2^E): the 53-bit significand aligned to bit 62,

@@ -11,8 +11,8 @@
 // thread per line (168 registers, 12 warps per SM) the integer pipes stood at
 // 37% waiting for dependent results; this layout runs 24 warps per SM. Measured
 // at 64^3 N = 3, a fused stage's volume kernel: FP64 8.47 ms, fixed point with
-// one thread per line 3.87, this layout 2.76; rhs at 24^3 N = 7: 8.14 ms to
-// 2.26. The threads of a line share a warp
+// one thread per line 3.87, this layout 2.49; rhs at 24^3 N = 7: 8.14 ms to
+// 2.0. The threads of a line share a warp
 // (32/T lines per warp), so rounds are separated by a warp barrier. At N = 3
 // in 3D a warp owns a whole element (16 lines x 2) and no block barrier runs
 // at all.
@@ -175,59 +175,117 @@ __device__ __forceinline__ int fx_table_exponent(const Tables<double>& tb) {
   return fx::exp_above(m);
 }
 
-// primitives of the group's nodes (rho, e, p, v in FP64 slots) and the keys
-// of their elements' scales. gi/gs: thread index and size of the group (whole
-// warps)
+// primitives of a node and the keys of its element's scale
+template <int D>
+struct FxPrim {
+  double rho, e, p, v[D];
+};
+template <int D>
+__device__ __forceinline__ FxPrim<D> fx_prim(const double* c, const Geom& g, unsigned& bad) {
+  double rr;
+  const Prim<double, D> q = prim_rcp<D>(c, g.gm1, rr);
+  bad |= prim_check(q);
+  FxPrim<D> r;
+  r.rho = q.rho;
+  r.p = q.p;
+  r.e = q.p * rr * g.gm1inv;
+#pragma unroll
+  for (int k = 0; k < D; ++k) r.v[k] = q.v[k];
+  return r;
+}
+
+struct FxKeys {
+  unsigned r, e, v, p;
+};
+template <int D>
+__device__ __forceinline__ FxKeys fx_keys(const FxPrim<D>& q) {
+  FxKeys k;
+  k.r = (unsigned)__double2hiint(q.rho);
+  k.e = (unsigned)__double2hiint(q.e);
+  k.p = (unsigned)__double2hiint(q.p);
+  k.v = 0;
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    const unsigned h = (unsigned)__double2hiint(q.v[j]) & 0x7fffffffu;
+    k.v = h > k.v ? h : k.v;
+  }
+  return k;
+}
+// the keys of one element over the warp's lanes `mine`, by lane 0 into key
+__device__ __forceinline__ void fx_merge_keys(const FxKeys& k, bool mine, unsigned* key) {
+  const unsigned a = __reduce_max_sync(0xffffffffu, mine ? k.r : 0u);
+  const unsigned b = __reduce_min_sync(0xffffffffu, mine ? k.r : 0xffffffffu);
+  const unsigned c = __reduce_max_sync(0xffffffffu, mine ? k.e : 0u);
+  const unsigned d = __reduce_min_sync(0xffffffffu, mine ? k.e : 0xffffffffu);
+  const unsigned v = __reduce_max_sync(0xffffffffu, mine ? k.v : 0u);
+  const unsigned p = __reduce_max_sync(0xffffffffu, mine ? k.p : 0u);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&key[0], a);
+    atomicMin(&key[1], b);
+    atomicMax(&key[2], c);
+    atomicMin(&key[3], d);
+    atomicMax(&key[4], v);
+    atomicMax(&key[5], p);
+  }
+}
+
+// the staged slots of a node in its element's form, and its cleared sums
+template <int D, int N>
+__device__ __forceinline__ void fx_stage_node(const FxPrim<D>& q, const fx::Scale& sc, double gm1,
+                                              unsigned char* elem, int pl) {
+  constexpr int P = Shape<D, N>::P, NV = D + 2, SL = FxShape<D, N>::SLOTS;
+  double* sp = reinterpret_cast<double*>(elem);
+  fx::i64* sx = reinterpret_cast<fx::i64*>(elem);
+  if (sc.ok) {
+    sx[pl] = fx::half_fixed(q.rho, sc.er);
+    sx[P + pl] = fx::ln_fixed(q.rho, sc.er);
+    sx[2 * P + pl] = fx::half_fixed(q.e, sc.ee);
+    sx[3 * P + pl] = fx::ln_fixed(q.e, sc.ee);
+    sx[4 * P + pl] = fx::half_fixed(q.p, sc.em);
+#pragma unroll
+    for (int k = 0; k < D; ++k) sx[(5 + k) * P + pl] = fx::half_fixed(q.v[k], sc.ev);
+  } else {
+    node_slots<kVRanocha, double>(q.rho, q.p, gm1, sp[pl], sp[P + pl]);
+    sp[2 * P + pl] = half(q.p);
+#pragma unroll
+    for (int k = 0; k < D; ++k) sp[(3 + k) * P + pl] = q.v[k];
+  }
+  // the sums start at +0.0, or at the D N units by which the truncated
+  // products fall short on average; where nothing moves, mass and energy
+  // fluxes are zeros and so are their sums
+#pragma unroll
+  for (int v = 0; v < NV; ++v)
+    sx[(SL + v) * P + pl] = sc.ok && (sc.moves || (v > 0 && v <= D)) ? D * N : 0;
+}
+
+// primitives of the batch's nodes (rho, e, p, v in FP64 slots) and the keys of
+// their elements' scales, by the whole block
 template <int D, int N>
 __device__ __forceinline__ unsigned fx_load(const double* __restrict__ u, const Geom& g, int e0,
-                                            int count, unsigned char* smem, int stride,
-                                            unsigned (*key)[6], int gi, int gs) {
-  constexpr int P = Shape<D, N>::P, NV = D + 2;
+                                            int count, unsigned char* smem,
+                                            unsigned (*key)[6]) {
+  constexpr int P = Shape<D, N>::P, NV = D + 2, ELEM = FxShape<D, N>::ELEM;
   unsigned bad = 0;
-  for (int t0 = gi & ~31; t0 < count * P; t0 += gs) {
-    const int t = t0 + (gi & 31);
+  for (int t0 = threadIdx.x & ~31; t0 < count * P; t0 += blockDim.x) {
+    const int t = t0 + (threadIdx.x & 31);
     const bool in = t < count * P;
     const int el = t / P, node = t % P, pl = fx_place<D, N>(node);
-    unsigned kr = 0, ke = 0, kv = 0, kp = 0;
+    FxKeys k = {};
     if (in) {
-      double c[NV], rr;
+      double c[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) c[v] = u[((long long)(e0 + el) * NV + v) * P + node];
-      const Prim<double, D> q = prim_rcp<D>(c, g.gm1, rr);
-      bad |= prim_check(q);
-      const double ei = q.p * rr * g.gm1inv;
-      double* sp = reinterpret_cast<double*>(smem + el * stride);
+      const FxPrim<D> q = fx_prim<D>(c, g, bad);
+      k = fx_keys<D>(q);
+      double* sp = reinterpret_cast<double*>(smem + el * ELEM);
       sp[pl] = q.rho;
-      sp[P + pl] = ei;
+      sp[P + pl] = q.e;
       sp[2 * P + pl] = q.p;
-      kr = (unsigned)__double2hiint(q.rho);
-      ke = (unsigned)__double2hiint(ei);
-      kp = (unsigned)__double2hiint(q.p);
 #pragma unroll
-      for (int k = 0; k < D; ++k) {
-        sp[(3 + k) * P + pl] = q.v[k];
-        const unsigned h = (unsigned)__double2hiint(q.v[k]) & 0x7fffffffu;
-        kv = h > kv ? h : kv;
-      }
+      for (int j = 0; j < D; ++j) sp[(3 + j) * P + pl] = q.v[j];
     }
     const int last = (t0 + 31 < count * P ? t0 + 31 : count * P - 1) / P;
-    for (int ek = t0 / P; ek <= last; ++ek) {
-      const bool mine = in && el == ek;
-      const unsigned a = __reduce_max_sync(0xffffffffu, mine ? kr : 0u);
-      const unsigned b = __reduce_min_sync(0xffffffffu, mine ? kr : 0xffffffffu);
-      const unsigned c = __reduce_max_sync(0xffffffffu, mine ? ke : 0u);
-      const unsigned d = __reduce_min_sync(0xffffffffu, mine ? ke : 0xffffffffu);
-      const unsigned v = __reduce_max_sync(0xffffffffu, mine ? kv : 0u);
-      const unsigned p = __reduce_max_sync(0xffffffffu, mine ? kp : 0u);
-      if ((gi & 31) == 0) {
-        atomicMax(&key[ek][0], a);
-        atomicMin(&key[ek][1], b);
-        atomicMax(&key[ek][2], c);
-        atomicMin(&key[ek][3], d);
-        atomicMax(&key[ek][4], v);
-        atomicMax(&key[ek][5], p);
-      }
-    }
+    for (int ek = t0 / P; ek <= last; ++ek) fx_merge_keys(k, in && el == ek, key[ek]);
   }
   return bad;
 }
@@ -237,46 +295,27 @@ __device__ __forceinline__ void fx_clear_key(unsigned* key) {
   key[1] = key[3] = 0xffffffffu;
 }
 
-__device__ __forceinline__ fx::Scale fx_scale(const unsigned* key, double gm1, int ed) {
-  int c[2];
-  fx::scale_bits(gm1, c);
+__device__ __forceinline__ fx::Scale fx_scale(const unsigned* key, const int* c, int ed) {
   fx::Scale sc = fx::element_scale(key, c);
   if (ed > 300 || ed < -300) sc.ok = 0;
   return sc;
 }
 
-// the slots of each element's form, in place, and cleared sums
+// the slots of each element's form, in place, by the whole block
 template <int D, int N>
-__device__ __forceinline__ void fx_stage(const Geom& g, int count, unsigned char* smem, int stride,
-                                         const fx::Scale* scale, int gi, int gs) {
-  constexpr int P = Shape<D, N>::P, NV = D + 2, SL = FxShape<D, N>::SLOTS;
-  for (int t = gi; t < count * P; t += gs) {
+__device__ __forceinline__ void fx_stage(const Geom& g, int count, unsigned char* smem,
+                                         const fx::Scale* scale) {
+  constexpr int P = Shape<D, N>::P, ELEM = FxShape<D, N>::ELEM;
+  for (int t = threadIdx.x; t < count * P; t += blockDim.x) {
     const int el = t / P, pl = t % P;
-    const fx::Scale sc = scale[el];
-    double* sp = reinterpret_cast<double*>(smem + el * stride);
-    fx::i64* sx = reinterpret_cast<fx::i64*>(sp);
-    const double rho = sp[pl], ei = sp[P + pl], p = sp[2 * P + pl];
-    double v[D];
+    const double* sp = reinterpret_cast<const double*>(smem + el * ELEM);
+    FxPrim<D> q;
+    q.rho = sp[pl];
+    q.e = sp[P + pl];
+    q.p = sp[2 * P + pl];
 #pragma unroll
-    for (int k = 0; k < D; ++k) v[k] = sp[(3 + k) * P + pl];
-    if (sc.ok) {
-      sx[pl] = fx::half_fixed(rho, sc.er);
-      sx[P + pl] = fx::ln_fixed(rho, sc.er);
-      sx[2 * P + pl] = fx::half_fixed(ei, sc.ee);
-      sx[3 * P + pl] = fx::ln_fixed(ei, sc.ee);
-      sx[4 * P + pl] = fx::half_fixed(p, sc.em);
-#pragma unroll
-      for (int k = 0; k < D; ++k) sx[(5 + k) * P + pl] = fx::half_fixed(v[k], sc.ev);
-    } else {
-      node_slots<kVRanocha, double>(rho, p, g.gm1, sp[pl], sp[P + pl]);
-      sp[2 * P + pl] = half(p);
-    }
-    // the sums start at +0.0, or at the D N units by which the truncated
-    // products fall short on average; where nothing moves, mass and energy
-    // fluxes are zeros and so are their sums
-#pragma unroll
-    for (int q = 0; q < NV; ++q)
-      sx[(SL + q) * P + pl] = sc.ok && (sc.moves || (q > 0 && q <= D)) ? D * N : 0;
+    for (int k = 0; k < D; ++k) q.v[k] = sp[(3 + k) * P + pl];
+    fx_stage_node<D, N>(q, scale[el], g.gm1, smem + el * ELEM, pl);
   }
 }
 
@@ -351,6 +390,8 @@ __device__ __forceinline__ void fx_batch(double* u, double* __restrict__ du,
   }
   __syncthreads();  // tb is in place
   const int ed = fx_table_exponent<D>(tb);
+  int cb[2];
+  fx::scale_bits(g.gm1, cb);
   for (int i = threadIdx.x; i < D * NP * NP; i += blockDim.x) {
     const int dir = i / (NP * NP), a = (i / NP) % NP, b = i % NP;
     sh.Ds[dir][a][b] = fx::limbs(fx::half_fixed(tb.Ds[dir][a][b], ed));
@@ -361,11 +402,24 @@ __device__ __forceinline__ void fx_batch(double* u, double* __restrict__ du,
     for (int el = threadIdx.x >> 5; el < count; el += blockDim.x >> 5) {
       unsigned char* elem = smem + el * ELEM;
       const int e = e0 + el;
-      const unsigned bad = fx_load<D, N>(u, g, e, 1, elem, ELEM, sh.key + el, lane, 32);
+      constexpr int NPL = P / 32;  // nodes per lane
+      FxPrim<D> q[NPL];
+      unsigned bad = 0;
+#pragma unroll
+      for (int j = 0; j < NPL; ++j) {
+        double c[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) c[v] = u[((long long)e * NV + v) * P + lane + 32 * j];
+        q[j] = fx_prim<D>(c, g, bad);
+      }
       if (bad) atomicOr(err, bad);
+#pragma unroll
+      for (int j = 0; j < NPL; ++j) fx_merge_keys(fx_keys<D>(q[j]), true, sh.key[el]);
       __syncwarp();
-      const fx::Scale sc = fx_scale(sh.key[el], g.gm1, ed);
-      fx_stage<D, N>(g, 1, elem, ELEM, &sc, lane, 32);
+      const fx::Scale sc = fx_scale(sh.key[el], cb, ed);
+#pragma unroll
+      for (int j = 0; j < NPL; ++j)
+        fx_stage_node<D, N>(q[j], sc, g.gm1, elem, fx_place<D, N>(lane + 32 * j));
       __syncwarp();
       const int l = lane % T::LPW, t = lane / T::LPW;
 #pragma unroll 1
@@ -388,13 +442,13 @@ __device__ __forceinline__ void fx_batch(double* u, double* __restrict__ du,
       }
     }
   } else {
-    const unsigned bad = fx_load<D, N>(u, g, e0, count, smem, ELEM, sh.key, threadIdx.x, blockDim.x);
+    const unsigned bad = fx_load<D, N>(u, g, e0, count, smem, sh.key);
     if (bad) atomicOr(err, bad);
     __syncthreads();
     if ((int)threadIdx.x < count)
-      sh.scale[threadIdx.x] = fx_scale(sh.key[threadIdx.x], g.gm1, ed);
+      sh.scale[threadIdx.x] = fx_scale(sh.key[threadIdx.x], cb, ed);
     __syncthreads();
-    fx_stage<D, N>(g, count, smem, ELEM, sh.scale, threadIdx.x, blockDim.x);
+    fx_stage<D, N>(g, count, smem, sh.scale);
     __syncthreads();
     const int lane = threadIdx.x & 31, t = lane / T::LPW;
 #pragma unroll 1
@@ -476,6 +530,11 @@ struct FxPairPar {
   static constexpr int THREADS_F = THREADS + ((FITEMS + 31) / 32) * 32;
   static_assert(THREADS_F <= 1024, "face warps do not fit the CTA");
   static constexpr int SMEM_F = SMEM + EPB * 2 * D * NV * LINES * 8;
+  static_assert(EPB * P <= THREADS, "a node per volume thread");
+  // 32 warps per SM whatever the CTA's size: a mesh of a few hundred elements
+  // then needs one wave of CTAs fewer than with the compiler's own choice of
+  // up to 98 registers (8^3 N = 3: 35 us per rhs against 27)
+  static constexpr int MIN_CTAS = 1024 / THREADS_F < 1 ? 1 : 1024 / THREADS_F;
 };
 
 // node i's partner in round r of the tournament; -1: none
@@ -492,7 +551,8 @@ __device__ __forceinline__ int tourney_partner(int r, int i) {
 
 template <int D, int N, bool FACES, int EPB>
 __global__ void __launch_bounds__(FACES ? FxPairPar<D, N, EPB>::THREADS_F
-                                        : FxPairPar<D, N, EPB>::THREADS)
+                                        : FxPairPar<D, N, EPB>::THREADS,
+                                  FxPairPar<D, N, EPB>::MIN_CTAS)
     volume_fx_pp_kernel(double* u, double* __restrict__ du, const double* __restrict__ fs, Geom g,
                         Tables<double> tbg, unsigned* __restrict__ err, StageFuse fz, int sfk) {
   using C = FxPairPar<D, N, EPB>;
@@ -521,48 +581,60 @@ __global__ void __launch_bounds__(FACES ? FxPairPar<D, N, EPB>::THREADS_F
       const int e = e0 + el;
       const int owner = side == 0 ? e : neighbour32(g, e, dir, -1);
       double f[NV];
-      face_flux_nf_dir<D, N, double>(dir, u, g, sfk, owner, l, f);
+      face_flux_nf_dir<D, N, double, D == 3>(dir, u, g, sfk, owner, l, f);
       double* dst = sfc + (el * PER * NV + (side * D + dir) * NV * LINES + l);
 #pragma unroll
       for (int c = 0; c < NV; ++c) dst[c * LINES] = f[c];
     }
   } else {
-    const double sc0 = fz.k ? *fz.dt : 1.0;
-    int ed;
-    {
-      unsigned m = 0;
+    // one node per thread, its loads in flight while the tables are staged
+    const int t = threadIdx.x;
+    const bool in = t < count * P;
+    const int el = in ? t / P : 0, node = in ? t % P : 0;
+    double c[NV];
 #pragma unroll
-      for (int k = 0; k < D; ++k) {
-        const unsigned h = (unsigned)__double2hiint(sc0 * tbg.Ds[k][0][1]) & 0x7fffffffu;
-        m = h > m ? h : m;
-      }
-      ed = fx::exp_above(m);
+    for (int v = 0; v < NV; ++v) c[v] = in ? u[(long long)e0 * NV * P + (el * NV + v) * P + node] : 1.0;
+    const double sc0 = fz.k ? *fz.dt : 1.0;
+    unsigned m = 0;
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      const unsigned h = (unsigned)__double2hiint(sc0 * tbg.Ds[k][0][1]) & 0x7fffffffu;
+      m = h > m ? h : m;
     }
-    for (int i = threadIdx.x; i < D * NP * NP; i += wt) {
+    const int ed = fx::exp_above(m);
+    for (int i = t; i < D * NP * NP; i += wt) {
       const int dir = i / (NP * NP), a = (i / NP) % NP, b = i % NP;
       const double ds = sc0 * tbg.Ds[dir][a][b];
       tb.Ds[dir][a][b] = ds;
       sh.Ds[dir][a][b] = fx::limbs(fx::half_fixed(ds, ed));
     }
-    if ((int)threadIdx.x < D) {
-      tb.liftR[threadIdx.x] = sc0 * tbg.liftR[threadIdx.x];
-      tb.liftL[threadIdx.x] = sc0 * tbg.liftL[threadIdx.x];
+    if (t < D) {
+      tb.liftR[t] = sc0 * tbg.liftR[t];
+      tb.liftL[t] = sc0 * tbg.liftL[t];
     }
-    if ((int)threadIdx.x < count) {
-      fx_clear_key(sh.key[threadIdx.x]);
-      for (int k = 0; k < D; ++k)
-        sh.left[threadIdx.x][k] = neighbour32(g, e0 + threadIdx.x, k, -1);
+    if (t < count) {
+      fx_clear_key(sh.key[t]);
+      for (int k = 0; k < D; ++k) sh.left[t][k] = neighbour32(g, e0 + t, k, -1);
+    }
+    if (t == 0) sh.ed = ed;
+    int cb[2];
+    fx::scale_bits(g.gm1, cb);
+    FxPrim<D> q = {};
+    if (in) {
+      unsigned bad = 0;
+      q = fx_prim<D>(c, g, bad);
+      if (bad) atomicOr(err, bad);
     }
     vsync();
-    const unsigned bad = fx_load<D, N>(u, g, e0, count, smem, C::ELEM, sh.key, threadIdx.x, wt);
-    if (bad) atomicOr(err, bad);
+    const int first = (t & ~31) / P, lastt = (t | 31) < count * P ? (t | 31) : count * P - 1;
+    const FxKeys kk = fx_keys<D>(q);
+    for (int ek = first; ek <= lastt / P; ++ek) fx_merge_keys(kk, in && el == ek, sh.key[ek]);
     vsync();
-    if ((int)threadIdx.x < count) {
-      sh.scale[threadIdx.x] = fx_scale(sh.key[threadIdx.x], g.gm1, ed);
-      if (threadIdx.x == 0) sh.ed = ed;
+    if (in) {
+      const fx::Scale sc = fx_scale(sh.key[el], cb, ed);
+      if (node == 0) sh.scale[el] = sc;
+      fx_stage_node<D, N>(q, sc, g.gm1, smem + el * C::ELEM, fx_place<D, N>(node));
     }
-    vsync();
-    fx_stage<D, N>(g, count, smem, C::ELEM, sh.scale, threadIdx.x, wt);
     vsync();
   }
 #pragma unroll 1

@@ -35,6 +35,7 @@
 #include "dg_device.cuh"
 #include "dg_f32.cuh"
 #include "dg_fixed.cuh"
+#include "dg_fixed_face.cuh"
 
 namespace dg {
 
@@ -508,7 +509,7 @@ __device__ __forceinline__ double pick(const double* a, int k) {
 // tangential momenta (directions dir+1, dir+2), f[D+1] energy. dir is a
 // value (the face kernel passes a constant, the one-launch small-mesh kernel
 // its thread's direction: the same arithmetic either way).
-template <int D, int N, typename R>
+template <int D, int N, typename R, bool FIXED = true>
 __device__ __forceinline__ void face_flux_nf_dir(int dir, const double* __restrict__ u,
                                                  const Geom& g, int sf, int e, int l,
                                                  R f[D + 2]) {
@@ -517,12 +518,32 @@ __device__ __forceinline__ void face_flux_nf_dir(int dir, const double* __restri
   const R gamma = R(g.gamma), gm1inv = R(g.gm1inv);
   const int t1 = (dir + 1) % D, t2 = (dir + 2) % D;
   const int er = neighbour32(g, e, dir, +1);
-  const int nl = line_node_rt<D, N>(dir, l, N), nr = line_node_rt<D, N>(dir, l, 0);
+  const int ndl = line_node_rt<D, N>(dir, l, N), ndr = line_node_rt<D, N>(dir, l, 0);
   double cl[NV], cr[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    cl[v] = u[((long long)e * NV + v) * P + nl];
-    cr[v] = u[((long long)er * NV + v) * P + nr];
+    cl[v] = u[((long long)e * NV + v) * P + ndl];
+    cr[v] = u[((long long)er * NV + v) * P + ndr];
+  }
+  // small 2D meshes have one warp of faces per CTA, whose FP64 chain is the
+  // shorter one (16^2 N = 1..3: 35 to 43 us per graph step, 37 to 45 in fixed
+  // point; FIXED false keeps the other form's code out of their kernel);
+  // elsewhere the fixed-point form
+  if (FIXED && (sf == kSLLF || sf == kSHLL) && (D == 3 || g.nelem >= kPairParallelElems)) {
+    double nl[NV], nr[NV];  // normal component first
+    nl[0] = cl[0];
+    nr[0] = cr[0];
+    nl[1] = pick<D>(cl + 1, dir);
+    nr[1] = pick<D>(cr + 1, dir);
+    nl[2] = pick<D>(cl + 1, t1);
+    nr[2] = pick<D>(cr + 1, t1);
+    if (D == 3) {
+      nl[D] = pick<D>(cl + 1, t2);
+      nr[D] = pick<D>(cr + 1, t2);
+    }
+    nl[D + 1] = cl[D + 1];
+    nr[D + 1] = cr[D + 1];
+    if (fx::face_fixed<D>(sf == kSHLL, nl, nr, g.gamma, g.gm1, f)) return;
   }
   Trace<R, D> L, Rt;
   double rrl, rrr;
@@ -560,31 +581,9 @@ __device__ __forceinline__ void face_flux_nf_dir(int dir, const double* __restri
   surface_nf<R, D>(sf, L, Rt, dE, gamma, gm1inv, f);
 }
 
-template <int D, int N, typename R, int dir>
-__device__ __forceinline__ void face_flux_nf(const double* __restrict__ u, const Geom& g, int sf,
-                                             int e, int l, R f[D + 2]) {
-  face_flux_nf_dir<D, N, R>(dir, u, g, sf, e, l, f);
-}
-
-template <int D, int N, typename R, int dir>
-__device__ __forceinline__ void face_flux(const double* __restrict__ u, R* __restrict__ fs,
-                                          const Geom& g, int sf, int e, int l) {
-  constexpr int NV = D + 2, NF = Shape<D, N>::LINES;
-  constexpr int t1 = (dir + 1) % D, t2 = (dir + 2) % D;
-  const int nelem = (int)g.nelem;
-  R f[NV];
-  face_flux_nf<D, N, R, dir>(u, g, sf, e, l, f);
-  const long long base = (long long)nelem * NF;
-  const long long off = (long long)e * NF + l;
-  fs[(long long)(dir * NV + 0) * base + off] = f[0];
-  fs[(long long)(dir * NV + 1 + dir) * base + off] = f[1];
-  fs[(long long)(dir * NV + 1 + t1) * base + off] = f[2];
-  if (D == 3) fs[(long long)(dir * NV + 1 + t2) * base + off] = f[D];
-  fs[(long long)(dir * NV + NV - 1) * base + off] = f[NV - 1];
-}
-
-// face_flux with the direction as a value: warps whose lanes hold faces of
-// different directions run one instruction stream (the same arithmetic)
+// its store in fs[dir][v][e][l]. The direction is a value: one code body serves
+// every direction, and warps whose lanes hold faces of different directions run
+// one instruction stream
 template <int D, int N, typename R>
 __device__ __forceinline__ void face_flux_rt(int dir, const double* __restrict__ u,
                                              R* __restrict__ fs, const Geom& g, int sf, int e,
@@ -603,21 +602,13 @@ __device__ __forceinline__ void face_flux_rt(int dir, const double* __restrict__
   fs[(long long)(dir * NV + NV - 1) * base + off] = f[NV - 1];
 }
 
-template <int D, int N, typename R, int dir>
-__device__ __forceinline__ void surface_body(const double* __restrict__ u, R* __restrict__ fs,
-                                             const Geom& g, int sf) {
+template <int D, int N, typename R>
+__global__ void __launch_bounds__(256, 3) surface_kernel(const double* __restrict__ u, R* __restrict__ fs, Geom g, int sf) {
   constexpr int NF = Shape<D, N>::LINES;
   const long long total = g.nelem * NF;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x)
-    face_flux<D, N, R, dir>(u, fs, g, sf, (int)(t / NF), (int)(t % NF));
-}
-
-template <int D, int N, typename R>
-__global__ void surface_kernel(const double* __restrict__ u, R* __restrict__ fs, Geom g, int sf) {
-  if (blockIdx.y == 0) surface_body<D, N, R, 0>(u, fs, g, sf);
-  else if (blockIdx.y == 1) surface_body<D, N, R, 1>(u, fs, g, sf);
-  else surface_body<D, N, R, (D == 3 ? 2 : 1)>(u, fs, g, sf);
+    face_flux_rt<D, N, R>(blockIdx.y, u, fs, g, sf, (int)(t / NF), (int)(t % NF));
 }
 
 // ---- pair-parallel volume kernel for tiny meshes (FP64) ----
@@ -752,7 +743,7 @@ __device__ __forceinline__ void pp_elements(double* u, double* __restrict__ du,
         const int e = e0 + el;
         const int owner = side == 0 ? e : neighbour32(g, e, dir, -1);
         double f[NV];
-        face_flux_nf_dir<D, N, double>(dir, u, g, sfk, owner, l, f);
+        face_flux_nf_dir<D, N, double, D == 3>(dir, u, g, sfk, owner, l, f);
         double* dst = sfc + (long long)el * PER * NV + (side * D + dir) * NV * LINES + l;
 #pragma unroll
         for (int c = 0; c < NV; ++c) dst[c * LINES] = f[c];

@@ -39,7 +39,90 @@ __device__ __forceinline__ i64 normalised(i64 d, int& n) {
   return d << n;
 }
 
+// sqrt(x 2^-62) in 2^-62 for 0 <= x < 2^62, within a few units of the shifted
+// argument's 2^-60: a 23-bit reciprocal square root, then g += (x - g^2) r/2
+// twice (each squares the relative error down to the residual's rounding)
+__device__ __forceinline__ i64 sqrt_fixed(i64 x) {
+  if (x <= 0) return 0;
+  const int n = (__clzll(x) - 2) & ~1;
+  const i64 xs = x << n;  // in [2^60, 2^62)
+  const float f = __int2float_rn((int)(xs >> 32)) * 0x1p-30f;
+  const Limbs r = limbs((i64)__float2int_rn(rsqrtf(f) * 0x1p29f) << 32);  // 61
+  i64 g = mul(limbs(xs), r) << 3;                                         // 62
+  i64 d = (xs >> 2) - sqr(limbs(g));                                      // 60, below 2^40
+  g += mul(limbs(d << 20), r) >> 16;
+  d = (xs >> 2) - sqr(limbs(g));                                          // below 2^20
+  g += mul(limbs(d << 40), r) >> 36;
+  return g >> (n / 2);
+}
+
 __device__ __forceinline__ i64 abs64(i64 a) { return a < 0 ? -a : a; }
+
+// f = fr + w (fl - fr) + kappa (qR - qL) of the two traces, for LLF (w = 1/2,
+// kappa = -lambda/2) and HLL (w = sR/(sR - sL), kappa = w sL)
+struct FaceBlend {
+  bool hll;
+  Limbs kap, w;  // kappa (62 - eL + kx), w (62)
+  int eL, kx;
+
+  // from the normal velocities (62 - ev) and sound speeds (62 - ec; LLF: the
+  // larger one in both)
+  __device__ __forceinline__ void speeds(bool is_hll, i64 vl, i64 vr, int ev, i64 cl, i64 cr,
+                                         int ec) {
+    hll = is_hll;
+    eL = (ev > ec ? ev : ec) + 1;
+    const int dv = eL - ev < 63 ? eL - ev : 63, dc = eL - ec < 63 ? eL - ec : 63;
+    vl >>= dv;
+    vr >>= dv;
+    cl >>= dc;
+    cr >>= dc;
+    i64 k, x = 0;
+    kx = 0;
+    if (!hll) {
+      const i64 a = abs64(vl), b = abs64(vr);
+      k = -((a > b ? a : b) + cl);  // -lambda
+      kx = 1;                       // halved
+    } else {
+      const i64 sL = vl - cl < vr - cr ? vl - cl : vr - cr;
+      const i64 sR = vl + cl > vr + cr ? vl + cl : vr + cr;
+      if (sL >= 0) {
+        x = 1LL << 62;
+        k = 0;
+      } else if (sR <= 0) {
+        x = 0;
+        k = 0;
+      } else {
+        // sR/(sR - sL), both speeds below 2^62: the quotient in FP64
+        const double sr = to_double(sR, 0), sl = to_double(sL, 0);
+        x = half_fixed(sr * rcp(sr - sl), 0);
+        if (x > (1LL << 62)) x = 1LL << 62;
+        k = mul(limbs(x), limbs(sL)) << 2;
+      }
+    }
+    kap = limbs(k);
+    w = limbs(x);
+  }
+  // one component: the fluxes in units 2^ea, the jump d in 2^ed
+  __device__ __forceinline__ double operator()(i64 fl, i64 fr, int ea, i64 d, int ed) const {
+    i64 a;
+    if (!hll) {
+      a = (fl >> 1) + (fr >> 1);
+    } else {
+      a = (fr >> 1) + (mul(w, limbs((fl >> 1) - (fr >> 1))) << 2);
+    }
+    ea += hll ? 1 : 0;
+    int n;
+    const i64 dn = normalised(d, n);
+    const i64 b = mul(kap, limbs(dn));
+    const int eb = ed - n + eL + 2 - kx;
+    if (b == 0) return to_double_int(a, ea);
+    if (a == 0) return to_double_int(b, eb);
+    // both to the coarser unit, one bit of headroom
+    const int base = (ea > eb ? ea : eb) + 1;
+    const int sa = base - ea < 63 ? base - ea : 63, sb = base - eb < 63 ? base - eb : 63;
+    return to_double_int((a >> sa) + (b >> sb), base);
+  }
+};
 
 // one trace: v (62 - ev, normal first), p (62 - ee), c2 = p/rho (61 - ee - er1)
 // and the physical flux: mass (62 - em), momenta (61 - em - ev, without p),
@@ -51,9 +134,8 @@ struct FaceSide {
   i64 vn, p, c2, fm[D], fe;
 };
 
-// f = fr + w (fl - fr) + kappa (qR - qL) for LLF (w = 1/2, kappa = -lambda/2)
-// and HLL (w = sR/(sR - sL), kappa = w sL) from the conserved traces, normal
-// component first. Returns false (f not written) if the FP64 form is due.
+// LLF or HLL from the conserved traces, normal component first. Returns false
+// (f not written) if the FP64 form is due.
 template <int D>
 __device__ __forceinline__ bool face_fixed(bool hll, const double* cl, const double* cr,
                                            double gamma, double gm1, double f[D + 2]) {
@@ -133,56 +215,9 @@ __device__ __forceinline__ bool face_fixed(bool hll, const double* cl, const dou
   const double cb = hll ? sqrt_pos(gamma * to_double(S[1].c2, ec)) : ca;
   const unsigned kc = hiword(ca) > hiword(cb) ? hiword(ca) : hiword(cb);
   if (kc >= hi) return false;
-  int eL = exp_above(kc) + 1;
-  if (eL < ev + 1) eL = ev + 1;
-  const int dv = eL - ev < 63 ? eL - ev : 63;
-  i64 kap;                       // kappa in 62 - eL + kx
-  int kx = 0;
-  i64 w = 0;                     // HLL: w in 62
-  if (!hll) {
-    const i64 a = abs64(S[0].vn), b = abs64(S[1].vn);
-    kap = -(((a > b ? a : b) >> dv) + half_fixed(ca, eL));  // -lambda
-    kx = 1;                                                 // halved
-  } else {
-    const i64 vl = S[0].vn >> dv, vr = S[1].vn >> dv;
-    const i64 xl = half_fixed(ca, eL), xr = half_fixed(cb, eL);
-    const i64 sL = vl - xl < vr - xr ? vl - xl : vr - xr;
-    const i64 sR = vl + xl > vr + xr ? vl + xl : vr + xr;
-    if (sL >= 0) {
-      w = 1LL << 62;
-      kap = 0;
-    } else if (sR <= 0) {
-      w = 0;
-      kap = 0;
-    } else {
-      // sR/(sR - sL), both speeds below 2^62: the quotient in FP64
-      const double sr = to_double(sR, 0), sl = to_double(sL, 0);
-      w = half_fixed(sr * rcp(sr - sl), 0);
-      if (w > (1LL << 62)) w = 1LL << 62;
-      kap = mul(limbs(w), limbs(sL)) << 2;
-    }
-  }
-  const Limbs kl = limbs(kap), wl = limbs(w);
-  // one component: the mean part a (units 2^ea) plus kappa d (d in 2^ed)
-  auto blend = [&](i64 fl, i64 fr, int ea, i64 d, int ed) {
-    i64 a;
-    if (!hll) {
-      a = (fl >> 1) + (fr >> 1);
-    } else {
-      a = (fr >> 1) + (mul(wl, limbs((fl >> 1) - (fr >> 1))) << 2);
-    }
-    ea += hll ? 1 : 0;
-    int n;
-    const i64 dn = normalised(d, n);
-    i64 b = mul(kl, limbs(dn));  // units 2^(64 + ed - n + eL - 62 - kx)
-    int eb = ed - n + eL + 2 - kx;
-    if (b == 0) return to_double_int(a, ea);
-    if (a == 0) return to_double_int(b, eb);
-    // align the finer one to the coarser one's unit, one bit of headroom
-    const int base = (ea > eb ? ea : eb) + 1;
-    const int sa = base - ea < 63 ? base - ea : 63, sb = base - eb < 63 ? base - eb : 63;
-    return to_double_int((a >> sa) + (b >> sb), base);
-  };
+  const int es = exp_above(kc);
+  FaceBlend blend;
+  blend.speeds(hll, S[0].vn, S[1].vn, ev, half_fixed(ca, es), half_fixed(cb, es), es);
   const i64 drho = full_fixed(cr[0], er) - full_fixed(cl[0], er);
   f[0] = blend(S[0].m[0], S[1].m[0], em - 63, drho, er - 63);
 #pragma unroll

@@ -25,11 +25,12 @@
 //     min(v_n,L - c_f,L, v_n,R - c_f,R), S_R = max(v_n,L + c_f,L, v_n,R +
 //     c_f,R), or the EC flux; and {B_n}; nine values per face node in
 //     fs[dir][q][e_left][l].
-//   mhd_volume_kernel (weak form): one CTA per EPB elements, one thread per
-//     node; per direction each thread writes f(u_i) (B_n in the slot of the
-//     zero normal induction flux) to shared memory, then applies its line's
-//     row of Dn and the lifting; epilogue: the Powell term, then the store
-//     of du or the fused stage update.
+//   mhd_volume_weak_kernel (weak form, dg_mhd_weak.cuh): one CTA per EPB
+//     elements, one thread per node; per direction each thread writes f(u_i)
+//     (B_n in the slot of the zero normal induction flux) to shared memory,
+//     then applies its line's row of Dn, in 64-bit fixed point; epilogue: the
+//     lifting, the Powell term, then the store of du or the fused stage
+//     update.
 //   mhd_volume_ec_kernel (EC flux differencing): one element per CTA; per
 //     direction one thread per (line, node pair) evaluates f# once for both
 //     nodes, then one thread per node sums its line (below).
@@ -39,6 +40,7 @@
 
 #include "dg_curved.cuh"  // pair_of, pair_index, line_of
 #include "dg_device.cuh"
+#include "dg_fixed_face.cuh"
 #include "dg_mhd_decl.cuh"
 
 namespace dg {
@@ -166,185 +168,70 @@ __device__ __forceinline__ void mhd_ec_flux(const ECq& a, const ECq& b, double h
   f[4] = fma(Ba[DIR], a.hvB + b.hvB, e);
 }
 
-template <int N, int DIR, int SF>
-__device__ __forceinline__ void mhd_surface_body(const double* __restrict__ u,
-                                                 double* __restrict__ fs, const Geom& g,
-                                                 unsigned& bad) {
+#include "dg_mhd_weak.cuh"
+
+// One thread per face node; the traces are read normal component first, so one
+// code body (direction 0) serves every direction. LLF and HLL in fixed point
+// (mhd_face_fixed), their FP64 form for the faces it declines.
+template <int N, int SF>
+__global__ void __launch_bounds__(256, SF == kMhdEc ? 1 : 2)
+    mhd_surface_kernel(const double* __restrict__ u, double* __restrict__ fs, Geom g,
+                       unsigned* __restrict__ err) {
   constexpr int NP = N + 1, P = NP * NP * NP, NF = NP * NP;
+  const int dir = blockIdx.y, t1 = dir == 2 ? 0 : dir + 1, t2 = t1 == 2 ? 0 : t1 + 1;
+  const int X[kMV] = {0, 1 + dir, 1 + t1, 1 + t2, 4, 5 + dir, 5 + t1, 5 + t2};
+  unsigned bad = 0;
   const long long total = g.nelem * NF;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += (long long)gridDim.x * blockDim.x) {
     const long long e = t / NF;
     const int l = (int)(t % NF);
-    const long long er = neighbour(g, e, DIR, +1);
-    const int nl = line_node<3, N, DIR>(l, N), nr = line_node<3, N, DIR>(l, 0);
-    double cl[kMV], cr[kMV];
+    const long long er = neighbour(g, e, dir, +1);
+    const int nl = line_node_rt<3, N>(dir, l, N), nr = line_node_rt<3, N>(dir, l, 0);
+    double cl[kMV], cr[kMV], f[kMV];
 #pragma unroll
     for (int v = 0; v < kMV; ++v) {
-      cl[v] = u[(e * kMV + v) * P + nl];
-      cr[v] = u[(er * kMV + v) * P + nr];
+      cl[v] = u[(e * kMV + X[v]) * P + nl];
+      cr[v] = u[(er * kMV + X[v]) * P + nr];
     }
-    const MState sl = mhd_state(cl, g.gm1, bad), sr = mhd_state(cr, g.gm1, bad);
-    double fl[kMV], fr[kMV];
-    mhd_flux<DIR>(sl, cl, fl);
-    mhd_flux<DIR>(sr, cr, fr);
+    if (SF == kMhdEc || !mhd_face_fixed(SF == kMhdHll, cl, cr, g.gamma, g.gm1, f)) {
+      const MState sl = mhd_state(cl, g.gm1, bad), sr = mhd_state(cr, g.gm1, bad);
+      if (SF == kMhdEc) {
+        mhd_ec_flux<0>(ec_of(sl), ec_of(sr), 0.5 * g.gm1inv, f);
+      } else {
+        double fl[kMV], fr[kMV];
+        mhd_flux<0>(sl, cl, fl);
+        mhd_flux<0>(sr, cr, fr);
+        if (SF == kMhdHll) {
+          const double cfl = sqrt(fast_speed2<0>(sl, g.gamma));
+          const double cfr = sqrt(fast_speed2<0>(sr, g.gamma));
+          const double sL = fmin(sl.v[0] - cfl, sr.v[0] - cfr);
+          const double sR = fmax(sl.v[0] + cfl, sr.v[0] + cfr);
+          const double inv = 1.0 / (sR - sL);
+#pragma unroll
+          for (int v = 0; v < kMV; ++v) {
+            if (sL >= 0.0) f[v] = fl[v];
+            else if (sR <= 0.0) f[v] = fr[v];
+            else f[v] = (sR * fl[v] - sL * fr[v] + sL * sR * (cr[v] - cl[v])) * inv;
+          }
+        } else {
+          // max(c_L, c_R) = sqrt(max(c_L^2, c_R^2)) exactly (sqrt is monotone
+          // and correctly rounded)
+          const double lam = fmax(fabs(sl.v[0]), fabs(sr.v[0])) +
+                             sqrt(fmax(fast_speed2<0>(sl, g.gamma), fast_speed2<0>(sr, g.gamma)));
+#pragma unroll
+          for (int v = 0; v < kMV; ++v)
+            f[v] = 0.5 * (fl[v] + fr[v]) - 0.5 * lam * (cr[v] - cl[v]);
+        }
+      }
+    }
     const long long base = g.nelem * NF;
-    const long long off = e * NF + l;
-    if (SF == kMhdEc) {
-      double f[kMV];
-      mhd_ec_flux<DIR>(ec_of(sl), ec_of(sr), 0.5 * g.gm1inv, f);
+    double* dst = fs + (long long)dir * kMQ * base + e * NF + l;
 #pragma unroll
-      for (int v = 0; v < kMV; ++v) fs[(long long)(DIR * kMQ + v) * base + off] = f[v];
-    } else if (SF == kMhdHll) {
-      const double cfl = sqrt(fast_speed2<DIR>(sl, g.gamma));
-      const double cfr = sqrt(fast_speed2<DIR>(sr, g.gamma));
-      const double sL = fmin(sl.v[DIR] - cfl, sr.v[DIR] - cfr);
-      const double sR = fmax(sl.v[DIR] + cfl, sr.v[DIR] + cfr);
-      const double inv = 1.0 / (sR - sL);
-#pragma unroll
-      for (int v = 0; v < kMV; ++v) {
-        double F;
-        if (sL >= 0.0) F = fl[v];
-        else if (sR <= 0.0) F = fr[v];
-        else F = (sR * fl[v] - sL * fr[v] + sL * sR * (cr[v] - cl[v])) * inv;
-        fs[(long long)(DIR * kMQ + v) * base + off] = F;
-      }
-    } else {
-      // max(c_L, c_R) = sqrt(max(c_L^2, c_R^2)) exactly (sqrt is monotone
-      // and correctly rounded)
-      const double lam = fmax(fabs(sl.v[DIR]), fabs(sr.v[DIR])) +
-                         sqrt(fmax(fast_speed2<DIR>(sl, g.gamma), fast_speed2<DIR>(sr, g.gamma)));
-#pragma unroll
-      for (int v = 0; v < kMV; ++v)
-        fs[(long long)(DIR * kMQ + v) * base + off] =
-            0.5 * (fl[v] + fr[v]) - 0.5 * lam * (cr[v] - cl[v]);
-    }
-    fs[(long long)(DIR * kMQ + 8) * base + off] = 0.5 * (cl[5 + DIR] + cr[5 + DIR]);
+    for (int v = 0; v < kMV; ++v) dst[X[v] * base] = f[v];
+    dst[8 * base] = 0.5 * (cl[5] + cr[5]);
   }
-}
-
-template <int N, int SF>
-__global__ void mhd_surface_kernel(const double* __restrict__ u, double* __restrict__ fs, Geom g,
-                                   unsigned* __restrict__ err) {
-  unsigned bad = 0;
-  if (blockIdx.y == 0) mhd_surface_body<N, 0, SF>(u, fs, g, bad);
-  else if (blockIdx.y == 1) mhd_surface_body<N, 1, SF>(u, fs, g, bad);
-  else mhd_surface_body<N, 2, SF>(u, fs, g, bad);
   if (bad) atomicOr(err, bad);
-}
-
-// one direction of the volume pass for the thread's node (index ia along
-// DIR). The normal induction flux v_n B_n - B_n v_n is zero, so its shared-
-// memory slot 5 + DIR carries B_n instead, whose derivative goes to -div B;
-// du of B_n gets only the lifting of F*_{5+DIR} (the LLF dissipation).
-// Contributions accumulate straight into acc and divneg.
-template <int N, int DIR, int EPB>
-__device__ __forceinline__ void mhd_direction(const MState& s, const double* c,
-                                              double (*sf)[kMV][(N + 1) * (N + 1) * (N + 1)],
-                                              const double (*sD)[N + 1][N + 1], int el, int node,
-                                              bool active, long long e, const Geom& g,
-                                              const Tables<double>& tb,
-                                              const double* __restrict__ fs, double* acc,
-                                              double& divneg) {
-  constexpr int NP = N + 1, NF = NP * NP;
-  constexpr int STRIDE = DIR == 0 ? 1 : (DIR == 1 ? NP : NF);
-  constexpr int QB = 5 + DIR;  // the slot of B_n
-  if (active) {
-    double f[kMV];
-    mhd_flux<DIR>(s, c, f);
-    f[QB] = s.B[DIR];
-#pragma unroll
-    for (int q = 0; q < kMV; ++q) sf[el][q][node] = f[q];
-  }
-  __syncthreads();
-  if (active) {
-    const int ia = (node / STRIDE) % NP;
-    const int first = node - ia * STRIDE;
-#pragma unroll
-    for (int b = 0; b < NP; ++b) {
-      const double w = sD[DIR][ia][b];
-#pragma unroll
-      for (int q = 0; q < kMV; ++q) {
-        if (q == QB) divneg = fma(w, sf[el][q][first + b * STRIDE], divneg);
-        else acc[q] = fma(w, sf[el][q][first + b * STRIDE], acc[q]);
-      }
-    }
-    if (ia == N || ia == 0) {
-      // face-node index of this line (see line_node)
-      const int l = DIR == 0 ? node / NP : (DIR == 1 ? node % NP + NP * (node / NF) : node % NF);
-      const long long ef = ia == N ? e : neighbour(g, e, DIR, -1);
-      const double lift = ia == N ? tb.liftR[DIR] : tb.liftL[DIR];
-      const long long base = g.nelem * NF;
-      const double* src = fs + (long long)DIR * kMQ * base + ef * NF + l;
-#pragma unroll
-      for (int q = 0; q < kMV; ++q) {
-        if (q == QB) acc[q] = fma(lift, src[q * base], acc[q]);
-        else acc[q] = fma(lift, src[q * base] - sf[el][q][node], acc[q]);
-      }
-      divneg = fma(lift, src[8 * base] - sf[el][QB][node], divneg);
-    }
-  }
-  __syncthreads();
-}
-
-template <int N, int EPB>
-__global__ void __launch_bounds__(EPB*(N + 1) * (N + 1) * (N + 1),
-                                  (EPB * (N + 1) * (N + 1) * (N + 1) <= kMhdThreads) ? kMhdMinBlocks
-                                                                                   : 1)
-    mhd_volume_kernel(double* u, double* __restrict__ du, const double* __restrict__ fs, Geom g,
-                      Tables<double> tb, int powell, unsigned* __restrict__ err, StageFuse fz) {
-  constexpr int NP = N + 1, P = NP * NP * NP;
-  extern __shared__ __align__(16) unsigned char dg_smem[];
-  double(*sf)[kMV][P] = reinterpret_cast<double(*)[kMV][P]>(dg_smem);
-  // the derivative rows, indexed per thread: from shared memory rather than
-  // the parameter bank, whose divergent reads serialise
-  __shared__ double sD[3][NP][NP];
-  for (int t = threadIdx.x; t < 3 * NP * NP; t += blockDim.x)
-    sD[t / (NP * NP)][(t / NP) % NP][t % NP] = tb.Ds[t / (NP * NP)][(t / NP) % NP][t % NP];
-  const int el = threadIdx.x / P, node = threadIdx.x % P;
-  const long long e = (long long)blockIdx.x * EPB + el;
-  const bool active = e < g.nelem;
-  double c[kMV];
-  if (active) {
-#pragma unroll
-    for (int v = 0; v < kMV; ++v) c[v] = u[(e * kMV + v) * P + node];
-  } else {
-#pragma unroll
-    for (int v = 0; v < kMV; ++v) c[v] = (v == 0 || v == 4) ? 1.0 : 0.0;
-  }
-  unsigned bad = 0;
-  const MState s = mhd_state(c, g.gm1, bad);
-  if (bad && active) atomicOr(err, bad);
-  double acc[kMV], divneg = 0.0;
-#pragma unroll
-  for (int v = 0; v < kMV; ++v) acc[v] = 0.0;
-  mhd_direction<N, 0, EPB>(s, c, sf, sD, el, node, active, e, g, tb, fs, acc, divneg);
-  mhd_direction<N, 1, EPB>(s, c, sf, sD, el, node, active, e, g, tb, fs, acc, divneg);
-  mhd_direction<N, 2, EPB>(s, c, sf, sD, el, node, active, e, g, tb, fs, acc, divneg);
-  if (!active) return;
-  if (powell) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      acc[1 + k] = fma(s.B[k], divneg, acc[1 + k]);
-      acc[5 + k] = fma(s.v[k], divneg, acc[5 + k]);
-    }
-    acc[4] = fma(s.vb, divneg, acc[4]);
-  }
-  const double dtv = fz.k ? *fz.dt : 0.0;
-  double* const uo = fz.u_out ? fz.u_out : u;
-#pragma unroll
-  for (int v = 0; v < kMV; ++v) {
-    const long long i = (e * kMV + v) * P + node;
-    if (fz.k) {
-      // the first stage (A = 0) neither reads k nor lets stale k values in
-      double kk = dtv * acc[v];
-      if (fz.a != 0.0) kk = fma(fz.a, fz.k[i], kk);
-      fz.k[i] = kk;
-      uo[i] = u[i] + fz.b * kk;
-    } else {
-      du[i] = acc[v];
-    }
-  }
 }
 
 // ---- entropy-conservative flux differencing: one element per CTA ----
@@ -985,14 +872,15 @@ cudaError_t mhd_volume_epb(const double* u, double* du, const double* fs, const 
                            const StageFuse& fz) {
   constexpr int P = MLaunch<N>::P;
   constexpr int SMEM = EPB * kMV * P * (int)sizeof(double);
-  auto kern = mhd_volume_kernel<N, EPB>;
+  constexpr int THREADS = 32 * ((EPB * P + 31) / 32);
+  auto kern = mhd_volume_weak_kernel<N, EPB>;
   if (SMEM > 48 * 1024) {
     const cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e != cudaSuccess) return e;
   }
   const long long grid = (g.nelem + EPB - 1) / EPB;
-  kern<<<(unsigned)grid, EPB * P, SMEM, st>>>(const_cast<double*>(u), du, fs, g, tb, powell, err,
+  kern<<<(unsigned)grid, THREADS, SMEM, st>>>(const_cast<double*>(u), du, fs, g, tb, powell, err,
                                                fz);
   return cudaGetLastError();
 }

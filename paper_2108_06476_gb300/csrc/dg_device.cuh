@@ -298,6 +298,31 @@ __device__ __forceinline__ double sqrt_pos(double x) {
 }
 __device__ __forceinline__ float sqrt_pos(float x) { return sqrtf(x); }
 
+// ---- wave speeds ----
+// Upper bounds of a node's wave speeds |v_k| + c in FP32: the pressure is
+// raised by a bound of its rounding (it cancels against the kinetic energy),
+// the rest by more than theirs. False if the node's state is too close to the
+// limits of physical states (or of FP32) for the bound to hold.
+template <int D>
+__device__ __forceinline__ bool speed_bound(const double* c, double gamma64, double gm164,
+                                            float* lam) {
+  const float gm1 = d2f(gm164), gamma = d2f(gamma64);
+  const float rho = d2f(c[0]), E = d2f(c[D + 1]);
+  const float r = 1.0f / rho;
+  float v[D], mv = 0.0f;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    const float m = d2f(c[1 + k]);
+    v[k] = m * r;
+    mv = fmaf(m, v[k], mv);
+  }
+  const float p = gm1 * (E - 0.5f * mv), off = gm1 * 2e-6f * (fabsf(E) + mv);
+  const float cs = sqrtf(gamma * (p + off) * r);
+#pragma unroll
+  for (int k = 0; k < D; ++k) lam[k] = fmaxf(lam[k], (fabsf(v[k]) + cs) * 1.000004f);
+  return rho > 1e-30f && rho < 1e30f && p > off && p > 1e-30f && E < 1e30f;
+}
+
 // ---- logarithmic mean ----
 // ln_mean(x, y) = (y - x) / ln(y / x). With s = x + y, t = (y - x)/s and
 // f2 = t^2, ln(y/x) = 2 atanh(t), so

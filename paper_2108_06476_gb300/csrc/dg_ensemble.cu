@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(kEnsMaxThreads, sizeof(R) == 8 ? 6 : 3) ensemb
 __global__ void ensemble_speed_kernel(const SimDesc* __restrict__ sims,
                                       const WorkItem* __restrict__ items, int nitems,
                                       const double* __restrict__ u, double gamma, double gm1,
-                                      unsigned long long* __restrict__ smax,
+                                      unsigned long long* smax,
                                       unsigned* __restrict__ err) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   unsigned bad = 0;
@@ -267,6 +267,26 @@ __global__ void ensemble_speed_kernel(const SimDesc* __restrict__ sims,
     const int P = (sd.N + 1) * (sd.N + 1) * (sd.N + 1);
     for (int el = warp; el < w.count; el += nw) {
       const long long base = sd.off + (long long)(w.e0 + el) * 5 * P;
+      // in FP64 only if the FP32 bound of the element's sum is not below the
+      // member's largest sum so far (see speed_kernel)
+      const unsigned long long seen = *(volatile unsigned long long*)(smax + w.sim);
+      float up[3] = {0.0f, 0.0f, 0.0f}, bound = 0.0f;
+      bool fine = true;
+      for (int node = lane; node < P; node += 32) {
+        double c[5];
+#pragma unroll
+        for (int v = 0; v < 5; ++v) c[v] = u[base + (long long)v * P + node];
+        fine = speed_bound<3>(c, gamma, gm1, up) && fine;
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        for (int off = 16; off > 0; off >>= 1)
+          up[k] = fmaxf(up[k], __shfl_xor_sync(0xffffffffu, up[k], off));
+        bound = fmaf((float)sd.lam_scale[k] * 1.000001f, up[k], bound);
+      }
+      if (__all_sync(0xffffffffu, fine) && bound > 1e-30f &&
+          bound < d2f(__longlong_as_double((long long)seen)) * 0.999999f)
+        continue;
       double lam[3] = {0.0, 0.0, 0.0};
       for (int node = lane; node < P; node += 32) {
         double c[5];

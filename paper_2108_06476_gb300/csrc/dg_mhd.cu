@@ -393,16 +393,48 @@ __global__ void __launch_bounds__(MPairs<N>::THREADS)
   }
 }
 
+// upper bounds of a node's wave speeds |v_k| + c_f,k in FP32 (see speed_bound
+// of the Euler pass): the pressure and the discriminant, which cancel, raised
+// by bounds of their rounding. False if the bound may not hold.
+__device__ __forceinline__ bool mhd_speed_bound(const double* c, const Geom& g, float* lam) {
+  const float gm1 = d2f(g.gm1), gamma = d2f(g.gamma);
+  const float rho = d2f(c[0]), E = d2f(c[4]);
+  const float r = 1.0f / rho;
+  float v[3], B[3], mv = 0.0f, b2 = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float m = d2f(c[1 + k]);
+    v[k] = m * r;
+    mv = fmaf(m, v[k], mv);
+    B[k] = d2f(c[5 + k]);
+    b2 = fmaf(B[k], B[k], b2);
+  }
+  const float p = gm1 * (E - 0.5f * (mv + b2)), off = gm1 * 2e-6f * (fabsf(E) + mv + b2);
+  const float a2 = gamma * (p + off), q = a2 + b2;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float disc = fmaxf(q * q - 4.0f * a2 * B[k] * B[k], 0.0f) + 4e-6f * q * q;
+    lam[k] = fmaxf(lam[k], (fabsf(v[k]) + sqrtf(0.5f * r * (q + sqrtf(disc)))) * 1.000004f);
+  }
+  return rho > 1e-15f && rho < 1e15f && p > off && p > 1e-15f && E < 1e15f;
+}
+
+// As the Euler pass: an element is evaluated in FP64 (about 100 instructions
+// per node) only if its bound is not below the largest sum found so far by any
+// warp; the maximum is the same.
 __global__ void mhd_speed_kernel(const double* __restrict__ u, Geom g, int P, double s0, double s1,
                                  double s2, unsigned long long* out, unsigned* err,
-                                 double* __restrict__ copy_to) {
+                                 double* copy_to) {
   const int lane = threadIdx.x & 31;
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   double best = 0.0;
   unsigned bad = 0;
+  const float sf[3] = {(float)s0 * 1.000001f, (float)s1 * 1.000001f, (float)s2 * 1.000001f};
   for (long long e = warp; e < g.nelem; e += nwarps) {
-    double lam[3] = {0.0, 0.0, 0.0};
+    const unsigned long long seen = *(volatile unsigned long long*)out;
+    float up[3] = {0.0f, 0.0f, 0.0f}, bound = 0.0f;
+    bool fine = true;
     for (int node = lane; node < P; node += 32) {
       double c[kMV];
 #pragma unroll
@@ -411,6 +443,22 @@ __global__ void mhd_speed_kernel(const double* __restrict__ u, Geom g, int P, do
 #pragma unroll
         for (int v = 0; v < kMV; ++v) copy_to[(e * kMV + v) * P + node] = c[v];
       }
+      fine = mhd_speed_bound(c, g, up) && fine;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      for (int off = 16; off > 0; off >>= 1)
+        up[k] = fmaxf(up[k], __shfl_xor_sync(0xffffffffu, up[k], off));
+      bound = fmaf(sf[k], up[k], bound);
+    }
+    const double most = fmax(best, __longlong_as_double((long long)seen));
+    if (__all_sync(0xffffffffu, fine) && bound > 1e-30f && bound < d2f(most) * 0.999999f) continue;
+    const double* uc = copy_to ? copy_to : u;
+    double lam[3] = {0.0, 0.0, 0.0};
+    for (int node = lane; node < P; node += 32) {
+      double c[kMV];
+#pragma unroll
+      for (int v = 0; v < kMV; ++v) c[v] = uc[(e * kMV + v) * P + node];
       const MState s = mhd_state(c, g.gm1, bad);
       lam[0] = fmax(lam[0], fabs(s.v[0]) + sqrt(fast_speed2<0>(s, g.gamma)));
       lam[1] = fmax(lam[1], fabs(s.v[1]) + sqrt(fast_speed2<1>(s, g.gamma)));
@@ -423,6 +471,7 @@ __global__ void mhd_speed_kernel(const double* __restrict__ u, Geom g, int P, do
     double sum = s0 * lam[0];
     sum = sum + s1 * lam[1];
     sum = sum + s2 * lam[2];
+    if (lane == 0 && sum > best) atomicMax(out, (unsigned long long)__double_as_longlong(sum));
     best = fmax(best, sum);
   }
   __shared__ double sb[32];

@@ -377,8 +377,8 @@ int dg_ensemble_rk_reset(dg_ensemble *ens);
  * DG_ERR_TIMEOUT if a stage's barrier gave up; *flags gets the bits */
 int dg_ensemble_check(dg_ensemble *ens, int *flags);
 /* CTA shape: threads per CTA (multiple of 32, at most 128) and requested
- * resident CTAs per SM (the launch takes at most what fits); elements per
- * work item follow as threads / (N+1)^2 for each degree. */
+ * resident CTAs per SM (the launch takes at most what fits); the elements per
+ * work item follow for each degree (threads >= (N+1)^2 is required). */
 int dg_ensemble_set_block(dg_ensemble *ens, int threads, int blocks_per_sm);
 /* the current shape: threads per CTA, requested CTAs per SM, CTAs launched */
 int dg_ensemble_get_block(const dg_ensemble *ens, int *threads, int *ctas_per_sm, int *grid);

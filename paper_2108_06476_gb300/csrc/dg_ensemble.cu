@@ -362,12 +362,19 @@ struct dg_ensemble {
 
 namespace {
 
-// elements per work item for degree N with `block` threads per CTA
-int items_epb(int N, int block) {
+// elements per work item for degree N with `block` threads per CTA: FP64, as
+// many as one pass over their lines takes (Tourney: 32/T lines per warp; more
+// would only hold shared memory: 128 threads with an element per 16 to 36
+// threads left three CTAs per SM, 13.8 ms per stage of the 48 members against
+// 11.3); FP32, one thread per line
+int items_epb(int precision, int N, int block) {
   const int lines = (N + 1) * (N + 1);
   int e = block / lines;
-  if (e > kEnsMaxItem) e = kEnsMaxItem;
-  return e < 1 ? 0 : e;
+  if (precision == DG_FP64 && e > 0) {
+    const int lpw = N == 3 ? Tourney<3>::LPW : (N == 4 ? Tourney<4>::LPW : Tourney<5>::LPW);
+    e = std::max(1, block / 32 * lpw / lines);
+  }
+  return e > kEnsMaxItem ? kEnsMaxItem : e;
 }
 
 // dynamic shared memory of a work item: FP64, node slots + accumulators;
@@ -376,7 +383,7 @@ int items_epb(int N, int block) {
 int smem_for(int precision, int block, int pair) {
   int m = 0;
   for (int N = kEnsMinN; N <= kEnsMaxN; ++N) {
-    const int P = (N + 1) * (N + 1) * (N + 1), epb = pair ? 1 : items_epb(N, block);
+    const int P = (N + 1) * (N + 1) * (N + 1), epb = pair ? 1 : items_epb(precision, N, block);
     const int b = precision == DG_FP64 ? epb * (8 + 5) * P * 8
                                        : ((4 * epb * 14 * P + 15) & ~15) + 8 * epb * 5 * P;
     if (b > m) m = b;
@@ -387,7 +394,7 @@ int smem_for(int precision, int block, int pair) {
 int build_items(dg_ensemble* E) {
   std::vector<WorkItem> items;
   for (int N = kEnsMaxN; N >= kEnsMinN; --N) {
-    const int epb = items_epb(N, E->block);
+    const int epb = items_epb(E->opt.precision, N, E->block);
     if (epb < 1) return fail(DG_ERR_ARG, "dg_ensemble: CTA too small for the degree");
     for (int s = 0; s < E->nsims; ++s) {
       if (E->sims[s].N != N) continue;
@@ -540,7 +547,7 @@ int dg_ensemble_create(int n_sims, const int* d, const int* N, const int* elemen
   E->opt = o;
   E->stream = (cudaStream_t)cuda_stream;
   E->block = 128;
-  E->per_sm = 4;
+  E->per_sm = 6;  // at most what fits: FP64 six CTAs of 80 registers, FP32 three
   E->pair = 0;
   E->d_sims = nullptr;
   E->d_items = nullptr;
@@ -739,7 +746,7 @@ int dg_ensemble_set_block(dg_ensemble* E, int threads, int blocks_per_sm) {
       blocks_per_sm > 32)
     return fail(DG_ERR_ARG, "dg_ensemble_set_block: bad configuration");
   for (int N = kEnsMinN; N <= kEnsMaxN; ++N)
-    if (items_epb(N, threads) < 1) return fail(DG_ERR_ARG, "dg_ensemble_set_block: CTA too small");
+    if (items_epb(E->opt.precision, N, threads) < 1) return fail(DG_ERR_ARG, "dg_ensemble_set_block: CTA too small");
   cudaStreamSynchronize(E->stream);
   E->block = threads;
   E->per_sm = blocks_per_sm;

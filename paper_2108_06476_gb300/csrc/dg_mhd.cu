@@ -31,9 +31,9 @@
 //     then applies its line's row of Dn, in 64-bit fixed point; epilogue: the
 //     lifting, the Powell term, then the store of du or the fused stage
 //     update.
-//   mhd_volume_ec_kernel (EC flux differencing): one element per CTA; per
-//     direction one thread per (line, node pair) evaluates f# once for both
-//     nodes, then one thread per node sums its line (below).
+//   mhd_volume_ec_fx_kernel (EC flux differencing, dg_mhd_ec.cuh): f# once per
+//     node pair in 64-bit fixed point, the pairs of a line spread over several
+//     threads.
 //   mhd_speed_kernel: one warp per element; sum_dir (2/h) max(|v_dir| + c_f)
 //     into the mesh's wave-speed word (CFL step).
 #include <cuda_runtime.h>
@@ -41,6 +41,7 @@
 #include "dg_curved.cuh"  // pair_of, pair_index, line_of
 #include "dg_device.cuh"
 #include "dg_fixed_face.cuh"
+#include "dg_rhs_kernels.cuh"
 #include "dg_mhd_decl.cuh"
 
 namespace dg {
@@ -54,6 +55,9 @@ constexpr int kMhdLlf = 0, kMhdHll = 1, kMhdEc = 2;  // surface fluxes
 // kMhdMinBlocks resident CTAs per SM (80 registers a thread at 256 threads)
 constexpr int kMhdThreads = 256;
 constexpr int kMhdMinBlocks = 3;
+// EC meshes with fewer elements than this spread an element's directions over
+// warps (see dg_mhd_ec.cuh)
+constexpr long long kMhdSpreadElems = 4 * 152;
 
 struct MState {
   double rho, rr, v[3], p, B[3], b2, vb, pt, E;
@@ -170,11 +174,13 @@ __device__ __forceinline__ void mhd_ec_flux(const ECq& a, const ECq& b, double h
 
 #include "dg_mhd_weak.cuh"
 
+#include "dg_mhd_ec.cuh"
+
 // One thread per face node; the traces are read normal component first, so one
 // code body (direction 0) serves every direction. LLF and HLL in fixed point
 // (mhd_face_fixed), their FP64 form for the faces it declines.
 template <int N, int SF>
-__global__ void __launch_bounds__(256, SF == kMhdEc ? 1 : 2)
+__global__ void __launch_bounds__(256, 2)
     mhd_surface_kernel(const double* __restrict__ u, double* __restrict__ fs, Geom g,
                        unsigned* __restrict__ err) {
   constexpr int NP = N + 1, P = NP * NP * NP, NF = NP * NP;
@@ -194,7 +200,9 @@ __global__ void __launch_bounds__(256, SF == kMhdEc ? 1 : 2)
       cl[v] = u[(e * kMV + X[v]) * P + nl];
       cr[v] = u[(er * kMV + X[v]) * P + nr];
     }
-    if (SF == kMhdEc || !mhd_face_fixed(SF == kMhdHll, cl, cr, g.gamma, g.gm1, f)) {
+    const bool done = SF == kMhdEc ? mhd_ec_face_fixed(cl, cr, g, bad, f)
+                                   : mhd_face_fixed(SF == kMhdHll, cl, cr, g.gamma, g.gm1, f);
+    if (!done) {
       const MState sl = mhd_state(cl, g.gm1, bad), sr = mhd_state(cr, g.gm1, bad);
       if (SF == kMhdEc) {
         mhd_ec_flux<0>(ec_of(sl), ec_of(sr), 0.5 * g.gm1inv, f);
@@ -232,165 +240,6 @@ __global__ void __launch_bounds__(256, SF == kMhdEc ? 1 : 2)
     dst[8 * base] = 0.5 * (cl[5] + cr[5]);
   }
   if (bad) atomicOr(err, bad);
-}
-
-// ---- entropy-conservative flux differencing: one element per CTA ----
-// Per direction, one thread per (line, node pair) evaluates the EC flux once
-// for both nodes into shared memory (the flux is symmetric and the split-
-// form matrix has a zero diagonal); then one thread per node sums
-// Ds_ij f#(u_i, u_j) over its line, the Powell part Ds_ij (B_i + B_j)/2 of
-// -div B, and the lifting of F* and {B_n} at the line ends (Ds = -(2/h) Dt,
-// the split form of the oracle). Epilogue: the Powell term, the store or the
-// fused stage update.
-template <int N>
-struct MPairs {
-  static constexpr int NP = N + 1, P = NP * NP * NP, LINES = NP * NP;
-  static constexpr int NPAIRS = N * (N + 1) / 2;
-  static constexpr int WORK = LINES * NPAIRS;
-  static constexpr int MAXW = WORK > P ? WORK : P;
-  static constexpr int THREADS = MAXW < 512 ? ((MAXW + 31) / 32) * 32 : 512;
-  static constexpr int NQ = 12;  // the ECq slots: rho, beta, hv, hB, pm, qv2, qB2, hvB
-  static constexpr int SMEM = (NQ + kMV + 1) * P * (int)sizeof(double) +
-                              WORK * kMV * (int)sizeof(double);
-};
-
-template <int N>
-__device__ __forceinline__ ECq ec_load(const double (*sq)[(N + 1) * (N + 1) * (N + 1)], int n) {
-  ECq q;
-  q.rho = sq[0][n];
-  q.beta = sq[1][n];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    q.hv[k] = sq[2 + k][n];
-    q.hB[k] = sq[5 + k][n];
-  }
-  q.pm = sq[8][n];
-  q.qv2 = sq[9][n];
-  q.qB2 = sq[10][n];
-  q.hvB = sq[11][n];
-  return q;
-}
-
-template <int N, int DIR>
-__device__ __forceinline__ void mhd_ec_direction(const double (*sq)[(N + 1) * (N + 1) * (N + 1)],
-                                                 double (*sa)[(N + 1) * (N + 1) * (N + 1)],
-                                                 double* pf, const double (*sD)[N + 1][N + 1],
-                                                 long long e, const Geom& g,
-                                                 const Tables<double>& tb,
-                                                 const double* __restrict__ fs) {
-  using C = MPairs<N>;
-  constexpr int NP = C::NP, P = C::P, LINES = C::LINES, NPAIRS = C::NPAIRS;
-  for (int w = threadIdx.x; w < C::WORK; w += blockDim.x) {
-    const int l = w / NPAIRS;
-    int a, b;
-    pair_of<N>(w % NPAIRS, a, b);
-    double f[kMV];
-    mhd_ec_flux<DIR>(ec_load<N>(sq, line_node<3, N, DIR>(l, a)),
-                     ec_load<N>(sq, line_node<3, N, DIR>(l, b)), 0.5 * g.gm1inv, f);
-#pragma unroll
-    for (int v = 0; v < kMV; ++v) pf[v * C::WORK + w] = f[v];
-  }
-  __syncthreads();
-  for (int node = threadIdx.x; node < P; node += blockDim.x) {
-    int l, i;
-    line_of<N>(DIR, node, l, i);
-    // the line sums continue the running totals of the earlier directions
-    double acc[kMV], dn = sa[kMV][node];
-#pragma unroll
-    for (int v = 0; v < kMV; ++v) acc[v] = sa[v][node];
-    const double bi = sq[5 + DIR][node];  // B_n / 2
-    for (int j = 0; j < NP; ++j) {
-      if (j == i) continue;
-      const int p = j < i ? pair_index<N>(j, i) : pair_index<N>(i, j);
-      const double dij = sD[DIR][i][j];
-#pragma unroll
-      for (int v = 0; v < kMV; ++v) acc[v] = fma(dij, pf[v * C::WORK + l * NPAIRS + p], acc[v]);
-      dn = fma(dij, bi + sq[5 + DIR][line_node<3, N, DIR>(l, j)], dn);
-    }
-    if (i == N || i == 0) {
-      const long long ef = i == N ? e : neighbour(g, e, DIR, -1);
-      const double lift = i == N ? tb.liftR[DIR] : tb.liftL[DIR];
-      const long long base = g.nelem * LINES;
-      const double* src = fs + (long long)DIR * kMQ * base + ef * LINES + l;
-#pragma unroll
-      for (int v = 0; v < kMV; ++v) acc[v] = fma(lift, src[v * base], acc[v]);
-      dn = fma(lift, src[8 * base], dn);
-    }
-#pragma unroll
-    for (int v = 0; v < kMV; ++v) sa[v][node] = acc[v];
-    sa[kMV][node] = dn;
-  }
-  __syncthreads();
-}
-
-template <int N>
-__global__ void __launch_bounds__(MPairs<N>::THREADS)
-    mhd_volume_ec_kernel(double* u, double* __restrict__ du, const double* __restrict__ fs, Geom g,
-                         Tables<double> tb, int powell, unsigned* __restrict__ err, StageFuse fz) {
-  using C = MPairs<N>;
-  constexpr int NP = C::NP, P = C::P;
-  extern __shared__ __align__(16) unsigned char dg_smem[];
-  double(*sq)[P] = reinterpret_cast<double(*)[P]>(dg_smem);                              // [NQ][P]
-  double(*sa)[P] = reinterpret_cast<double(*)[P]>(dg_smem + sizeof(double) * C::NQ * P);  // [9][P]
-  double* pf = reinterpret_cast<double*>(dg_smem + sizeof(double) * (C::NQ + kMV + 1) * P);
-  __shared__ double sD[3][NP][NP];
-  for (int t = threadIdx.x; t < 3 * NP * NP; t += blockDim.x)
-    sD[t / (NP * NP)][(t / NP) % NP][t % NP] = tb.Ds[t / (NP * NP)][(t / NP) % NP][t % NP];
-  const long long e = blockIdx.x;
-  unsigned bad = 0;
-  for (int node = threadIdx.x; node < P; node += blockDim.x) {
-    double c[kMV];
-#pragma unroll
-    for (int v = 0; v < kMV; ++v) c[v] = u[(e * kMV + v) * P + node];
-    const ECq q = ec_of(mhd_state(c, g.gm1, bad));
-    sq[0][node] = q.rho;
-    sq[1][node] = q.beta;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      sq[2 + k][node] = q.hv[k];
-      sq[5 + k][node] = q.hB[k];
-    }
-    sq[8][node] = q.pm;
-    sq[9][node] = q.qv2;
-    sq[10][node] = q.qB2;
-    sq[11][node] = q.hvB;
-#pragma unroll
-    for (int v = 0; v <= kMV; ++v) sa[v][node] = 0.0;
-  }
-  if (bad) atomicOr(err, bad);
-  __syncthreads();
-  mhd_ec_direction<N, 0>(sq, sa, pf, sD, e, g, tb, fs);
-  mhd_ec_direction<N, 1>(sq, sa, pf, sD, e, g, tb, fs);
-  mhd_ec_direction<N, 2>(sq, sa, pf, sD, e, g, tb, fs);
-  const double dtv = fz.k ? *fz.dt : 0.0;
-  double* const uo = fz.u_out ? fz.u_out : u;
-  for (int node = threadIdx.x; node < P; node += blockDim.x) {
-    double acc[kMV];
-#pragma unroll
-    for (int v = 0; v < kMV; ++v) acc[v] = sa[v][node];
-    if (powell) {
-      // Phi = (0, B, v.B, v) from the halved slots: 2 x (hB, hvB, hv)
-      const double dn2 = 2.0 * sa[kMV][node];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        acc[1 + k] = fma(sq[5 + k][node], dn2, acc[1 + k]);
-        acc[5 + k] = fma(sq[2 + k][node], dn2, acc[5 + k]);
-      }
-      acc[4] = fma(sq[11][node], dn2, acc[4]);
-    }
-#pragma unroll
-    for (int v = 0; v < kMV; ++v) {
-      const long long i = (e * kMV + v) * P + node;
-      if (fz.k) {
-        double kk = dtv * acc[v];
-        if (fz.a != 0.0) kk = fma(fz.a, fz.k[i], kk);
-        fz.k[i] = kk;
-        uo[i] = u[i] + fz.b * kk;
-      } else {
-        du[i] = acc[v];
-      }
-    }
-  }
 }
 
 // upper bounds of a node's wave speeds |v_k| + c_f,k in FP32 (see speed_bound
@@ -494,6 +343,24 @@ __global__ void mhd_speed_kernel(const double* __restrict__ u, Geom g, int P, do
 // |g|, or EC), the Powell divergence as (1/J) times the split-form sums of
 // g . (B_i + B_m)/2 and {B} . g, du = (1/J) (...) with the unscaled
 // split-form table Ds = -Dt and liftR = -1/w_N, liftL = 1/w_0.
+
+// the staged EC quantities of node n: rho, beta, hv, hB, pm, qv2, qB2, hvB
+template <int N>
+__device__ __forceinline__ ECq ec_load(const double (*sq)[(N + 1) * (N + 1) * (N + 1)], int n) {
+  ECq q;
+  q.rho = sq[0][n];
+  q.beta = sq[1][n];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    q.hv[k] = sq[2 + k][n];
+    q.hB[k] = sq[5 + k][n];
+  }
+  q.pm = sq[8][n];
+  q.qv2 = sq[9][n];
+  q.qB2 = sq[10][n];
+  q.hvB = sq[11][n];
+  return q;
+}
 
 // node quantities of the directional physical flux
 struct CMq {
@@ -934,19 +801,21 @@ cudaError_t mhd_volume_epb(const double* u, double* du, const double* fs, const 
   return cudaGetLastError();
 }
 
-template <int N>
+template <int N, int EPB, bool SPREAD>
 cudaError_t mhd_volume_ec(const double* u, double* du, const double* fs, const Geom& g,
                           const Tables<double>& tdt, int powell, unsigned* err, cudaStream_t st,
                           const StageFuse& fz) {
-  using C = MPairs<N>;
-  auto kern = mhd_volume_ec_kernel<N>;
-  if (C::SMEM > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e != cudaSuccess) return e;
-  }
-  kern<<<(unsigned)g.nelem, C::THREADS, C::SMEM, st>>>(const_cast<double*>(u), du, fs, g, tdt,
-                                                        powell, err, fz);
+  using L = MELaunch<N>;
+  constexpr int SMEM = SPREAD ? L::ELEM_SPREAD : EPB * L::ELEM;
+  auto kern = mhd_volume_ec_fx_kernel<N, EPB, SPREAD>;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM)) !=
+          cudaSuccess ||
+      (e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                (int)cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
+    return e;
+  kern<<<(unsigned)((g.nelem + EPB - 1) / EPB), (SPREAD ? 3 : 1) * L::threads(EPB), SMEM, st>>>(
+      const_cast<double*>(u), du, fs, g, tdt, powell, err, fz);
   return cudaGetLastError();
 }
 
@@ -969,7 +838,15 @@ cudaError_t mhd_rhs_n(const double* u, double* du, double* fs, const Geom& g,
       mhd_surface_kernel<N, kMhdLlf><<<dim3((unsigned)blocks, 3), threads, 0, st>>>(u, fs, g, err);
   }
   if (!(parts & 2)) return cudaGetLastError();
-  if (vf == 1) return mhd_volume_ec<N>(u, du, fs, g, tdt, powell, err, st, fz);
+  if (vf == 1) {
+    // fewer elements than a few per SM: the directions side by side
+    constexpr int EPB = MELaunch<N>::EPB;
+    if (g.nelem < kMhdSpreadElems)
+      return mhd_volume_ec<N, 1, true>(u, du, fs, g, tdt, powell, err, st, fz);
+    if (EPB > 1 && g.nelem < 2LL * 152 * EPB)
+      return mhd_volume_ec<N, 1, false>(u, du, fs, g, tdt, powell, err, st, fz);
+    return mhd_volume_ec<N, EPB, false>(u, du, fs, g, tdt, powell, err, st, fz);
+  }
   constexpr int EPB = MLaunch<N>::EPB;
   if (EPB > 1 && g.nelem < 2LL * 152 * EPB)
     return mhd_volume_epb<N, 1>(u, du, fs, g, tb, powell, err, st, fz);

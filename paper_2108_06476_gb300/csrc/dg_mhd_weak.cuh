@@ -10,7 +10,8 @@
 // values, non-positive densities or densities spread over more than 2^6 take
 // the same steps in FP64.
 //
-// Included by dg_mhd.cu. 64^3 N = 3, rhs only: 6.34 ms in FP64.
+// Included by dg_mhd.cu. 48^3 N = 3, rhs only: 2.68 ms in FP64, 0.98 here; HLL
+// faces 1.81 and 0.57 ms, LLF 1.55 and 0.51.
 #pragma once
 
 // |m_k| < 2^em, |v_k| < 2^ev, |B_k| < 2^eb, energies below 2^(ee - 1), 1/rho < 2^e1

@@ -275,3 +275,47 @@ def test_weak_form_against_the_oracle(d, N, n, kind):
     for e in elems:
         err = np.linalg.norm(got[e] - ref[e]) / np.linalg.norm(ref[e])
         assert err <= 1e-12, (kind, int(e), err)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,n", [(1, (3, 4, 5)), (2, (3, 2, 4)), (3, (3, 2, 3)), (3, (10, 9, 8)),
+                                 (4, (2, 3, 2)), (4, (9, 10, 8)), (5, (3, 2, 2)), (6, (2, 2, 2)),
+                                 (7, (2, 1, 2))])
+@pytest.mark.parametrize("vf,sf", [("central", "hll"), ("central", "llf"), ("ec", "ec")])
+@pytest.mark.parametrize("kind", ["random", "nofield", "strong", "still", "fast", "mixed", "units"])
+def test_mhd_rhs_inside_and_outside_the_accepted_range(N, n, vf, sf, kind):
+    torch = _gpu()
+    import oracle
+    from paper_2108_06476_gb300 import Mesh, workloads as W
+    oracle.build()
+    rng = np.random.default_rng([N, 8])
+    ne, P = int(np.prod(n)), (N + 1) ** 3
+    rho = np.exp(rng.uniform(-0.6, 0.6, (ne, P)))
+    p = 2.0 * np.exp(rng.uniform(-0.6, 0.6, (ne, P)))
+    v = rng.uniform(-0.5, 0.5, (3, ne, P))
+    B = rng.uniform(-1, 1, (3, ne, P))
+    if kind == "nofield":
+        B *= 0.0
+    if kind == "strong":
+        B *= 10.0
+    if kind == "still":
+        v *= 0.0
+    if kind == "fast":
+        v[0] += 8.0
+    if kind == "mixed":  # every third element beyond the accepted ratio
+        rho[::3, 0] = 1e4
+        p[1::3, P - 1] = 5e3
+    if kind == "units":
+        rho, p, v, B = rho * 1e-20, p * 1e-8, v * 1e6, B * 1e-4
+    E = p / (5.0 / 3.0 - 1.0) + 0.5 * rho * (v ** 2).sum(0) + 0.5 * (B ** 2).sum(0)
+    u = np.ascontiguousarray(np.stack([rho, *(rho * v), E, *B], axis=1).reshape(-1))
+    m = Mesh(3, N, n, equations="mhd", volume_flux=vf, surface_flux=sf)
+    got = m.rhs(torch.from_numpy(u).cuda()).cpu().numpy().reshape(ne, 8, P)
+    assert m.check() == 0
+    elems = np.unique(np.linspace(0, ne - 1, 30).astype(np.int64))
+    ref = oracle.mhd_rhs(N, n, W.box(3), u, sflux=sf, vflux=vf, elems=elems).reshape(ne, 8, P)
+    # "strong" and "fast" lose digits of p in E - m.v/2 - |B|^2/2 on either side
+    bar = 1e-12 * (20.0 if kind in ("strong", "fast") else 1.0)
+    for e in elems:
+        err = np.linalg.norm(got[e] - ref[e]) / np.linalg.norm(ref[e])
+        assert err <= bar, (kind, int(e), err)

@@ -54,6 +54,37 @@ cudaError_t volume_n(double* u, double* du, const double* fs, const double* Ja,
   return volume_epb<N, VF, L::EPB>(u, du, fs, Ja, invJ, X, g, tb, err, st, fz, src);
 }
 
+template <int N, int EPB, bool SPREAD>
+cudaError_t volume_fx(double* u, double* du, const double* fs, const double* Ja,
+                      const double* invJ, const double* X, const Geom& g, const CTables& tb,
+                      unsigned* err, cudaStream_t st, const StageFuse& fz, const SourceArgs& src) {
+  using L = CFxLaunch<N>;
+  constexpr int SMEM = SPREAD ? L::ELEM_SPREAD : EPB * L::ELEM;
+  cudaError_t e;
+  if ((e = allow_smem(curved_volume_fx_kernel<N, EPB, SPREAD>, SMEM)) != cudaSuccess ||
+      (e = prefer_shared(curved_volume_fx_kernel<N, EPB, SPREAD>)) != cudaSuccess)
+    return e;
+  curved_volume_fx_kernel<N, EPB, SPREAD>
+      <<<(unsigned)((g.nelem + EPB - 1) / EPB), (SPREAD ? 3 : 1) * L::threads(EPB), SMEM, st>>>(
+          u, du, fs, Ja, invJ, X, g, tb, err, fz, src);
+  return cudaGetLastError();
+}
+
+// Ranocha's flux: the directions on warps of their own below a few elements
+// per SM
+template <int N>
+cudaError_t volume_fx_n(double* u, double* du, const double* fs, const double* Ja,
+                        const double* invJ, const double* X, const Geom& g, const CTables& tb,
+                        unsigned* err, cudaStream_t st, const StageFuse& fz,
+                        const SourceArgs& src) {
+  constexpr int EPB = CFxLaunch<N>::EPB;
+  if (g.nelem < kPairParallelElems)
+    return volume_fx<N, 1, true>(u, du, fs, Ja, invJ, X, g, tb, err, st, fz, src);
+  if (EPB > 1 && g.nelem < 2LL * 152 * EPB)
+    return volume_fx<N, 1, false>(u, du, fs, Ja, invJ, X, g, tb, err, st, fz, src);
+  return volume_fx<N, EPB, false>(u, du, fs, Ja, invJ, X, g, tb, err, st, fz, src);
+}
+
 template <int N>
 cudaError_t rhs_n(double* u, double* du, double* fs, const double* Ja, const double* invJ,
                   const double* X, const Geom& g, const CTables& tb, int vf, int sf,
@@ -71,7 +102,7 @@ cudaError_t rhs_n(double* u, double* du, double* fs, const double* Ja, const dou
     if (e != cudaSuccess) return e;
   }
   if (!(parts & 2)) return cudaSuccess;
-  if (vf == kVRanocha) return volume_n<N, kVRanocha>(u, du, fs, Ja, invJ, X, g, tb, err, st, fz, src);
+  if (vf == kVRanocha) return volume_fx_n<N>(u, du, fs, Ja, invJ, X, g, tb, err, st, fz, src);
   if (vf == kVChandrashekar)
     return volume_n<N, kVChandrashekar>(u, du, fs, Ja, invJ, X, g, tb, err, st, fz, src);
   return volume_n<N, kVCentral>(u, du, fs, Ja, invJ, X, g, tb, err, st, fz, src);

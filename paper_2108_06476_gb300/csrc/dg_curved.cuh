@@ -241,6 +241,41 @@ __device__ __forceinline__ void curved_surface_flux(int sf, const double* cl, co
   }
 }
 
+// pair (a, b), a < b, of index p in the order (0,1), (0,2), ..., (0,N), (1,2), ...
+template <int N>
+__device__ __forceinline__ void pair_of(int p, int& a, int& b) {
+  a = 0;
+  while (p >= N - a) {
+    p -= N - a;
+    ++a;
+  }
+  b = a + 1 + p;
+}
+template <int N>
+__device__ __forceinline__ int pair_index(int a, int b) {  // a < b
+  return a * N - a * (a - 1) / 2 + (b - a - 1);
+}
+
+// line l and position i along direction r of a node (inverse of line_node)
+template <int N>
+__device__ __forceinline__ void line_of(int r, int node, int& l, int& i) {
+  constexpr int NP = N + 1;
+  if (r == 0) {
+    l = node / NP;
+    i = node % NP;
+  } else if (r == 1) {
+    i = (node / NP) % NP;
+    l = node % NP + NP * (node / (NP * NP));
+  } else {
+    i = node / (NP * NP);
+    l = node % (NP * NP);
+  }
+}
+
+}  // namespace dg
+#include "dg_curved_fx.cuh"
+namespace dg {
+
 // face-parallel: blockIdx.y = reference direction r; fs[r][v][e_left][l]
 template <int N>
 __global__ void curved_surface_kernel(const double* __restrict__ u, double* __restrict__ fs,
@@ -262,13 +297,16 @@ __global__ void curved_surface_kernel(const double* __restrict__ u, double* __re
 #pragma unroll
     for (int k = 0; k < 3; ++k) gv[k] = Ja[(((long long)e * 3 + r) * 3 + k) * P + nl];
     double f[NV];
-    curved_surface_flux(sf, cl, cr, gv, g.gamma, g.gm1, f);
+    if (sf != kSRanocha || !curved_face_fixed(cl, cr, gv, g, f))
+      curved_surface_flux(sf, cl, cr, gv, g.gamma, g.gm1, f);
 #pragma unroll
     for (int v = 0; v < NV; ++v) fs[((long long)r * NV + v) * total + t] = f[v];
   }
 }
 
-// ---- volume: flux differencing, lifting, 1/J, source, optional stage update ----
+// ---- volume (Chandrashekar's and the central flux; Ranocha's:
+// dg_curved_fx.cuh): flux differencing, lifting, 1/J, source, optional stage
+// update ----
 template <int N>
 struct CLaunch {
   static constexpr int NP = N + 1, P = NP * NP * NP, LINES = NP * NP;
@@ -318,8 +356,7 @@ __device__ __forceinline__ void curved_direction(int r, double (*sp)[9][(N + 1) 
       double gv[3], f[NV];
 #pragma unroll
       for (int k = 0; k < 3; ++k) gv[k] = hg[a][k] + hg[b][k];
-      if (VF == kVRanocha) ranocha_contra(q[a], q[b], gv, f);
-      else generic_contra<VF>(q[a], q[b], gv, gm1inv, f);
+      generic_contra<VF>(q[a], q[b], gv, gm1inv, f);
       const double dab = tb.Ds[a][b], dba = tb.Ds[b][a];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
@@ -446,37 +483,6 @@ struct CPairs {
   static constexpr int SMEM = (9 + 3 + 5) * P * (int)sizeof(double) + WORK * 5 * (int)sizeof(double);
 };
 
-// pair (a, b), a < b, of index p in the order (0,1), (0,2), ..., (0,N), (1,2), ...
-template <int N>
-__device__ __forceinline__ void pair_of(int p, int& a, int& b) {
-  a = 0;
-  while (p >= N - a) {
-    p -= N - a;
-    ++a;
-  }
-  b = a + 1 + p;
-}
-template <int N>
-__device__ __forceinline__ int pair_index(int a, int b) {  // a < b
-  return a * N - a * (a - 1) / 2 + (b - a - 1);
-}
-
-// line l and position i along direction r of a node (inverse of line_node)
-template <int N>
-__device__ __forceinline__ void line_of(int r, int node, int& l, int& i) {
-  constexpr int NP = N + 1;
-  if (r == 0) {
-    l = node / NP;
-    i = node % NP;
-  } else if (r == 1) {
-    i = (node / NP) % NP;
-    l = node % NP + NP * (node / (NP * NP));
-  } else {
-    i = node / (NP * NP);
-    l = node % (NP * NP);
-  }
-}
-
 template <int N, int VF>
 __global__ void __launch_bounds__(CPairs<N>::THREADS)
     curved_volume_pp_kernel(double* u, double* __restrict__ du, const double* __restrict__ fs,
@@ -541,8 +547,7 @@ __global__ void __launch_bounds__(CPairs<N>::THREADS)
         qb.hv[k] = sp[6 + k][nb];
         gv[k] = sg[k][na] + sg[k][nb];
       }
-      if (VF == kVRanocha) ranocha_contra(qa, qb, gv, f);
-      else generic_contra<VF>(qa, qb, gv, g.gm1inv, f);
+      generic_contra<VF>(qa, qb, gv, g.gm1inv, f);
 #pragma unroll
       for (int v = 0; v < NV; ++v) sf[w * NV + v] = f[v];
     }

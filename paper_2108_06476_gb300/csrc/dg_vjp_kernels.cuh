@@ -6,9 +6,11 @@
 // (d f#/d u_a)^T g to ubar_a and (d f#/d u_b)^T g to ubar_b. A face adds
 // liftR F* to du at node N of its left element and liftL F* at node 0 of its
 // right element: g = liftR w_L + liftL w_R, ubar_L += (dF*/du_L)^T g,
-// ubar_R += (dF*/du_R)^T g. The flux Jacobians come from forward-mode dual
-// numbers seeded with the 2 (d+2) conserved components of the two states; the
-// two-point fluxes are recomputed, nothing is stored from the forward pass.
+// ubar_R += (dF*/du_R)^T g. In general the flux Jacobians come from
+// forward-mode dual numbers seeded with the 2 (d+2) conserved components of
+// the two states; FP64 meshes have Ranocha's volume flux (vjp_volume_fx_kernel)
+// and the LLF surface flux (llf_rev) in reverse mode. The two-point fluxes are
+// recomputed, nothing is stored from the forward pass.
 //
 //  vjp_face_kernel: one thread per face node; writes the two adjoint
 //    contributions of every face to fb[dir][side][v][e_left][l].
@@ -69,7 +71,8 @@ __device__ __forceinline__ void pair_vjp(int vf, int sf, bool surface, const R* 
   }
 }
 
-// Reverse mode for Ranocha's volume flux, on primitive variables: the adjoint
+// Reverse mode for Ranocha's volume flux, on primitive variables (elements
+// outside the limits of dg_vjp_fixed.cuh): the adjoint
 // of one two-point flux f#(q_a, q_b) (q = (rho, v normal-first, p)) for the
 // cotangent g (normal-first), added to ba and bb (adjoints of q_a, q_b). The
 // flux is flux_ranocha's:
@@ -142,99 +145,68 @@ __device__ __forceinline__ void ranocha_pair_rev(const R* qa, const R* qb, const
 
 // Reverse mode for the LLF surface flux F* = (f(u_L) + f(u_R))/2 - lam (u_R -
 // u_L)/2, lam = max(|v_n,L|, |v_n,R|) + max(c_L, c_R), in normal-first
-// conserved variables: gl = J(u_L)^T g / 2 + lam g / 2 - (g . (u_R - u_L))
-// dlam/du_L / 2 and gr likewise, with the Euler flux Jacobian's transpose
-// written out (H = (E + p)/rho):
-//   (J^T g)_rho = g_1 (gm1 |v|^2/2 - v_n^2) - sum_t g_t v_t v_n + g_E v_n (gm1 |v|^2/2 - H)
-//   (J^T g)_mn  = g_0 + g_1 (2 - gm1) v_n + sum_t g_t v_t + g_E (H - gm1 v_n^2)
-//   (J^T g)_mt  = -g_1 gm1 v_t + g_t v_n - g_E gm1 v_t v_n
-//   (J^T g)_E   = g_1 gm1 + g_E gamma v_n
-// and the derivative of lam taken along its maxima (ties: the left state;
-// d|x|/dx = +1 at 0), as the dual-number evaluation of the same flux does.
-template <typename R, int D>
-__device__ __forceinline__ void llf_side_rev(const R* c, const R* g, R gamma, R gm1, R half_lam,
-                                             R* out) {
-  constexpr int NV = D + 2;
-  const R rho = c[0], ir = R(1) / rho;
-  R v[D], v2 = R(0);
+// conserved variables. With f(u) = v_n u + p (0, n, v_n), a side contributes
+//   g (v_n +- lam)/2 + cv d(v_n)/du + cp dp/du,
+//   cv = (g.u + g_E p)/2 + s sign(v_n),    d(v_n)/du = (-v_n, 1, 0, 0)/rho,
+//   cp = (g_1 + g_E v_n)/2 + s gamma/(2 c rho),
+//   dp/du = (gamma-1) (|v|^2/2, -v, 1),
+// and -s p gamma/(2 c rho^2) to rho, s = -g.(u_R - u_L)/2 the cotangent of
+// lam, its terms on the side where the maximum is (ties: the left state;
+// d|x|/dx = +1 at 0), as the dual-number evaluation of the same flux takes it.
+// About 110 FP64 instructions per face node, reciprocals and roots once per
+// side; with IEEE divisions and both sides' Jacobians written out about 250.
+template <int D>
+struct LlfSide {
+  double ir, v[D], v2, p, c;
+};
+template <int D>
+__device__ __forceinline__ LlfSide<D> llf_side(const double* u, double gamma, double gm1) {
+  LlfSide<D> q;
+  q.ir = rcp(u[0]);
+  q.v2 = 0.0;
 #pragma unroll
   for (int k = 0; k < D; ++k) {
-    v[k] = c[1 + k] * ir;
-    v2 += v[k] * v[k];
+    q.v[k] = u[1 + k] * q.ir;
+    q.v2 = ::fma(q.v[k], q.v[k], q.v2);
   }
-  const R p = gm1 * (c[NV - 1] - R(0.5) * rho * v2);
-  const R H = (c[NV - 1] + p) * ir, vn = v[0], k2 = R(0.5) * gm1 * v2;
-  R gtv = R(0), gtvs = R(0);  // sum_t g_t v_t
+  q.p = gm1 * ::fma(-half(u[0]), q.v2, u[D + 1]);
+  q.c = sqrt_pos(gamma * q.p * q.ir);
+  return q;
+}
+template <int D>
+__device__ __forceinline__ void llf_side_rev(const LlfSide<D>& q, const double* u, const double* g,
+                                             double gm1, double half_lam, double sv, double sa,
+                                             double* out) {
+  double gu = g[D + 1] * q.p;
 #pragma unroll
-  for (int k = 1; k < D; ++k) gtv += g[1 + k] * v[k];
-  gtvs = gtv;
-  out[0] = R(0.5) * (g[1] * (k2 - vn * vn) - gtvs * vn + g[NV - 1] * vn * (k2 - H)) + half_lam * g[0];
-  out[1] = R(0.5) * (g[0] + g[1] * (R(2) - gm1) * vn + gtv + g[NV - 1] * (H - gm1 * vn * vn)) +
-           half_lam * g[1];
+  for (int v = 0; v < D + 2; ++v) gu = ::fma(g[v], u[v], gu);
+  const double k = half(q.v[0]) + half_lam;
+  const double cv = ::fma(half(gu), q.ir, sv * q.ir);
+  const double cp = gm1 * ::fma(half(g[D + 1]), q.v[0], half(g[1]) + sa);
+  out[0] = ::fma(k, g[0], ::fma(-cv, q.v[0], ::fma(cp, half(q.v2), -(sa * q.p * q.ir))));
+  out[1] = ::fma(k, g[1], ::fma(-cp, q.v[0], cv));
 #pragma unroll
-  for (int k = 1; k < D; ++k)
-    out[1 + k] = R(0.5) * (-g[1] * gm1 * v[k] + g[1 + k] * vn - g[NV - 1] * gm1 * v[k] * vn) +
-                 half_lam * g[1 + k];
-  out[NV - 1] = R(0.5) * (g[1] * gm1 + g[NV - 1] * gamma * vn) + half_lam * g[NV - 1];
+  for (int t = 1; t < D; ++t) out[1 + t] = ::fma(k, g[1 + t], -(cp * q.v[t]));
+  out[D + 1] = ::fma(k, g[D + 1], cp);
+}
+template <int D>
+__device__ __forceinline__ void llf_rev(const double* cl, const double* cr, const double* g,
+                                        double gamma, double gm1, double* gl, double* gr) {
+  const LlfSide<D> a = llf_side<D>(cl, gamma, gm1), b = llf_side<D>(cr, gamma, gm1);
+  const bool vleft = ::fabs(a.v[0]) >= ::fabs(b.v[0]), cleft = a.c >= b.c;
+  const double vm = vleft ? a.v[0] : b.v[0], cm = cleft ? a.c : b.c;
+  const double hl = half(::fabs(vm) + cm);
+  double jump = 0.0;
+#pragma unroll
+  for (int v = 0; v < D + 2; ++v) jump = ::fma(g[v], cr[v] - cl[v], jump);
+  const double s = -half(jump), sv = vm < 0.0 ? -s : s;
+  const double sa = s * half(gamma) * (cleft ? a.ir : b.ir) * rcp(cm);
+  llf_side_rev<D>(a, cl, g, gm1, hl, vleft ? sv : 0.0, cleft ? sa : 0.0, gl);
+  llf_side_rev<D>(b, cr, g, gm1, -hl, vleft ? 0.0 : sv, cleft ? 0.0 : sa, gr);
 }
 
-// d|v_n|/du and dc/du of one state (normal-first conserved), scaled by s
-template <typename R, int D>
-__device__ __forceinline__ void lam_terms(const R* c, R gamma, R gm1, bool take_v, bool take_c,
-                                          R s, R* out) {
-  constexpr int NV = D + 2;
-  const R rho = c[0], ir = R(1) / rho;
-  R v[D], v2 = R(0);
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    v[k] = c[1 + k] * ir;
-    v2 += v[k] * v[k];
-  }
-  if (take_v) {
-    const R sg = v[0] < R(0) ? R(-1) : R(1);
-    out[0] += s * sg * (-v[0] * ir);
-    out[1] += s * sg * ir;
-  }
-  if (take_c) {
-    const R p = gm1 * (c[NV - 1] - R(0.5) * rho * v2);
-    const R cs = ::sqrt(gamma * p * ir);
-    const R a = gamma / (R(2) * cs * rho);
-    out[0] += s * a * (gm1 * R(0.5) * v2 - p * ir);
-#pragma unroll
-    for (int k = 0; k < D; ++k) out[1 + k] += s * a * (-gm1 * v[k]);
-    out[NV - 1] += s * a * gm1;
-  }
-}
-
-template <typename R, int D>
-__device__ __forceinline__ void llf_rev(const R* cl, const R* cr, const R* g, R gamma, R gm1,
-                                        R* gl, R* gr) {
-  constexpr int NV = D + 2;
-  // lam from the two states, as the flux computes it
-  const R irl = R(1) / cl[0], irr = R(1) / cr[0];
-  R v2l = R(0), v2r = R(0);
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    v2l += (cl[1 + k] * irl) * (cl[1 + k] * irl);
-    v2r += (cr[1 + k] * irr) * (cr[1 + k] * irr);
-  }
-  const R vnl = cl[1] * irl, vnr = cr[1] * irr;
-  const R pl = gm1 * (cl[NV - 1] - R(0.5) * cl[0] * v2l);
-  const R pr = gm1 * (cr[NV - 1] - R(0.5) * cr[0] * v2r);
-  const R csl = ::sqrt(gamma * pl * irl), csr = ::sqrt(gamma * pr * irr);
-  const bool vleft = ::fabs(vnl) >= ::fabs(vnr), cleft = csl >= csr;
-  const R lam = (vleft ? ::fabs(vnl) : ::fabs(vnr)) + (cleft ? csl : csr);
-  llf_side_rev<R, D>(cl, g, gamma, gm1, R(0.5) * lam, gl);
-  llf_side_rev<R, D>(cr, g, gamma, gm1, R(-0.5) * lam, gr);
-  R jump = R(0);
-#pragma unroll
-  for (int v = 0; v < NV; ++v) jump += g[v] * (cr[v] - cl[v]);
-  const R s = R(-0.5) * jump;
-  lam_terms<R, D>(cl, gamma, gm1, vleft, cleft, s, gl);
-  lam_terms<R, D>(cr, gamma, gm1, !vleft, !cleft, s, gr);
-}
-
-template <int D, int N, typename R, int dir>
+// FORWARD: dual numbers, else the LLF flux of FP64 meshes in reverse mode
+template <int D, int N, typename R, int dir, bool FORWARD>
 __device__ __forceinline__ void vjp_face_body(const double* __restrict__ u,
                                               const double* __restrict__ w,
                                               double* __restrict__ fb, const Geom& g,
@@ -257,8 +229,8 @@ __device__ __forceinline__ void vjp_face_body(const double* __restrict__ u,
       gg[c] = R(tb.liftR[dir] * w[((long long)e * NV + v) * P + nl] +
                 tb.liftL[dir] * w[((long long)er * NV + v) * P + nr]);
     }
-    if (sf == kSLLF && sizeof(R) == 8)
-      llf_rev<R, D>(ul, ur, gg, R(g.gamma), R(g.gm1), gl, gr);
+    if constexpr (!FORWARD)
+      llf_rev<D>(ul, ur, gg, g.gamma, g.gm1, gl, gr);
     else
       pair_vjp<R, D>(0, sf, true, ul, ur, gg, R(g.gamma), R(g.gm1), R(g.gm1inv), gl, gr);
 #pragma unroll
@@ -270,12 +242,12 @@ __device__ __forceinline__ void vjp_face_body(const double* __restrict__ u,
   }
 }
 
-template <int D, int N, typename R>
+template <int D, int N, typename R, bool FORWARD>
 __global__ void vjp_face_kernel(const double* __restrict__ u, const double* __restrict__ w,
                                 double* __restrict__ fb, Geom g, Tables<double> tb, int sf) {
-  if (blockIdx.y == 0) vjp_face_body<D, N, R, 0>(u, w, fb, g, tb, sf);
-  else if (blockIdx.y == 1) vjp_face_body<D, N, R, 1>(u, w, fb, g, tb, sf);
-  else vjp_face_body<D, N, R, (D == 3 ? 2 : 1)>(u, w, fb, g, tb, sf);
+  if (blockIdx.y == 0) vjp_face_body<D, N, R, 0, FORWARD>(u, w, fb, g, tb, sf);
+  else if (blockIdx.y == 1) vjp_face_body<D, N, R, 1, FORWARD>(u, w, fb, g, tb, sf);
+  else vjp_face_body<D, N, R, (D == 3 ? 2 : 1), FORWARD>(u, w, fb, g, tb, sf);
 }
 
 template <int D, int N, typename R, int EPB>
@@ -362,123 +334,13 @@ __global__ void __launch_bounds__(EPB* Shape<D, N>::LINES)
   }
 }
 
-// Ranocha's volume flux in reverse mode: the primitives of every node once
-// per element in shared memory, the pair adjoints (ranocha_pair_rev)
-// accumulated as adjoints of the primitives, and in the epilogue one
-// conversion per node to the adjoint of the conserved variables,
-//   ubar_rho = rhobar - sum_k vbar_k v_k / rho + pbar (gamma-1) |v|^2 / 2,
-//   ubar_m_k = vbar_k / rho - pbar (gamma-1) v_k,   ubar_E = pbar (gamma-1),
-// plus the face contributions.
-template <int D, int N, typename R, int EPB>
-__global__ void __launch_bounds__(EPB* Shape<D, N>::LINES)
-    vjp_volume_rev_kernel(const double* __restrict__ u, const double* __restrict__ w,
-                          double* __restrict__ ubar, const double* __restrict__ fb, Geom g,
-                          Tables<double> tb) {
-  using S = Shape<D, N>;
-  constexpr int NP = S::NP, P = S::P, NV = S::NV, LINES = S::LINES;
-  extern __shared__ __align__(16) unsigned char dg_smem[];
-  double(*sq)[NV][P] = reinterpret_cast<double(*)[NV][P]>(dg_smem);  // rho, v, p
-  double(*sw)[NV][P] = sq + EPB;
-  double(*sb)[NV][P] = sw + EPB;  // adjoints of rho, v, p
-  __shared__ int s_left[EPB][3];
-  const int e0 = blockIdx.x * EPB;
-  const int nelem = (int)g.nelem;
-  if (threadIdx.x < EPB && e0 + (int)threadIdx.x < nelem) {
-    const int el = threadIdx.x, e = e0 + el;
-    const int x = e % g.n[0], r = e / g.n[0], y = r % g.n[1], z = r / g.n[1];
-    s_left[el][0] = elem_index(g, x == 0 ? g.n[0] - 1 : x - 1, y, z);
-    s_left[el][1] = elem_index(g, x, y == 0 ? g.n[1] - 1 : y - 1, z);
-    s_left[el][2] = (D == 3) ? elem_index(g, x, y, z == 0 ? g.n[2] - 1 : z - 1) : 0;
-  }
-  for (int t = threadIdx.x; t < EPB * P; t += blockDim.x) {
-    const int el = t / P, node = t % P;
-    const int e = e0 + el;
-    if (e >= nelem) continue;
-    double c[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      c[v] = u[((long long)e * NV + v) * P + node];
-      sw[el][v][node] = w[((long long)e * NV + v) * P + node];
-      sb[el][v][node] = 0.0;
-    }
-    const Prim<double, D> q = cons2prim<double, D>(c, g.gm1);
-    sq[el][0][node] = q.rho;
-#pragma unroll
-    for (int k = 0; k < D; ++k) sq[el][1 + k][node] = q.v[k];
-    sq[el][D + 1][node] = q.p;
-  }
-  __syncthreads();
-  const int el = threadIdx.x / LINES, l = threadIdx.x % LINES;
-  const bool active = (e0 + el) < nelem;
-  const R gm1inv = R(g.gm1inv);
-#pragma unroll 1
-  for (int dir = 0; dir < D; ++dir) {
-    if (active) {
-#pragma unroll 1
-      for (int a = 0; a < NP; ++a) {
-        const int na = line_node_rt<D, N>(dir, l, a);
-#pragma unroll 1
-        for (int b = a + 1; b < NP; ++b) {
-          const int nb = line_node_rt<D, N>(dir, l, b);
-          const double dab = tb.Ds[dir][a][b], dba = tb.Ds[dir][b][a];
-          R qa[NV], qb[NV], gg[NV], ga[NV], gb[NV];
-#pragma unroll
-          for (int c = 0; c < NV; ++c) {
-            const int v = nf_index<D>(dir, c);
-            qa[c] = R(sq[el][v][na]);
-            qb[c] = R(sq[el][v][nb]);
-            gg[c] = R(dab * sw[el][v][na] + dba * sw[el][v][nb]);
-            ga[c] = R(0);
-            gb[c] = R(0);
-          }
-          ranocha_pair_rev<R, D>(qa, qb, gg, gm1inv, ga, gb);
-#pragma unroll
-          for (int c = 0; c < NV; ++c) {
-            const int v = nf_index<D>(dir, c);
-            sb[el][v][na] += (double)ga[c];
-            sb[el][v][nb] += (double)gb[c];
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-  const double gm1 = g.gm1;
-  for (int t = threadIdx.x; t < EPB * P; t += blockDim.x) {
-    const int ell = t / P, node = t % P;
-    const int e = e0 + ell;
-    if (e >= nelem) continue;
-    const double rho = sq[ell][0][node], pb = sb[ell][D + 1][node];
-    const double irho = 1.0 / rho;
-    double val[NV], v2 = 0.0, rb = sb[ell][0][node];
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-      const double vk = sq[ell][1 + k][node], vbk = sb[ell][1 + k][node];
-      v2 += vk * vk;
-      rb -= vbk * vk * irho;
-      val[1 + k] = vbk * irho - pb * gm1 * vk;
-    }
-    val[0] = rb + pb * gm1 * 0.5 * v2;
-    val[D + 1] = pb * gm1;
-    const int c[3] = {node % NP, (node / NP) % NP, node / (NP * NP)};
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      double acc = val[v];
-#pragma unroll
-      for (int dir = 0; dir < D; ++dir) {
-        const int lf = (D == 2) ? ((dir == 0) ? c[1] : c[0])
-                                : (dir == 0) ? (c[1] + NP * c[2])
-                                : (dir == 1) ? (c[0] + NP * c[2]) : (c[0] + NP * c[1]);
-        if (c[dir] == N) acc += fb[((long long)((dir * 2 + 0) * NV + v) * nelem + e) * LINES + lf];
-        if (c[dir] == 0)
-          acc += fb[((long long)((dir * 2 + 1) * NV + v) * nelem + s_left[ell][dir]) * LINES + lf];
-      }
-      ubar[((long long)e * NV + v) * P + node] = acc;
-    }
-  }
-}
+}  // namespace dg
 
-// elements per CTA of the VJP volume kernels (one thread per element line):
+#include "dg_vjp_fixed.cuh"
+
+namespace dg {
+
+// elements per CTA of the forward-mode volume kernel (one thread per element line):
 // about 64 threads, unless their warps would leave more than a tenth of the
 // lanes idle (a warp's FP64 instruction costs the same whatever its active
 // lanes); then the count of at most 256 threads and 96 KB of shared memory
@@ -509,15 +371,23 @@ cudaError_t launch_vjp_dn(const double* u, const double* w, double* ubar, double
     long long blocks = (total + 127) / 128;
     if (blocks > 152 * 16) blocks = 152 * 16;
     if (blocks < 1) blocks = 1;
-    vjp_face_kernel<D, N, R><<<dim3((unsigned)blocks, D), 128, 0, st>>>(u, w, fb, g, tb, sf);
+    const dim3 grid((unsigned)blocks, D);
+    if (sf == kSLLF && sizeof(R) == 8)
+      vjp_face_kernel<D, N, R, sizeof(R) != 8><<<grid, 128, 0, st>>>(u, w, fb, g, tb, sf);
+    else
+      vjp_face_kernel<D, N, R, true><<<grid, 128, 0, st>>>(u, w, fb, g, tb, sf);
   }
   const long long grid = (g.nelem + EPB - 1) / EPB;
   cudaError_t e;
-  if (vf == kVRanocha && sizeof(R) == 8) {
-    if ((e = allow_smem(vjp_volume_rev_kernel<D, N, R, EPB>, SM)) != cudaSuccess) return e;
-    vjp_volume_rev_kernel<D, N, R, EPB><<<(unsigned)grid, EPB * S::LINES, SM, st>>>(u, w, ubar,
-                                                                                  fb, g, tb);
-    return cudaGetLastError();
+  if constexpr (sizeof(R) == 8) {
+    if (vf == kVRanocha) {
+      using V = VjpFx<D, N>;
+      constexpr int SMX = V::EPB * V::ELEM;
+      if ((e = allow_smem(vjp_volume_fx_kernel<D, N>, SMX)) != cudaSuccess) return e;
+      vjp_volume_fx_kernel<D, N><<<(unsigned)((g.nelem + V::EPB - 1) / V::EPB),
+                                   V::threads(V::EPB), SMX, st>>>(u, w, ubar, fb, g, tb);
+      return cudaGetLastError();
+    }
   }
   if ((e = allow_smem(vjp_volume_kernel<D, N, R, EPB>, SM)) != cudaSuccess) return e;
   vjp_volume_kernel<D, N, R, EPB><<<(unsigned)grid, EPB * S::LINES, SM, st>>>(u, w, ubar, fb, g,

@@ -17,6 +17,10 @@
   (|D| < 4.18, a ratio of 2^6) as polynomials in z = (x - 8.75)/16; the
   coefficients are negated and stored in units of 2^-61.
 
+* TanhD*/SinhD*: the derivatives with respect to D of tanh(D/2)/(D/2) and
+  D/sinh(D), divided by D, as polynomials in the same variables; coefficient k
+  of x^k in units of 2^-(63 + 2k), far ones in 2^-61, all negated.
+
 Usage: python gen_fixed_tables.py > dg_fixed_tables.cuh
 """
 import mpmath as mp
@@ -36,6 +40,20 @@ def sinhc(x):
         return mp.mpf(1) / 6
     d = mp.sqrt(x)
     return (1 - d / mp.sinh(d)) / x
+
+
+def tanhd(x):  # -(d/dD tanh(D/2)/(D/2))/D
+    if x < mp.mpf(10) ** -20:
+        return mp.mpf(1) / 6
+    d = mp.sqrt(x)
+    return -(mp.sech(d / 2) ** 2 / d - 2 * mp.tanh(d / 2) / x) / d
+
+
+def sinhd(x):  # -(d/dD D/sinh(D))/D
+    if x < mp.mpf(10) ** -20:
+        return mp.mpf(1) / 3
+    d = mp.sqrt(x)
+    return -(1 / mp.sinh(d) - d * mp.cosh(d) / mp.sinh(d) ** 2) / d
 
 
 def fit(fun, a, n):
@@ -67,18 +85,22 @@ def emit(name, fun, a, n, off, narrow_from=None):
     print(f"#define DG_FX_{name}32 {{" + ", ".join(str(v) for v in s[narrow_from:]) + "}")
 
 
-def emit_far(name, fun, n):
+def emit_far(name, fun, n, times_x=True):
+    f0 = fun
+    if not times_x:
+        fun = lambda x: f0(x) / x if x else mp.mpf(0)  # noqa: E731
     a, h = mp.mpf("17.5"), mp.mpf("8.75")
     nodes = [a * (1 + mp.cos(mp.pi * (2 * k + 1) / (2 * n))) / 2 for k in range(n)]
     z = [(x - h) / 16 for x in nodes]
     V = mp.matrix([[y ** j for j in range(n)] for y in z])
     c = mp.lu_solve(V, mp.matrix([x * fun(x) for x in nodes]))
     e = max(abs(sum(c[j] * ((a * k / 400 - h) / 16) ** j for j in range(n))
-                - (a * k / 400) * fun(a * k / 400)) for k in range(401))
+                - (a * k / 400) * fun(a * k / 400)) for k in range(1, 401))
     q = [int(mp.nint(-c[k] * mp.mpf(2) ** 61)) for k in range(n)]
     assert sum(abs(v) * 0.547 ** k for k, v in enumerate(q)) < 2 ** 62.5
     print(f"// z = (x - 8.75)/16, {n} coefficients: largest error {float(e):.1e}")
-    print(f"constexpr int kFarN = {n};" if name == "TanhFar" else f"static_assert(kFarN == {n}, \"\");")
+    print(f"constexpr int kFarN = {n};" if name == "TanhFar"
+          else f'static_assert(kFarN == {n}, "");')
     print(f"#define DG_FX_{name} {{" + ", ".join(f"{v}LL" for v in q) + "}")
 
 
@@ -92,6 +114,12 @@ def main():
     emit("SinhMid", sinhc, "1", 11, 63)
     emit_far("TanhFar", tanhc, 32)
     emit_far("SinhFar", sinhc, 32)
+    emit("TanhDShort", tanhd, "0.0625", 6, 61, 3)
+    emit("SinhDShort", sinhd, "0.0625", 6, 61, 3)
+    emit("TanhDMid", tanhd, "1", 11, 61)
+    emit("SinhDMid", sinhd, "1", 11, 61)
+    emit_far("TanhDFar", tanhd, 32, False)
+    emit_far("SinhDFar", sinhd, 32, False)
     print("struct __align__(16) LogEntry {\n  long long l;\n  int r, pad;\n};")
     rows, zmax = [], 0.0
     for i in range(128):

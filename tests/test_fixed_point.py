@@ -319,3 +319,54 @@ def test_mhd_rhs_inside_and_outside_the_accepted_range(N, n, vf, sf, kind):
     for e in elems:
         err = np.linalg.norm(got[e] - ref[e]) / np.linalg.norm(ref[e])
         assert err <= bar, (kind, int(e), err)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,N,n", [(2, 1, (3, 4)), (2, 2, (5, 3)), (2, 7, (3, 3)), (3, 1, (3, 2, 4)),
+                                   (3, 2, (2, 3, 4)), (3, 3, (3, 4, 2)), (3, 4, (3, 2, 3)),
+                                   (3, 5, (2, 3, 1)), (3, 6, (2, 1, 2)), (3, 7, (2, 2, 1))])
+@pytest.mark.parametrize("kind", ["mild", "wide", "far", "mixed", "fast", "still", "units", "mass",
+                                  "momentum", "energy"])
+def test_vjp_inside_and_outside_the_accepted_range(d, N, n, kind):
+    # <w, J v> from the oracle's exact JVP against <J^T w, v>, v supported on
+    # one element at a time: every element's block of J^T w meets the bar,
+    # relative to the sum of the products' magnitudes (2^-53 times some
+    # hundreds of operations per entry stays below 1e-12)
+    torch = _gpu()
+    import oracle
+    from paper_2108_06476_gb300 import Mesh, workloads as W
+    oracle.build()
+    rng = np.random.default_rng([d, N, 9])
+    ne, P = int(np.prod(n)), (N + 1) ** d
+    s = {"mild": 0.05, "wide": 0.45, "far": 2.0}.get(kind, 0.3)
+    rho = np.exp(rng.uniform(-s, s, (ne, P)))
+    p = 2.0 * np.exp(rng.uniform(-s, s, (ne, P)))
+    v = [rng.uniform(-0.5, 0.5, (ne, P)) for _ in range(d)]
+    w = rng.standard_normal((ne, d + 2, P))
+    if kind == "mixed":
+        rho[::3, 0] = 1e4
+        p[1::3, P - 1] = 5e3
+        w[2::3, :, 0] = 0.0
+        w[2] = 0.0
+    if kind == "fast":
+        v = [30.0 + 2.0 * x for x in v]
+    if kind == "still":
+        v = [0.0 * x for x in v]
+    if kind == "units":
+        rho, p, v = rho * 1e-20, p * 1e-8, [x * 1e6 for x in v]
+    if kind in ("mass", "momentum", "energy"):
+        keep = {"mass": [0], "momentum": list(range(1, d + 1)), "energy": [d + 1]}[kind]
+        w[:, [k for k in range(d + 2) if k not in keep]] = 0.0
+    u = np.ascontiguousarray(W.prim_to_cons(rho, v, p).reshape(-1))
+    w = np.ascontiguousarray(w.reshape(-1))
+    m = Mesh(d, N, n)
+    ub = m.rhs_vjp(torch.from_numpy(u).cuda(), torch.from_numpy(w).cuda()).cpu().numpy()
+    ub = ub.reshape(ne, -1)
+    scale = np.abs(u.reshape(ne, d + 2, P)).max(axis=(0, 2))
+    for e in range(min(ne, 6)):
+        t = np.zeros((ne, d + 2, P))
+        t[e] = rng.standard_normal((d + 2, P)) * scale[:, None]
+        jv = oracle.rhs_jvp(d, N, n, W.box(d), u, np.ascontiguousarray(t.reshape(-1)))
+        gap = abs(float(w @ jv) - float(ub[e] @ t[e].reshape(-1)))
+        size = float(np.abs(w * jv).sum())
+        assert gap <= 1e-12 * size or size == 0.0, (kind, e, gap, size)

@@ -12,7 +12,9 @@
 // 37% waiting for dependent results; this layout runs 24 warps per SM. Measured
 // at 64^3 N = 3, a fused stage's volume kernel: FP64 8.47 ms, fixed point with
 // one thread per line 3.87, this layout 2.49; rhs at 24^3 N = 7: 8.14 ms to
-// 2.0. The threads of a line share a warp
+// 2.0. About 40 FP64 instructions per node are left (prologue, lifting, stage
+// update); the sums become doubles on the integer pipe (to_double's two
+// additions per value cost the step 4%: 14.98 and 14.30 ms). The threads of a line share a warp
 // (32/T lines per warp), so rounds are separated by a warp barrier. At N = 3
 // in 3D a warp owns a whole element (16 lines x 2) and no block barrier runs
 // at all.
@@ -182,15 +184,20 @@ struct FxPrim {
 };
 template <int D>
 __device__ __forceinline__ FxPrim<D> fx_prim(const double* c, const Geom& g, unsigned& bad) {
-  double rr;
-  const Prim<double, D> q = prim_rcp<D>(c, g.gm1, rr);
-  bad |= prim_check(q);
+  Prim<double, D> q;
   FxPrim<D> r;
-  r.rho = q.rho;
-  r.p = q.p;
-  r.e = q.p * rr * g.gm1inv;
+  q.rho = r.rho = c[0];
+  const double rr = rcp(c[0]);
+  double mv = 0.0;
 #pragma unroll
-  for (int k = 0; k < D; ++k) r.v[k] = q.v[k];
+  for (int k = 0; k < D; ++k) {
+    q.v[k] = r.v[k] = c[1 + k] * rr;
+    mv = fma(c[1 + k], r.v[k], mv);
+  }
+  const double i = fma(-0.5, mv, c[D + 1]);  // rho e
+  q.p = r.p = g.gm1 * i;
+  r.e = i * rr;
+  bad |= prim_check(q);
   return r;
 }
 
@@ -323,8 +330,8 @@ __device__ __forceinline__ void fx_stage(const Geom& g, int count, unsigned char
 template <int D>
 __device__ __forceinline__ double fx_value(fx::i64 a, int v, const fx::Scale& sc, int ed) {
   if (!sc.ok) return __longlong_as_double(a);
-  return fx::to_double(a, ed + (v == 0 ? sc.er + sc.ev - 60 : v <= D ? sc.em - 61
-                                                                     : sc.em + sc.ev - 59));
+  return fx::to_double_int(a, ed + (v == 0 ? sc.er + sc.ev - 60 : v <= D ? sc.em - 61
+                                                                         : sc.em + sc.ev - 59));
 }
 
 // the sums of a node as doubles, with the lifting of the faces it lies on
@@ -433,7 +440,12 @@ __device__ __forceinline__ void fx_batch(double* u, double* __restrict__ du,
         }
       }
       __syncwarp();
-      for (int node = lane; node < P; node += 32) {
+#pragma unroll 1
+      for (int j = 0; j < NPL; ++j) {
+        // N = 3: the nodes of the two z faces first, then those that have no
+        // face in z, so that the second pass skips that direction's lifting
+        const int node = D == 3 && N == 3 ? (lane & 15) + 16 * (lane < 16 ? j : 3 - j)
+                                          : lane + 32 * j;
         double val[NV];
         fx_result<D, N>(elem, sc, ed, tb, fs, nelem, e, sh.left[el], node, val);
 #pragma unroll

@@ -93,7 +93,7 @@ struct FaceBlend {
         k = 0;
       } else {
         // sR/(sR - sL), both speeds below 2^62: the quotient in FP64
-        const double sr = to_double(sR, 0), sl = to_double(sL, 0);
+        const double sr = to_double_int(sR, 0), sl = to_double_int(sL, 0);
         x = half_fixed(sr * rcp(sr - sl), 0);
         if (x > (1LL << 62)) x = 1LL << 62;
         k = mul(limbs(x), limbs(sL)) << 2;

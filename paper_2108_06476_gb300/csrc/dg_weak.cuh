@@ -12,7 +12,9 @@
 //
 // One thread per node, its primitives and sums in registers, the fluxes of one
 // direction in shared memory. 32^3 N = 4: rhs 2.11 ms with a pair flux per pair
-// in FP64, 0.92 ms here with the same (HLL) faces.
+// in FP64, 0.92 ms here with the same (HLL) faces, 0.50 with faces on integers and
+// the sums made doubles on the integer pipe (0.54 by FP64 additions: the FP64
+// unit, 77% busy with prologue, lifting and stage update, bounds the kernel).
 #pragma once
 
 namespace dg {
@@ -206,7 +208,8 @@ __global__ void __launch_bounds__(WeakLaunch<D, N>::THREADS)
   double val[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v)
-    val[v] = w.ok ? fx::to_double(acc[v], ed + (v == 0 ? w.em : v <= D ? w.ef : w.eh + w.ev) - 60)
+    val[v] = w.ok ? fx::to_double_int(acc[v],
+                                      ed + (v == 0 ? w.em : v <= D ? w.ef : w.eh + w.ev) - 60)
                   : __longlong_as_double(acc[v]);
   const long long base = g.nelem * LINES;
 #pragma unroll

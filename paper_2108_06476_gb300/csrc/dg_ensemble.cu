@@ -790,7 +790,10 @@ int dg_ensemble_get_block(const dg_ensemble* E, int* threads, int* ctas_per_sm, 
 // Autotuner: times one stage for every candidate (threads per CTA, CTAs per
 // SM and, for FP64, elements of an item at once or in turn) from u into u_tmp
 // (u is not changed) and keeps the fastest; the RK register is saved and
-// restored around the trials.
+// restored around the trials, and so are the time steps: the trials take 1e-8
+// (with the zeros of an ensemble that has not stepped yet the coefficients
+// times dt would be zeros and every element take the FP64 form: 30 ms a stage
+// instead of 11, and another shape the fastest).
 int dg_ensemble_tune(dg_ensemble* E, const double* u, double* u_tmp, int* best_threads,
                      int* best_blocks_per_sm, float* best_ms) {
   if (!E || !u || !u_tmp || u == u_tmp) return fail(DG_ERR_ARG, "dg_ensemble_tune: bad argument");
@@ -800,9 +803,14 @@ int dg_ensemble_tune(dg_ensemble* E, const double* u, double* u_tmp, int* best_t
   int bt = E->block, bb = E->per_sm, bp_mode = E->pair;
   const int n_modes = E->opt.precision == DG_FP64 ? 2 : 1;
   double* ksave = nullptr;
-  if (cudaMalloc(&ksave, E->nvalues * sizeof(double)) != cudaSuccess)
+  const size_t n_sims = E->sims.size(), dt_bytes = n_sims * sizeof(double);
+  if (cudaMalloc(&ksave, E->nvalues * sizeof(double) + dt_bytes) != cudaSuccess)
     return fail(DG_ERR_OOM, "dg_ensemble_tune: cudaMalloc");
+  double* const dtsave = ksave + E->nvalues;
+  const std::vector<double> trial(n_sims, 1e-8);
   cudaMemcpyAsync(ksave, E->k, E->nvalues * sizeof(double), cudaMemcpyDeviceToDevice, E->stream);
+  cudaMemcpyAsync(dtsave, E->dt, dt_bytes, cudaMemcpyDeviceToDevice, E->stream);
+  cudaMemcpyAsync(E->dt, trial.data(), dt_bytes, cudaMemcpyHostToDevice, E->stream);
   cudaEvent_t a, b;
   cudaEventCreate(&a);
   cudaEventCreate(&b);
@@ -830,6 +838,7 @@ int dg_ensemble_tune(dg_ensemble* E, const double* u, double* u_tmp, int* best_t
     }
   }
   cudaMemcpyAsync(E->k, ksave, E->nvalues * sizeof(double), cudaMemcpyDeviceToDevice, E->stream);
+  cudaMemcpyAsync(E->dt, dtsave, dt_bytes, cudaMemcpyDeviceToDevice, E->stream);
   cudaStreamSynchronize(E->stream);
   cudaFree(ksave);
   cudaEventDestroy(a);

@@ -341,11 +341,25 @@ __global__ void speed_kernel(const double* __restrict__ u, Geom g, int P, int ep
       speed_node(c, D, g, lamr, bad, R(0));
     }
     double lam[3];
+    if (sizeof(R) == 4) {
+      // FP32: the maxima by shuffles of floats, and the sum in FP64 only if it
+      // may be the largest (in FP64 throughout, the 22 instructions per element
+      // held the unit 81% of the pass: 167 us at 48^3 N = 3)
+      float sum = 0.0f;
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        for (int off = seg / 2; off > 0; off >>= 1)
+          lamr[k] = fmaxf(lamr[k], __shfl_xor_sync(0xffffffffu, lamr[k], off));
+        sum = fmaf(k == 0 ? s0f : (k == 1 ? s1f : s2f), lamr[k], sum);
+      }
+      if (__all_sync(0xffffffffu, sum > 1e-30f && sum < dg::d2f(best) * 0.999999f)) continue;
+    }
 #pragma unroll
     for (int k = 0; k < D; ++k) {
       lam[k] = (double)lamr[k];
-      for (int off = seg / 2; off > 0; off >>= 1)
-        lam[k] = fmax(lam[k], __shfl_xor_sync(0xffffffffu, lam[k], off));
+      if (sizeof(R) == 8)
+        for (int off = seg / 2; off > 0; off >>= 1)
+          lam[k] = fmax(lam[k], __shfl_xor_sync(0xffffffffu, lam[k], off));
     }
     double s = s0 * lam[0];
     s = s + s1 * lam[1];

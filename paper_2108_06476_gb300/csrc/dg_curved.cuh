@@ -632,21 +632,21 @@ __global__ void curved_speed_kernel(const double* __restrict__ u, const double* 
       }
       const Prim<double, 3> q = prim_rcp<3>(c, g.gm1, rr);
       bad |= prim_check(q);
-      const double cs = sqrt(g.gamma * q.p * rr), ij = invJ[e * P + node];
+      const double cs = sqrt_pos(g.gamma * q.p * rr), ij = invJ[e * P + node];
 #pragma unroll
       for (int r = 0; r < 3; ++r) {
         double gv[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) gv[k] = Ja[((e * 3 + r) * 3 + k) * P + node];
         const double vg = fma(q.v[2], gv[2], fma(q.v[1], gv[1], q.v[0] * gv[0]));
-        const double gn = sqrt(fma(gv[2], gv[2], fma(gv[1], gv[1], gv[0] * gv[0])));
+        const double gn = sqrt_pos(fma(gv[2], gv[2], fma(gv[1], gv[1], gv[0] * gv[0])));
         lam[r] = fmax(lam[r], (fabs(vg) + cs * gn) * ij);
       }
     }
 #pragma unroll
     for (int r = 0; r < 3; ++r)
       for (int off = 16; off > 0; off >>= 1)
-        lam[r] = fmax(lam[r], __shfl_xor_sync(0xffffffffu, lam[r], off));
+        lam[r] = fmax_nn(lam[r], __shfl_xor_sync(0xffffffffu, lam[r], off));
     best = fmax(best, lam[0] + lam[1] + lam[2]);
   }
   __shared__ double sb[32];

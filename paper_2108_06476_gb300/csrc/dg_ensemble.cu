@@ -207,7 +207,7 @@ __device__ void ens_volume_pp(const EnsArgs& a, const SimDesc& sd, const WorkIte
 // one cooperative launch per stage: blocks walk the work list (largest
 // degrees first) in each phase; CTAs of at most 128 threads. FP64: 80 registers
 // a thread, so that six CTAs fit an SM (48 members: 154 ms per step with one
-// thread per line in FP64 at 168 registers, 71 ms in fixed point); FP32: at
+// thread per line in FP64 at 168 registers, 57 ms in fixed point); FP32: at
 // most 168, three CTAs.
 constexpr int kEnsMaxThreads = 128;
 template <typename R>

@@ -325,8 +325,7 @@ __global__ void speed_kernel(const double* __restrict__ u, Geom g, int P, int ep
         sum = fmaf(k == 0 ? s0f : (k == 1 ? s1f : s2f), up[k], sum);
       }
       const double most = fmax(best, __longlong_as_double((long long)seen));
-      if (__all_sync(0xffffffffu, fine) && sum > 1e-30f && sum < dg::d2f(most) * 0.999999f)
-        continue;
+      if (dg::speed_skip(fine, sum, most)) continue;
     }
     const double* uc = sizeof(R) == 8 && epw == 1 && copy_to ? copy_to : u;
     R lamr[3] = {R(0), R(0), R(0)};
@@ -352,7 +351,7 @@ __global__ void speed_kernel(const double* __restrict__ u, Geom g, int P, int ep
           lamr[k] = fmaxf(lamr[k], __shfl_xor_sync(0xffffffffu, lamr[k], off));
         sum = fmaf(k == 0 ? s0f : (k == 1 ? s1f : s2f), lamr[k], sum);
       }
-      if (__all_sync(0xffffffffu, sum > 1e-30f && sum < dg::d2f(best) * 0.999999f)) continue;
+      if (dg::speed_skip(true, sum, best)) continue;
     }
 #pragma unroll
     for (int k = 0; k < D; ++k) {

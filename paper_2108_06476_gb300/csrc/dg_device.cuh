@@ -323,6 +323,14 @@ __device__ __forceinline__ bool speed_bound(const double* c, double gamma64, dou
   return rho > 1e-30f && rho < 1e30f && p > off && p > 1e-30f && E < 1e30f;
 }
 
+// Whether the warp passes over an element whose sum of wave speeds is at most
+// `bound`, the largest sum found so far being `most`. Each lane may have read
+// another value of the running maximum, which other warps raise: one vote, so
+// that all lanes take the same way (the shuffles that follow name every lane).
+__device__ __forceinline__ bool speed_skip(bool fine, float bound, double most) {
+  return __all_sync(0xffffffffu, fine && bound > 1e-30f && bound < d2f(most) * 0.999999f);
+}
+
 // ---- logarithmic mean ----
 // ln_mean(x, y) = (y - x) / ln(y / x). With s = x + y, t = (y - x)/s and
 // f2 = t^2, ln(y/x) = 2 atanh(t), so

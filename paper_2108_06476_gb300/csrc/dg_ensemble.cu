@@ -284,9 +284,7 @@ __global__ void ensemble_speed_kernel(const SimDesc* __restrict__ sims,
           up[k] = fmaxf(up[k], __shfl_xor_sync(0xffffffffu, up[k], off));
         bound = fmaf((float)sd.lam_scale[k] * 1.000001f, up[k], bound);
       }
-      if (__all_sync(0xffffffffu, fine) && bound > 1e-30f &&
-          bound < d2f(__longlong_as_double((long long)seen)) * 0.999999f)
-        continue;
+      if (speed_skip(fine, bound, __longlong_as_double((long long)seen))) continue;
       double lam[3] = {0.0, 0.0, 0.0};
       for (int node = lane; node < P; node += 32) {
         double c[5];

@@ -301,7 +301,7 @@ __global__ void mhd_speed_kernel(const double* __restrict__ u, Geom g, int P, do
       bound = fmaf(sf[k], up[k], bound);
     }
     const double most = fmax(best, __longlong_as_double((long long)seen));
-    if (__all_sync(0xffffffffu, fine) && bound > 1e-30f && bound < d2f(most) * 0.999999f) continue;
+    if (speed_skip(fine, bound, most)) continue;
     const double* uc = copy_to ? copy_to : u;
     double lam[3] = {0.0, 0.0, 0.0};
     for (int node = lane; node < P; node += 32) {

@@ -320,7 +320,8 @@ __device__ __forceinline__ bool speed_bound(const double* c, double gamma64, dou
   const float cs = sqrtf(gamma * (p + off) * r);
 #pragma unroll
   for (int k = 0; k < D; ++k) lam[k] = fmaxf(lam[k], (fabsf(v[k]) + cs) * 1.000004f);
-  return rho > 1e-30f && rho < 1e30f && p > off && p > 1e-30f && E < 1e30f;
+  // p/rho normal by a wide margin: an underflow of c^2 would leave c out
+  return rho > 1e-30f && rho < 1e30f && p > off && p > 1e-30f && p * r > 1e-30f && E < 1e30f;
 }
 
 // Whether the warp passes over an element whose sum of wave speeds is at most

@@ -5,6 +5,7 @@ other warps raise it. Shown on the host: the function with the lanes of a warp
 one after another, the votes collected first.
 """
 import ctypes
+import itertools
 import os
 import re
 import subprocess
@@ -75,3 +76,45 @@ extern "C" int decide(const int* fine, float bound, const double* most) {
         assert decide([1] * 32, 1.5, [1.0] * k + [2.0] * (32 - k)) in (0, 32)
     assert decide([1] * 31 + [0], 1.0, [2.0] * 32) == 0
     assert decide([1] * 32, float("nan"), [2.0] * 32) == 0
+
+
+def test_the_bound_holds_wherever_it_is_used(tmp_path):
+    # speed_bound on the host (FP32 with subnormals, as on the device) against
+    # 40-digit wave speeds, over every size of state that it accepts
+    mp = pytest.importorskip("mpmath")
+    mp.mp.dps = 40
+    src, so = tmp_path / "bound.cpp", tmp_path / "bound.so"
+    body = _function(_text("dg_device.cuh"), "__device__ __forceinline__ bool speed_bound(")
+    src.write_text(r"""
+#include <cmath>
+using std::fabs;
+#define __device__
+#define __forceinline__ inline
+static float d2f(double x) { return (float)x; }
+template <int D>
+""" + body + r"""
+extern "C" int bound(const double* c, double gamma, float* lam) {
+  return speed_bound<3>(c, gamma, gamma - 1.0, lam);
+}
+""")
+    subprocess.run(["g++", "-O1", "-ffp-contract=off", "-fPIC", "-shared", str(src), "-o",
+                    str(so)], check=True)
+    lib = ctypes.CDLL(str(so))
+    used = 0
+    for rho, prel, mach, gamma in itertools.product(
+            (1e-29, 1e-10, 1.0, 1e10, 1e22, 9e29), (1e-50, 1e-44, 1e-38, 1e-29, 1e-12, 1.0, 1e12),
+            (0.0, 1e-2, 0.7, 3.0), (1.4, 5.0 / 3.0)):
+        p = prel * rho
+        cs = (gamma * prel) ** 0.5
+        v = [mach * cs * s for s in (1.0, -0.5, 0.25)]
+        c = [rho, *(rho * x for x in v), p / (gamma - 1.0) + 0.5 * rho * sum(x * x for x in v)]
+        lam = (ctypes.c_float * 3)(0.0, 0.0, 0.0)
+        if not lib.bound((ctypes.c_double * 5)(*c), ctypes.c_double(gamma), lam):
+            continue
+        used += 1
+        m = [mp.mpf(x) for x in c]
+        pe = (mp.mpf(gamma) - 1) * (m[4] - sum(x * x for x in m[1:4]) / m[0] / 2)
+        ce = mp.sqrt(mp.mpf(gamma) * pe / m[0])
+        for k in range(3):
+            assert lam[k] >= abs(m[1 + k] / m[0]) + ce, (rho, prel, mach, gamma, k)
+    assert used > 60

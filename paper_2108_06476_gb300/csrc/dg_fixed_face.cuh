@@ -6,9 +6,11 @@
 // traces once 1/rho and the sound speeds are known: the reciprocals and the
 // square roots stay in FP64 (15 instructions for LLF), the rest runs on
 // integers with power-of-two exponents chosen per face node from its two
-// traces, 61 to 63 bits below the larger one. Faces whose densities differ by
-// more than 2^6, or with non-finite or non-positive values, take the FP64
-// form (surface_nf). Measured at 64^3 N = 3 (12.6 M face nodes, LLF): 1.38 ms
+// traces, 61 to 63 bits below the larger one. Faces whose densities or energies
+// differ by more than 2^6, or with non-finite or non-positive values, take the
+// FP64 form (surface_nf): beyond that the weaker trace would keep fewer bits
+// than FP64 has. Where HLL takes one trace's own flux, that is evaluated in
+// FP64 from this trace, whatever the other one's size. Measured at 64^3 N = 3 (12.6 M face nodes, LLF): 1.38 ms
 // in FP64, 0.64 ms here (80 registers, 24 warps per SM; 0.72 at 96 registers).
 #pragma once
 #include "dg_fixed.cuh"
@@ -62,6 +64,7 @@ __device__ __forceinline__ i64 abs64(i64 a) { return a < 0 ? -a : a; }
 // kappa = -lambda/2) and HLL (w = sR/(sR - sL), kappa = w sL)
 struct FaceBlend {
   bool hll;
+  int side;      // HLL: 1 or 2 where the flux is the left or the right one
   Limbs kap, w;  // kappa (62 - eL + kx), w (62)
   int eL, kx;
 
@@ -70,6 +73,7 @@ struct FaceBlend {
   __device__ __forceinline__ void speeds(bool is_hll, i64 vl, i64 vr, int ev, i64 cl, i64 cr,
                                          int ec) {
     hll = is_hll;
+    side = 0;
     eL = (ev > ec ? ev : ec) + 1;
     const int dv = eL - ev < 63 ? eL - ev : 63, dc = eL - ec < 63 ? eL - ec : 63;
     vl >>= dv;
@@ -85,12 +89,11 @@ struct FaceBlend {
     } else {
       const i64 sL = vl - cl < vr - cr ? vl - cl : vr - cr;
       const i64 sR = vl + cl > vr + cr ? vl + cl : vr + cr;
+      k = 0;
       if (sL >= 0) {
-        x = 1LL << 62;
-        k = 0;
+        side = 1;
       } else if (sR <= 0) {
-        x = 0;
-        k = 0;
+        side = 2;
       } else {
         // sR/(sR - sL), both speeds below 2^62: the quotient in FP64
         const double sr = to_double_int(sR, 0), sl = to_double_int(sL, 0);
@@ -151,8 +154,10 @@ __device__ __forceinline__ bool face_fixed(bool hll, const double* cl, const dou
   }
   const unsigned el = hiword(cl[D + 1]), er_ = hiword(cr[D + 1]);
   const unsigned ke = el > er_ ? el : er_;  // above 0x7ff... if one is negative or NaN
+  const unsigned kd = ke - (el > er_ ? er_ : el);
   const unsigned lo = (kBias - 150u) << 20, hi = (kBias + 150u) << 20;
-  if (!(rmax < hi && rmin > lo && rmax - rmin < (6u << 20) && km < hi && ke < hi && ke > lo))
+  if (!(rmax < hi && rmin > lo && rmax - rmin < (6u << 20) && km < hi && ke < hi && ke > lo &&
+        kd < (6u << 20)))
     return false;
   const int eg = exp_above(hiword(gm1));
   const int er = exp_above(rmax);
@@ -218,6 +223,19 @@ __device__ __forceinline__ bool face_fixed(bool hll, const double* cl, const dou
   const int es = exp_above(kc);
   FaceBlend blend;
   blend.speeds(hll, S[0].vn, S[1].vn, ev, half_fixed(ca, es), half_fixed(cb, es), es);
+  if (blend.side) {
+    const double* c = blend.side == 1 ? cl : cr;
+    double cc[D + 2];
+#pragma unroll
+    for (int v = 0; v < D + 2; ++v) cc[v] = c[v];
+    double rr;
+    const Prim<double, D> q = prim_rcp<D>(cc, gm1, rr);
+    f[0] = cc[1];
+#pragma unroll
+    for (int k = 0; k < D; ++k) f[1 + k] = fma(cc[1], q.v[k], k == 0 ? q.p : 0.0);
+    f[D + 1] = (cc[D + 1] + q.p) * q.v[0];
+    return true;
+  }
   const i64 drho = full_fixed(cr[0], er) - full_fixed(cl[0], er);
   f[0] = blend(S[0].m[0], S[1].m[0], em - 63, drho, er - 63);
 #pragma unroll

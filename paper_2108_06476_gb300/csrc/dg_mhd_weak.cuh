@@ -132,7 +132,10 @@ __device__ __forceinline__ bool mhd_face_fixed(bool hll, const double* cl, const
     key[2] = max(key[2], max(hw(cl[1 + k]) & 0x7fffffffu, hw(cr[1 + k]) & 0x7fffffffu));
     key[3] = max(key[3], max(hw(cl[5 + k]) & 0x7fffffffu, hw(cr[5 + k]) & 0x7fffffffu));
   }
-  const MWScale w = mw_scale(key, gm1, true);
+  // energies more than 2^6 apart: the weaker trace would keep fewer bits than
+  // FP64 has
+  const unsigned kd = key[4] - min(hw(cl[4]), hw(cr[4]));
+  const MWScale w = mw_scale(key, gm1, kd < (6u << 20));
   if (!w.ok) return false;
   const MWNode L = mw_node(cl, vl, w, gm1), R = mw_node(cr, vr, w, gm1);
   if (L.p <= 0 || R.p <= 0) return false;
@@ -153,6 +156,14 @@ __device__ __forceinline__ bool mhd_face_fixed(bool hll, const double* cl, const
   }
   fx::FaceBlend blend;
   blend.speeds(hll, L.v[0], R.v[0], w.ev, ca, cb, ec);
+  if (blend.side) {  // one trace's own flux, in FP64 whatever the other's size
+    double c[kMV];
+#pragma unroll
+    for (int v = 0; v < kMV; ++v) c[v] = blend.side == 1 ? cl[v] : cr[v];
+    unsigned dummy = 0;
+    mhd_flux<0>(mhd_state(c, gm1, dummy), c, f);
+    return true;
+  }
   fx::i64 fl[kMV], fr[kMV];
   mw_flux(L, w, 0, fl);
   mw_flux(R, w, 0, fr);

@@ -1,0 +1,78 @@
+"""The integer kernels on data that spans many orders of magnitude.
+
+Each variable is compared with the oracle node by node or plane by plane of an
+element, relative to the largest entry there: a strong trace or node must not
+cost a weak one its digits. The bar is the project's 1e-12 (some hundreds of
+operations of 2^-53 on data whose sums do not cancel by more than a factor of a
+hundred).
+"""
+import numpy as np
+import pytest
+
+BAR = 1e-12
+
+
+def _gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import oracle
+    oracle.build()
+    return torch
+
+
+def _mhd(rho, v, p, B):
+    E = p / (5.0 / 3.0 - 1.0) + 0.5 * rho * (v ** 2).sum(0) + 0.5 * (B ** 2).sum(0)
+    return np.ascontiguousarray(np.stack([rho, *(rho * v), E, *B], axis=1))
+
+
+def _euler(rho, v, p):
+    E = p / 0.4 + 0.5 * rho * (v ** 2).sum(0)
+    return np.ascontiguousarray(np.stack([rho, *(rho * v), E], axis=1))
+
+
+def _rhs(torch, eq, d, N, n, vf, sf, u):
+    import oracle
+    from paper_2108_06476_gb300 import Mesh, workloads as W
+    m = Mesh(d, N, n, volume_flux=vf, surface_flux=sf, equations=eq)
+    got = m.rhs(torch.from_numpy(u.reshape(-1)).cuda()).cpu().numpy().reshape(u.shape)
+    assert m.check() == 0
+    if eq == "mhd":
+        ref = oracle.mhd_rhs(N, n, W.box(3), u.reshape(-1), sflux=sf, vflux=vf)
+    else:
+        ref = oracle.rhs(d, N, n, W.box(d), u.reshape(-1),
+                         vflux={"ranocha": 0, "central": 2}[vf],
+                         sflux={"llf": 0, "ranocha": 1, "hll": 2}[sf])
+    return got, ref.reshape(u.shape)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("eq,d,vf,sf", [("euler", 3, "ranocha", "hll"), ("euler", 3, "central", "hll"),
+                                        ("euler", 2, "central", "hll"), ("euler", 3, "ranocha", "llf"),
+                                        ("mhd", 3, "central", "hll"), ("mhd", 3, "central", "llf")])
+@pytest.mark.parametrize("ratio", [1.0, 60.0, 1e3, 1e6, 1e8])
+@pytest.mark.parametrize("flow", ["right", "left", "slow"])
+def test_faces_between_traces_of_different_size(eq, d, vf, sf, ratio, flow):
+    # element by element along x cold and hot gas, both supersonic by their own
+    # sound speeds (HLL: the face flux is the upwind trace's own) or slow; the
+    # planes of nodes x = const of an element each by themselves (only the two
+    # outer ones see a face's flux)
+    torch = _gpu()
+    N, n = 2, ((6, 11, 10) if d == 3 else (26, 24))
+    ne, P = int(np.prod(n)), (N + 1) ** d
+    rng = np.random.default_rng(int(ratio) + d)
+    hot = (np.arange(ne) % n[0]) % 2 == 1
+    rho = rng.uniform(0.7, 1.4, (ne, P))
+    p = np.where(hot[:, None], ratio, 1.0) * rng.uniform(0.9, 1.1, (ne, P))
+    c = np.sqrt(np.where(hot, ratio, 1.0))[:, None] * 1.5
+    v = c * rng.uniform(-0.3, 0.3, (d, ne, P))
+    if flow != "slow":
+        v[0] += c * (2.0 if flow == "right" else -2.0)
+    if eq == "mhd":
+        u = _mhd(rho, v, p, 0.2 * c * rng.uniform(-1, 1, (3, ne, P)))
+    else:
+        u = _euler(rho, v, p)
+    got, ref = _rhs(torch, eq, d, N, n, vf, sf, u)
+    err, size = (np.abs(x).reshape(ne, u.shape[1], -1, N + 1).max(axis=2) for x in (got - ref, ref))
+    err = err / size
+    assert err.max() <= BAR, (err.max(axis=(0, 2)), np.unravel_index(err.argmax(), err.shape))

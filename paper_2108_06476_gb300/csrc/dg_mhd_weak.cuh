@@ -1,12 +1,15 @@
 // The weak-form MHD volume term in 64-bit fixed point (dg_fixed.cuh), one
 // thread per node as mhd_volume_kernel did in FP64 (191 FP64 instructions per
 // node, 64 cycles of the sub-partition's FP64 unit each). The primitives, the
-// nodal fluxes and the product with the derivative rows run on integers scaled
-// by per-element powers of two; the reciprocal of the density, the lifting of
-// the face values, the Powell term and the stage update stay in FP64 (about 60
-// instructions), so that both pipes are busy. The lifting's - lift f(u_i) at
-// the line ends is part of the diagonal (M_00 = -liftL/2, M_NN = -liftR/2, the
-// rows of the derivative matrix summing to zero). Elements with non-finite
+// nodal fluxes, the product with the derivative rows and the lifting of the face
+// values run on integers scaled by per-element powers of two; the reciprocal of
+// the density, the Powell term and the stage update stay in FP64, so that both
+// pipes are busy. The lifting's - lift f(u_i) at the line ends is part of the
+// diagonal (M_00 = -liftL/2, M_NN = -liftR/2, the rows of the derivative matrix
+// summing to zero), and + lift F* is added before the sum is rounded to FP64:
+// the two cancel (added afterwards in FP64, the error of smooth data was up to
+// 2.2 times that of lift (F* - f(u_i)), at a supersonic outflow 25 times). A
+// face value beyond the element's units is added in FP64. Elements with non-finite
 // values, non-positive densities or densities spread over more than 2^6 take
 // the same steps in FP64.
 //
@@ -52,6 +55,14 @@ __device__ __forceinline__ MWScale mw_scale(const unsigned* key, double gm1, boo
   if (w.ee < 2 * w.eb + 1) w.ee = 2 * w.eb + 1;
   w.ee += 1 + (eg > 0 ? eg : 0);
   return w;
+}
+
+// The halves of a unit that a product with the coefficient k loses on average to
+// truncation (fma64: one for each limb), and in the upper 16 bits those with a
+// factor of 53 bits (momenta and B_n): its low 8 bits are zeros, so a high limb
+// of 8 bits loses nothing (N = 1 and 2, where the rows are few-bit numbers).
+__device__ __forceinline__ int mw_cut(fx::Limbs k) {
+  return (k.h != 0) + (k.l != 0) + (((k.h & 0xffffff) != 0) + (k.l != 0)) * 65536;
 }
 
 __device__ __forceinline__ fx::i64 shr(fx::i64 a, int n) { return a >> (n < 63 ? n : 63); }
@@ -192,6 +203,8 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
   __shared__ fx::Limbs s_m[3][NP][NP + 1];            // M, format 62 - ed
   __shared__ double s_m64[3][NP][NP + 1];
   __shared__ double s_lift[2][3];
+  __shared__ fx::Limbs s_liftx[2][3];                 // 62 - ed
+  __shared__ int s_cut[3][NP];  // mw_cut over a row and its lifting
   __shared__ unsigned s_key[EPB][6];                  // see mw_scale
   const int e0 = blockIdx.x * EPB;
   const int count = (int)g.nelem - e0 < EPB ? (int)g.nelem - e0 : EPB;
@@ -203,8 +216,9 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
 #pragma unroll
   for (int v = 0; v < kMV; ++v)
     c[v] = in ? u[((long long)e * kMV + v) * P + node] : (v == 0 || v == 4 ? 1.0 : 0.0);
-  // the largest coefficient is that of D_01; with the diagonal the absolute
-  // row sums stay below 8.2 times it
+  // the largest coefficient is that of D_01, the lifting's at most twice it;
+  // with the diagonal the absolute row sums stay below 8.2 times it, with the
+  // lifting of three directions below 12.6 times (of the 16 that fit)
   unsigned mk = 0;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -217,11 +231,13 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
     double m = sc * tb.Ds[dir][a][b];
     if (a == b) m = a == 0 ? -0.5 * sc * tb.liftL[dir] : (a == N ? -0.5 * sc * tb.liftR[dir] : 0.0);
     s_m64[dir][a][b] = m;
-    s_m[dir][a][b] = fx::limbs(fx::half_fixed(m, ed));
+    s_m[dir][a][b] = fx::limbs(fx::half_fixed(m, ed));  // the diagonal: below
   }
   if (t < 3) {
     s_lift[0][t] = sc * tb.liftL[t];
     s_lift[1][t] = sc * tb.liftR[t];
+    s_liftx[0][t] = fx::limbs(fx::half_fixed(s_lift[0][t], ed));
+    s_liftx[1][t] = fx::limbs(fx::half_fixed(s_lift[1][t], ed));
   }
   if (t < count) {
     s_key[t][0] = s_key[t][2] = s_key[t][3] = s_key[t][4] = s_key[t][5] = 0u;
@@ -230,6 +246,23 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
   const double rr = rcp(c[0]);
   const double vel[3] = {c[1] * rr, c[2] * rr, c[3] * rr};
   __syncthreads();
+  if (t < 3 * NP) {
+    // the rows with their lifting sum to zero exactly (the coefficients'
+    // roundings would leave 2^-53 of a constant flux or field)
+    const int dir = t / NP, a = t % NP;
+    fx::i64 x = 0;
+    int cut = 0;
+    auto take = [&](fx::Limbs k) {
+      x -= (fx::i64)k.h * (1LL << 32) + k.l;
+      cut += mw_cut(k);
+    };
+    for (int b = 0; b < NP; ++b)
+      if (b != a) take(s_m[dir][a][b]);
+    if (a == 0) take(s_liftx[0][dir]);
+    if (a == N) take(s_liftx[1][dir]);
+    s_m[dir][a][a] = fx::limbs(x);
+    s_cut[dir][a] = cut + mw_cut(fx::limbs(x));
+  }
   {
     auto hw = [](double x) { return (unsigned)__double2hiint(x); };
     unsigned km = 0, kb = 0, kv = 0;
@@ -272,12 +305,19 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
   }
   if (in && bad) atomicOr(err, bad);
   fx::i64 acc[kMV + 1];
-  // truncation (fma64): the sums start from their number of terms, those of
-  // zero fluxes from zero
+  // truncation (fma64): the sums start from what their products lose on
+  // average, those of zero fluxes from zero
+  int cut = 0;
+#pragma unroll
+  for (int dir = 0; dir < 3; ++dir) {
+    int l, a;
+    line_of<N>(dir, node, l, a);
+    cut += s_cut[dir][a];
+  }
 #pragma unroll
   for (int v = 0; v <= kMV; ++v) {
     const bool some = v == 0 || v == 4 ? w.moves : (v <= 3 ? true : (v < kMV ? w.moves && w.field : w.field));
-    acc[v] = w.ok && some ? 3 * NP : 0;
+    acc[v] = w.ok && some ? ((v == 0 || v == kMV ? cut >> 16 : cut & 0xffff) + 1) / 2 : 0;
   }
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
@@ -330,24 +370,52 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
     if (dir < 2) __syncthreads();
   }
   if (!in) return;
+  // exponents of the fluxes' units: below 2^62 for values below 2^x
+  auto unit = [&](int v) {
+    return v == 0 ? w.em : v <= 3 ? w.ee + 1 : v == 4 ? w.ev + w.ee + 1
+                                     : v < kMV ? w.ev + w.eb + 1 : w.eb;
+  };
+  const long long base = g.nelem * LINES;
+  auto face = [&](int dir, int i, int l) {
+    const long long ef = i == N ? e : neighbour(g, e, dir, -1);
+    return fs + (long long)dir * kMQ * base + ef * LINES + l;
+  };
+  // face values that are added in FP64: bit 9 dir + variable
+  static_assert(kMV + 1 == 9, "");
+  unsigned late = w.ok ? 0u : 0x7ffffffu;
+  if (w.ok) {
+#pragma unroll
+    for (int dir = 0; dir < 3; ++dir) {
+      int l, i;
+      line_of<N>(dir, node, l, i);
+      if (i == N || i == 0) {
+        const double* src = face(dir, i, l);
+        const fx::Limbs lift = s_liftx[i == N][dir];
+#pragma unroll
+        for (int v = 0; v <= kMV; ++v) {
+          const double f = src[v * base];
+          const unsigned most = (unsigned)(unit(v) + (int)fx::kBias) << 20;
+          if (((unsigned)__double2hiint(f) & 0x7fffffffu) < most)
+            acc[v] = fx::fma64(lift, fx::limbs(fx::half_fixed(f, unit(v))), acc[v]);
+          else
+            late |= 1u << (9 * dir + v);
+        }
+      }
+    }
+  }
   double val[kMV + 1];
 #pragma unroll
-  for (int v = 0; v <= kMV; ++v) {
-    const int x = v == 0 ? w.em : v <= 3 ? w.ee + 1 : v == 4 ? w.ev + w.ee + 1
-                                              : v < kMV ? w.ev + w.eb + 1 : w.eb;
-    val[v] = w.ok ? fx::to_double_int(acc[v], ed + x - 60) : __longlong_as_double(acc[v]);
-  }
-  const long long base = g.nelem * LINES;
-#pragma unroll
-  for (int dir = 0; dir < 3; ++dir) {
+  for (int v = 0; v <= kMV; ++v)
+    val[v] = w.ok ? fx::to_double_int(acc[v], ed + unit(v) - 60) : __longlong_as_double(acc[v]);
+  for (int dir = 0; late && dir < 3; ++dir, late >>= 9) {
     int l, i;
     line_of<N>(dir, node, l, i);
-    if (i == N || i == 0) {
-      const long long ef = i == N ? e : neighbour(g, e, dir, -1);
+    if ((late & 511u) && (i == N || i == 0)) {
       const double lift = s_lift[i == N][dir];
-      const double* src = fs + (long long)dir * kMQ * base + ef * LINES + l;
+      const double* src = face(dir, i, l);
 #pragma unroll
-      for (int v = 0; v <= kMV; ++v) val[v] = fma(lift, src[v * base], val[v]);
+      for (int v = 0; v <= kMV; ++v)
+        if (late >> v & 1u) val[v] = fma(lift, src[v * base], val[v]);
     }
   }
   if (powell) {

@@ -76,3 +76,42 @@ def test_faces_between_traces_of_different_size(eq, d, vf, sf, ratio, flow):
     err, size = (np.abs(x).reshape(ne, u.shape[1], -1, N + 1).max(axis=2) for x in (got - ref, ref))
     err = err / size
     assert err.max() <= BAR, (err.max(axis=(0, 2)), np.unravel_index(err.argmax(), err.shape))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,n", [(1, (12, 11, 10)), (2, (4, 3, 3)), (3, (9, 9, 8)), (3, (3, 3, 3)),
+                                 (4, (9, 9, 8)), (5, (3, 3, 2)), (7, (2, 2, 3))])
+def test_mhd_lifting_cancels_before_it_is_rounded(N, n):
+    # a nearly uniform flow, supersonic in every direction: the mass flux of
+    # HLL at a face is the left trace's momentum, so the volume sum and the lifting nearly cancel. In integers
+    # the 3 (N + 1) + 3 products of a node are each truncated by at most two
+    # halves of a unit about their mean (0.41 units rms), units of 2^-60 times
+    # the element's powers of two (at most 4 |D_01| and 2 |m|): below 2.1 units
+    # = 2^-55.9 |D_01| |m| rms. Rounded to FP64 in between the sums would be
+    # off by 0.29 2^-52 lift |m| = 2^-53.2 |D_01| |m| and more.
+    torch = _gpu()
+    from perf.cases import _lgl
+    ne, P = int(np.prod(n)), (N + 1) ** 3
+    rng = np.random.default_rng(N)
+    rho, p = np.full((ne, P), 1.0), rng.uniform(0.99, 1.01, (ne, P))
+    v = np.array([4.1, 5.3, 4.7])[:, None, None] * (1.0 + 1e-3 * rng.uniform(-1, 1, (3, ne, P)))
+    u = _mhd(rho, v, p, np.array([0.3, 0.2, 0.1])[:, None, None] * np.ones((3, ne, P)))
+    from paper_2108_06476_gb300 import Mesh
+    m = Mesh(3, N, n, equations="mhd", volume_flux="central", surface_flux="hll")
+    got = m.rhs(torch.from_numpy(u.reshape(-1)).cuda()).cpu().numpy().reshape(u.shape)[:, 0]
+    _, w, D = _lgl(N)
+    ref, size = 0, 0.0
+    for r in range(3):
+        a = 3 - r  # node axis of direction r in [e, k, j, i]
+        mr = u[:, 1 + r].astype(np.longdouble).reshape(ne, N + 1, N + 1, N + 1)
+        d = np.moveaxis(np.tensordot(mr, D, axes=([a], [1])), -1, a)
+        e = mr.reshape(n[::-1] + mr.shape[1:])
+        last = np.take(e, [N], axis=a + 2)
+        from_left = np.roll(last, 1, axis=2 - r).reshape(np.take(mr, [0], axis=a).shape)
+        first = [slice(None)] * 4
+        first[a] = slice(0, 1)
+        d[tuple(first)] -= (from_left - mr[tuple(first)]) / w[0]
+        ref = ref - n[r] * d
+        size = max(size, float(n[r] * abs(D[0, 1]) * np.abs(mr).max()))
+    rms = float(np.sqrt(np.mean((got.reshape(ref.shape) - ref) ** 2)))
+    assert rms <= 2.0 ** -55 * size, rms / size

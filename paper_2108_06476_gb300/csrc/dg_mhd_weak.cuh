@@ -113,16 +113,32 @@ __device__ __forceinline__ void mw_flux(const MWNode& q, const MWScale& w, int d
 }
 
 // half the squared fast speed of the normal (first) direction times the
-// density, and that over the density: c_f^2/2 in 61 - ee - e1
+// density, and that over the density: c_f^2/2 in 61 - ee - e1. With a = gamma p,
+// b_n and b_t the squares of the normal and transverse field, the discriminant
+// (a + b_n + b_t)^2 - 4 a b_n is taken as (a - b_n)^2 + b_t (b_t + 2 (a + b_n)),
+// whose terms do not cancel, and from operands shifted up to their leading bit:
+// where kinetic energy makes up most of the units 2^ee, squares of unshifted
+// ones would lose twice the bits (c_f off by 4e-9 at 100 times the sound
+// speed).
 __device__ __forceinline__ fx::i64 mw_fast2(const MWNode& q, const MWScale& w, fx::Limbs gamma,
                                             int egam, fx::Limbs r) {
-  // quarters of gamma p, |B|^2 and B_n^2 (62 - ee)
-  const fx::i64 a4 = fx::mul(fx::limbs(q.p), gamma) << egam;  // gamma > 1 in 62 - egam
-  const fx::i64 bn4 = shr(fx::mul(fx::limbs(q.B[0]), fx::limbs(q.B[0])), w.ee - 2 * w.eb);
-  const fx::i64 q4 = a4 + (q.hb2 >> 1);
-  const fx::i64 disc = fx::sqr(fx::limbs(q4)) - (fx::mul(fx::limbs(a4), fx::limbs(bn4)) << 2);
-  const fx::i64 k = q4 + fx::sqrt_fixed(disc << 2);  // half of rho c_f^2, halved again
-  return fx::mul(fx::limbs(k), r);
+  const fx::Limbs B0 = fx::limbs(q.B[0]), B1 = fx::limbs(q.B[1]), B2 = fx::limbs(q.B[2]);
+  // quarters: gamma p (62 - ee; gamma > 1 in 62 - egam), the squares (62 - 2 eb)
+  fx::i64 a = fx::mul(fx::limbs(q.p), gamma) << egam;
+  fx::i64 bn = fx::mul(B0, B0), bt = fx::fma64(B1, B1, fx::mul(B2, B2));
+  if (bn < 0) bn = 0;  // truncation (fma64)
+  if (bt < 0) bt = 0;
+  const int sh = w.ee - 2 * w.eb;  // >= 1
+  // shifted up by n: a, b_n and b_t below 2^59 each, their sum below 2^61
+  const int na = __clzll(a) - 5, nb = __clzll(bn + bt) - 5 + sh;
+  const int n = na < nb ? (na > 0 ? na : 0) : (nb > 0 ? nb : 0);
+  a <<= n;
+  bn = n < sh ? shr(bn, sh - n) : bn << (n - sh);
+  bt = n < sh ? shr(bt, sh - n) : bt << (n - sh);
+  const fx::Limbs d = fx::limbs(a - bn), t = fx::limbs(bt);
+  const fx::i64 disc = fx::fma64(t, fx::limbs(bt + 2 * (a + bn)), fx::sqr(d));
+  const fx::i64 k = a + bn + bt + fx::sqrt_fixed(disc << 2);  // half of rho c_f^2, halved again
+  return fx::mul(fx::limbs(k >> n), r);
 }
 
 // LLF or HLL from the conserved traces in normal-first order (rho, m, E, B),

@@ -115,3 +115,27 @@ def test_mhd_lifting_cancels_before_it_is_rounded(N, n):
         size = max(size, float(n[r] * abs(D[0, 1]) * np.abs(mr).max()))
     rms = float(np.sqrt(np.mean((got.reshape(ref.shape) - ref) ** 2)))
     assert rms <= 2.0 ** -55 * size, rms / size
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("sf", ["llf", "hll"])
+@pytest.mark.parametrize("field", [(1.0, 0.0, 0.0), (1.29, 1e-3, 0.0), (0.0, 0.0, 1.0), (1e-4, 1e-5, 0.0)])
+@pytest.mark.parametrize("flow", [(3.0, 0.3, 0.3), (30.0, 3.0, 3.0), (300.0, 30.0, 30.0),
+                                  (1000.0, 100.0, 100.0), (0.3, 3.0, 0.0)])
+def test_fast_speed_where_kinetic_energy_dominates(sf, field, flow):
+    # p = 1, so the energy is up to 1e6 p; B = 1.29: sound and Alfven speeds
+    # nearly equal, where the discriminant of the fast speed nearly vanishes.
+    # Velocities vary by 30%, so nothing cancels by more than a factor of ten.
+    # lambda = |v_n| + c_f carries the pressure's error 2^-53 E/p times
+    # c_f/(2 lambda): below 2e-13 for every flow here
+    torch = _gpu()
+    N, n = 3, (4, 3, 3)
+    ne, P = 36, 64
+    rng = np.random.default_rng(5)
+    rho, p = np.ones((ne, P)), rng.uniform(0.99, 1.01, (ne, P))
+    v = np.array(flow)[:, None, None] * (1.0 + 0.3 * rng.uniform(-1, 1, (3, ne, P)))
+    u = _mhd(rho, v, p, np.array(field)[:, None, None] * np.ones((3, ne, P)))
+    got, ref = _rhs(torch, "mhd", 3, N, n, "central", sf, u)
+    size = np.abs(ref).max(axis=2)
+    err = np.abs(got - ref).max(axis=2) / np.where(size > 0, size, 1.0)
+    assert err.max() <= BAR, err.max(axis=0)

@@ -133,6 +133,40 @@ __device__ __forceinline__ void pp_line_of(int dir, int node, int& l, int& i) {
   }
 }
 
+// The largest of at(n) over the nodes n of the D lines through a node. The
+// integer kernels hold an element's values in units of its largest ones, which
+// serves a node as long as its lines reach within 2^kCrossBits of them (what it
+// sums comes from these lines); elements with other nodes take the FP64 form.
+// Lines of zeros are exact: sums that saw nothing but zeros are set to zero.
+constexpr unsigned kCrossBits = 6;
+template <int D, int N, typename F>
+__device__ __forceinline__ unsigned cross_max(int node, const F& at) {
+  unsigned m = 0;
+#pragma unroll 1
+  for (int dir = 0; dir < D; ++dir) {
+    int l, i;
+    pp_line_of<D, N>(dir, node, l, i);
+#pragma unroll 1
+    for (int b = 0; b <= N; ++b) {
+      const unsigned k = at(line_node_rt<D, N>(dir, l, b));
+      m = k > m ? k : m;
+    }
+  }
+  return m;
+}
+// whether the key (high word) `most` of an element leaves one of `some` too far
+// below
+__device__ __forceinline__ bool cross_far(unsigned most, unsigned some) {
+  return some != 0u && most - some > (kCrossBits << 20);
+}
+// Energies: units 2^E serve a node whose energy density has the key `least` if
+// it lies at most 2^kSpreadBits below (of which up to 7 are the powers of two
+// that a uniform flow's units exceed its energy by)
+constexpr int kSpreadBits = 10;
+__device__ __forceinline__ bool energy_far(int E, unsigned least) {
+  return E - fx::exp_above(least) > kSpreadBits;
+}
+
 template <int D, int N, typename R, int VF, int EPB>
 __device__ __forceinline__ void volume_direction(int dir, R (*sp)[3 + 2 * D][Shape<D, N>::P],
                                                  R (*sa)[D + 2][Shape<D, N>::P], int el, int l,

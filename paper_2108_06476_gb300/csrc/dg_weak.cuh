@@ -7,8 +7,10 @@
 // B)_aa, M_00 = -liftL/2 and M_NN = -liftR/2. So each node's flux is evaluated
 // once per direction instead of once per pair, and what remains is the
 // product with M, in 64-bit fixed point like the pair fluxes of dg_fixed.cuh
-// (same rates, same per-element scales; elements with non-finite values take
-// FP64).
+// (same rates, same per-element scales). Elements with non-finite values, with
+// nodes whose energy lies far below the element's largest, or whose lines hold
+// far smaller momenta or velocities than the element (cross_far, energy_far)
+// take FP64.
 //
 // One thread per node, its primitives and sums in registers, the fluxes of one
 // direction in shared memory. 32^3 N = 4: rhs 2.11 ms with a pair flux per pair
@@ -30,7 +32,7 @@ struct WeakLaunch {
 // exponents of an element: |m_k| < 2^em, |v_k| < 2^ev, |E + p| < 2^eh, fluxes
 // of momentum below 2^ef
 struct WeakScale {
-  int em, ev, eh, ef, k, moves, ok;
+  int em, ev, eh, ef, k, ok;
 };
 
 template <int D, int N, int EPB>
@@ -42,7 +44,8 @@ __global__ void __launch_bounds__(WeakLaunch<D, N>::THREADS)
   __shared__ fx::Limbs s_m[D][NP][NP + 1];    // M, format 62 - ed
   __shared__ double s_m64[D][NP][NP + 1];
   __shared__ double s_lift[2][D];             // left, right
-  __shared__ unsigned s_key[EPB][4];          // |m|, |v|, |E + p|, |p|
+  __shared__ unsigned s_key[EPB][7];          // most |m|, |v|, |E + p|, |p|; least E, |m|, |v|
+  __shared__ int s_far[EPB];
   __shared__ int s_left[EPB][D];
   fx::i64* sf = reinterpret_cast<fx::i64*>(dg_smem);  // [el][NV][P]
   const int e0 = blockIdx.x * EPB;
@@ -79,17 +82,18 @@ __global__ void __launch_bounds__(WeakLaunch<D, N>::THREADS)
   }
   if (t < count) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s_key[t][k] = 0u;
+    for (int k = 0; k < 7; ++k) s_key[t][k] = k < 4 ? 0u : 0xffffffffu;
+    s_far[t] = 0;
     for (int k = 0; k < D; ++k) s_left[t][k] = neighbour32(g, e0 + t, k, -1);
   }
   __syncthreads();
   double rr;
   const Prim<double, D> q = prim_rcp<D>(c, g.gm1, rr);
   const double H = c[NV - 1] + q.p;
+  unsigned km = 0, kv = 0;  // of the node
   {
     const unsigned bad = in ? prim_check(q) : 0u;
     if (bad) atomicOr(err, bad);
-    unsigned km = 0, kv = 0;
 #pragma unroll
     for (int k = 0; k < D; ++k) {
       const unsigned hm = (unsigned)__double2hiint(c[1 + k]) & 0x7fffffffu;
@@ -106,30 +110,49 @@ __global__ void __launch_bounds__(WeakLaunch<D, N>::THREADS)
       const unsigned b = __reduce_max_sync(0xffffffffu, mine ? kv : 0u);
       const unsigned h = __reduce_max_sync(0xffffffffu, mine ? kh : 0u);
       const unsigned p = __reduce_max_sync(0xffffffffu, mine ? kp : 0u);
+      const unsigned le = __reduce_min_sync(
+          0xffffffffu, mine ? (unsigned)__double2hiint(c[NV - 1]) : 0xffffffffu);
+      const unsigned lm = __reduce_min_sync(0xffffffffu, mine ? km : 0xffffffffu);
+      const unsigned lv = __reduce_min_sync(0xffffffffu, mine ? kv : 0xffffffffu);
       if ((t & 31) == 0) {
         atomicMax(&s_key[ek][0], a);
         atomicMax(&s_key[ek][1], b);
         atomicMax(&s_key[ek][2], h);
         atomicMax(&s_key[ek][3], p);
+        atomicMin(&s_key[ek][4], le);
+        atomicMin(&s_key[ek][5], lm);
+        atomicMin(&s_key[ek][6], lv);
       }
     }
   }
   __syncthreads();
   WeakScale w;
+  bool cross;
   {
-    const unsigned km = s_key[el][0], kv = s_key[el][1], kh = s_key[el][2], kp = s_key[el][3];
-    w.em = fx::exp_above(km);
-    w.ev = fx::exp_above(kv);
+    const unsigned mm = s_key[el][0], mv = s_key[el][1], kh = s_key[el][2], kp = s_key[el][3];
+    w.em = fx::exp_above(mm);
+    w.ev = fx::exp_above(mv);
     w.eh = fx::exp_above(kh);
     w.ef = fx::exp_above(kp) + 1;
     if (w.em < -300) w.em = -300;  // nothing moves
     if (w.ev < -300) w.ev = -300;
     if (w.ef < w.em + w.ev + 1) w.ef = w.em + w.ev + 1;
-    w.k = w.ef - w.em - w.ev;
-    w.moves = kv != 0u;
+    w.k = w.ef - w.em - w.ev < 63 ? w.ef - w.em - w.ev : 63;
     const unsigned hi = (fx::kBias + 150u) << 20, lo = (fx::kBias - 150u) << 20;
-    w.ok = km < hi && kv < hi && kh < hi && kp < hi && kh > lo && kp > lo && ed <= 300 &&
-           ed >= -300;
+    w.ok = mm < hi && mv < hi && kh < hi && kp < hi && kh > lo && kp > lo && ed <= 300 &&
+           ed >= -300 && !energy_far(w.ef > w.eh ? w.ef : w.eh, s_key[el][4]);
+    cross = w.ok && (mm - s_key[el][5] > (kCrossBits << 20) || mv - s_key[el][6] > (kCrossBits << 20));
+  }
+  if (__syncthreads_or(in && cross)) {  // some node may lie too far below
+    uint2* sk = reinterpret_cast<uint2*>(sf + el * NV * P);
+    if (in) sk[node] = make_uint2(km, kv);
+    __syncthreads();
+    if (in && cross &&
+        (cross_far(s_key[el][0], cross_max<D, N>(node, [&](int n) { return sk[n].x; })) ||
+         cross_far(s_key[el][1], cross_max<D, N>(node, [&](int n) { return sk[n].y; }))))
+      s_far[el] = 1;
+    __syncthreads();
+    if (s_far[el]) w.ok = 0;
   }
   // fixed point: m (63 - em), v (63 - ev), p (62 - ef), E + p (63 - eh)
   fx::i64 xm[D], xv[D], xp = 0, xh = 0, acc[NV];
@@ -151,8 +174,7 @@ __global__ void __launch_bounds__(WeakLaunch<D, N>::THREADS)
     xh = __double_as_longlong(H);
   }
 #pragma unroll
-  for (int v = 0; v < NV; ++v)
-    acc[v] = w.ok && (w.moves || (v > 0 && v <= D)) ? D * NP : 0;  // truncation, see fma64
+  for (int v = 0; v < NV; ++v) acc[v] = w.ok ? D * NP : 0;  // truncation, see fma64
 #pragma unroll
   for (int dir = 0; dir < D; ++dir) {
     int l, a;
@@ -208,9 +230,11 @@ __global__ void __launch_bounds__(WeakLaunch<D, N>::THREADS)
   double val[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v)
-    val[v] = w.ok ? fx::to_double_int(acc[v],
-                                      ed + (v == 0 ? w.em : v <= D ? w.ef : w.eh + w.ev) - 60)
-                  : __longlong_as_double(acc[v]);
+    val[v] = !w.ok ? __longlong_as_double(acc[v])
+             : acc[v] == D * NP  // nothing but zeros
+                 ? 0.0
+                 : fx::to_double_int(acc[v],
+                                     ed + (v == 0 ? w.em : v <= D ? w.ef : w.eh + w.ev) - 60);
   const long long base = g.nelem * LINES;
 #pragma unroll
   for (int dir = 0; dir < D; ++dir) {

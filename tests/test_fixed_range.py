@@ -139,3 +139,52 @@ def test_fast_speed_where_kinetic_energy_dominates(sf, field, flow):
     size = np.abs(ref).max(axis=2)
     err = np.abs(got - ref).max(axis=2) / np.where(size > 0, size, 1.0)
     assert err.max() <= BAR, err.max(axis=0)
+
+
+def _corner(eq, d, N, ne, kind, rng, factor=1e8):
+    # random states with one corner node of every element, or all the others,
+    # far away; and the nodes whose lines do not reach that corner or a face
+    P = (N + 1) ** d
+    rho, p = rng.uniform(0.8, 1.2, (2, ne, P))
+    v, B = rng.uniform(-0.3, 0.3, (d, ne, P)), rng.uniform(-0.5, 0.5, (3, ne, P))
+    last = P - 1
+    if kind == "pressure":
+        p[:, last] *= factor
+    if kind == "density":  # the same momentum
+        rho[:, last] *= factor
+        v[:, :, last] /= factor
+    if kind == "velocity":
+        v[:, :, :last] /= factor
+    if kind == "field":
+        B[:, :, :last] /= factor
+    if kind == "all":
+        rho[:, last] *= factor
+        p[:, last] *= factor
+    if kind == "rest":  # exact zeros in place of small values
+        v[:, :, :last] = 0.0
+    if kind == "vacuum field":
+        B[:, :, :last] = 0.0
+    i = np.arange(P)
+    inner = np.ones(P, bool)
+    for k in range(d):
+        c = i // (N + 1) ** k % (N + 1)
+        inner &= (c != 0) & (c != N)
+    return (_mhd(rho, v, p, B) if eq == "mhd" else _euler(rho, v, p)), inner
+
+
+def _check_corner(torch, eq, d, N, n, vf, sf, kind):
+    ne = int(np.prod(n))
+    u, inner = _corner(eq, d, N, ne, kind, np.random.default_rng([d, N, 3]))
+    got, ref = _rhs(torch, eq, d, N, n, vf, sf, u)
+    size = np.abs(ref[:, :, inner]).max(axis=(0, 2))
+    err = np.abs(got - ref)[:, :, inner].max(axis=(0, 2))
+    assert (err[size == 0.0] == 0.0).all(), err
+    assert (err <= BAR * size).all(), err / np.where(size > 0, size, 1.0)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,N,n", [(2, 2, (26, 25)), (2, 5, (25, 26)), (3, 2, (9, 9, 8)),
+                                   (3, 3, (9, 9, 8)), (3, 4, (9, 9, 8)), (3, 7, (9, 9, 8))])
+@pytest.mark.parametrize("kind", ["pressure", "density", "velocity", "all", "rest"])
+def test_weak_form_far_from_a_strong_corner(d, N, n, kind):
+    _check_corner(_gpu(), "euler", d, N, n, "central", "hll", kind)

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(WeakLaunch<D, N>::THREADS)
   __shared__ fx::Limbs s_m[D][NP][NP + 1];    // M, format 62 - ed
   __shared__ double s_m64[D][NP][NP + 1];
   __shared__ double s_lift[2][D];             // left, right
-  __shared__ unsigned s_key[EPB][7];          // most |m|, |v|, |E + p|, |p|; least E, |m|, |v|
+  __shared__ unsigned s_key[EPB][4];          // |m|, |v|, |E + p|, |p|
   __shared__ int s_far[EPB];
   __shared__ int s_left[EPB][D];
   fx::i64* sf = reinterpret_cast<fx::i64*>(dg_smem);  // [el][NV][P]
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(WeakLaunch<D, N>::THREADS)
   }
   if (t < count) {
 #pragma unroll
-    for (int k = 0; k < 7; ++k) s_key[t][k] = k < 4 ? 0u : 0xffffffffu;
+    for (int k = 0; k < 4; ++k) s_key[t][k] = 0u;
     s_far[t] = 0;
     for (int k = 0; k < D; ++k) s_left[t][k] = neighbour32(g, e0 + t, k, -1);
   }
@@ -110,24 +110,17 @@ __global__ void __launch_bounds__(WeakLaunch<D, N>::THREADS)
       const unsigned b = __reduce_max_sync(0xffffffffu, mine ? kv : 0u);
       const unsigned h = __reduce_max_sync(0xffffffffu, mine ? kh : 0u);
       const unsigned p = __reduce_max_sync(0xffffffffu, mine ? kp : 0u);
-      const unsigned le = __reduce_min_sync(
-          0xffffffffu, mine ? (unsigned)__double2hiint(c[NV - 1]) : 0xffffffffu);
-      const unsigned lm = __reduce_min_sync(0xffffffffu, mine ? km : 0xffffffffu);
-      const unsigned lv = __reduce_min_sync(0xffffffffu, mine ? kv : 0xffffffffu);
       if ((t & 31) == 0) {
         atomicMax(&s_key[ek][0], a);
         atomicMax(&s_key[ek][1], b);
         atomicMax(&s_key[ek][2], h);
         atomicMax(&s_key[ek][3], p);
-        atomicMin(&s_key[ek][4], le);
-        atomicMin(&s_key[ek][5], lm);
-        atomicMin(&s_key[ek][6], lv);
       }
     }
   }
   __syncthreads();
   WeakScale w;
-  bool cross;
+  bool low, weak;
   {
     const unsigned mm = s_key[el][0], mv = s_key[el][1], kh = s_key[el][2], kp = s_key[el][3];
     w.em = fx::exp_above(mm);
@@ -140,16 +133,19 @@ __global__ void __launch_bounds__(WeakLaunch<D, N>::THREADS)
     w.k = w.ef - w.em - w.ev < 63 ? w.ef - w.em - w.ev : 63;
     const unsigned hi = (fx::kBias + 150u) << 20, lo = (fx::kBias - 150u) << 20;
     w.ok = mm < hi && mv < hi && kh < hi && kp < hi && kh > lo && kp > lo && ed <= 300 &&
-           ed >= -300 && !energy_far(w.ef > w.eh ? w.ef : w.eh, s_key[el][4]);
-    cross = w.ok && (mm - s_key[el][5] > (kCrossBits << 20) || mv - s_key[el][6] > (kCrossBits << 20));
+           ed >= -300;
+    low = in && w.ok &&
+          energy_far(w.ef > w.eh ? w.ef : w.eh, (unsigned)__double2hiint(c[NV - 1]));
+    weak = in && w.ok && (mm - km > (kCrossBits << 20) || mv - kv > (kCrossBits << 20));
   }
-  if (__syncthreads_or(in && cross)) {  // some node may lie too far below
+  if (__syncthreads_or(low || weak)) {  // some node may lie too far below
     uint2* sk = reinterpret_cast<uint2*>(sf + el * NV * P);
     if (in) sk[node] = make_uint2(km, kv);
     __syncthreads();
-    if (in && cross &&
-        (cross_far(s_key[el][0], cross_max<D, N>(node, [&](int n) { return sk[n].x; })) ||
-         cross_far(s_key[el][1], cross_max<D, N>(node, [&](int n) { return sk[n].y; }))))
+    if (low ||
+        (weak &&
+         (cross_far(s_key[el][0], cross_max<D, N>(node, [&](int n) { return sk[n].x; })) ||
+          cross_far(s_key[el][1], cross_max<D, N>(node, [&](int n) { return sk[n].y; })))))
       s_far[el] = 1;
     __syncthreads();
     if (s_far[el]) w.ok = 0;

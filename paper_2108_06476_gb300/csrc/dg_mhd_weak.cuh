@@ -10,8 +10,10 @@
 // the two cancel (added afterwards in FP64, the error of smooth data was up to
 // 2.2 times that of lift (F* - f(u_i)), at a supersonic outflow 25 times). A
 // face value beyond the element's units is added in FP64. Elements with non-finite
-// values, non-positive densities or densities spread over more than 2^6 take
-// the same steps in FP64.
+// values, non-positive densities, densities spread over more than 2^6, nodes
+// whose energy lies far below the element's units, or whose lines hold far
+// smaller momenta, velocities or fields than the element (energy_far,
+// cross_far), take the same steps in FP64.
 //
 // Included by dg_mhd.cu. 48^3 N = 3, rhs only: 2.68 ms in FP64, 0.98 here; HLL
 // faces 1.81 and 0.57 ms, LLF 1.55 and 0.51.
@@ -20,7 +22,6 @@
 // |m_k| < 2^em, |v_k| < 2^ev, |B_k| < 2^eb, energies below 2^(ee - 1), 1/rho < 2^e1
 struct MWScale {
   int em, ev, eb, ee, e1;
-  int moves, field;  // some momentum, some magnetic field is not zero
   int ok;
 };
 
@@ -40,8 +41,6 @@ __device__ __forceinline__ MWScale mw_scale(const unsigned* key, double gm1, boo
   const unsigned hi = (fx::kBias + 150u) << 20, lo = (fx::kBias - 150u) << 20;
   w.ok = usable && rmax < hi && rmin > lo && rmax - rmin < (6u << 20) && km < hi && kb < hi &&
          ke < hi && ke > lo && kv < hi;
-  w.moves = km != 0u;
-  w.field = kb != 0u;
   const int eg = fx::exp_above((unsigned)__double2hiint(gm1));
   w.em = fx::exp_above(km);
   w.eb = fx::exp_above(kb);
@@ -63,6 +62,11 @@ __device__ __forceinline__ MWScale mw_scale(const unsigned* key, double gm1, boo
 // of 8 bits loses nothing (N = 1 and 2, where the rows are few-bit numbers).
 __device__ __forceinline__ int mw_cut(fx::Limbs k) {
   return (k.h != 0) + (k.l != 0) + (((k.h & 0xffffff) != 0) + (k.l != 0)) * 65536;
+}
+
+// a sum's start from mw_cut over its products (v: variable, kMV: div B)
+__device__ __forceinline__ int mw_start(int cut, int v) {
+  return ((v == 0 || v == kMV ? cut >> 16 : cut & 0xffff) + 1) / 2;
 }
 
 __device__ __forceinline__ fx::i64 shr(fx::i64 a, int n) { return a >> (n < 63 ? n : 63); }
@@ -222,6 +226,7 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
   __shared__ fx::Limbs s_liftx[2][3];                 // 62 - ed
   __shared__ int s_cut[3][NP];  // mw_cut over a row and its lifting
   __shared__ unsigned s_key[EPB][6];                  // see mw_scale
+  __shared__ int s_far[EPB];
   const int e0 = blockIdx.x * EPB;
   const int count = (int)g.nelem - e0 < EPB ? (int)g.nelem - e0 : EPB;
   const double sc = fz.k ? *fz.dt : 1.0;
@@ -256,8 +261,9 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
     s_liftx[1][t] = fx::limbs(fx::half_fixed(s_lift[1][t], ed));
   }
   if (t < count) {
-    s_key[t][0] = s_key[t][2] = s_key[t][3] = s_key[t][4] = s_key[t][5] = 0u;
-    s_key[t][1] = 0xffffffffu;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) s_key[t][k] = k == 1 ? 0xffffffffu : 0u;
+    s_far[t] = 0;
   }
   const double rr = rcp(c[0]);
   const double vel[3] = {c[1] * rr, c[2] * rr, c[3] * rr};
@@ -279,9 +285,9 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
     s_m[dir][a][a] = fx::limbs(x);
     s_cut[dir][a] = cut + mw_cut(fx::limbs(x));
   }
+  unsigned km = 0, kb = 0, kv = 0;  // of the node
   {
     auto hw = [](double x) { return (unsigned)__double2hiint(x); };
-    unsigned km = 0, kb = 0, kv = 0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       kv = max(kv, hw(vel[k]) & 0x7fffffffu);
@@ -309,7 +315,30 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
     }
   }
   __syncthreads();
-  const MWScale w = mw_scale(s_key[el], g.gm1, ed <= 300 && ed >= -300);
+  MWScale w = mw_scale(s_key[el], g.gm1, ed <= 300 && ed >= -300);
+  {
+    const unsigned mm = s_key[el][2], mb = s_key[el][3], mv = s_key[el][5];
+    const bool low = in && w.ok && energy_far(w.ee, (unsigned)__double2hiint(c[4]));
+    const bool weak = in && w.ok && (mm - km > (kCrossBits << 20) ||
+                                     (mv - kv) + (mb - kb) > (kCrossBits << 20));
+    if (__syncthreads_or(low || weak)) {  // some node may lie too far below
+      uint3* sk = reinterpret_cast<uint3*>(sf + el * kMV * P);
+      if (in) sk[node] = make_uint3(km, kv, kb);
+      __syncthreads();
+      bool far = low;
+      if (weak) {
+        const unsigned cm = cross_max<3, N>(node, [&](int n) { return sk[n].x; });
+        const unsigned cv = cross_max<3, N>(node, [&](int n) { return sk[n].y; });
+        const unsigned cb = cross_max<3, N>(node, [&](int n) { return sk[n].z; });
+        // the induction rows hold products of v and B
+        far = far || cross_far(mm, cm) || cross_far(mv, cv) || cross_far(mb, cb) ||
+              (cv && cb && (mv - cv) + (mb - cb) > (kCrossBits << 20));
+      }
+      if (far) s_far[el] = 1;
+      __syncthreads();
+      if (s_far[el]) w.ok = 0;
+    }
+  }
   MWNode q;
   MState s;
   unsigned bad = 0;
@@ -321,8 +350,7 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
   }
   if (in && bad) atomicOr(err, bad);
   fx::i64 acc[kMV + 1];
-  // truncation (fma64): the sums start from what their products lose on
-  // average, those of zero fluxes from zero
+  // truncation (fma64): the sums start from what their products lose on average
   int cut = 0;
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
@@ -332,8 +360,7 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
   }
 #pragma unroll
   for (int v = 0; v <= kMV; ++v) {
-    const bool some = v == 0 || v == 4 ? w.moves : (v <= 3 ? true : (v < kMV ? w.moves && w.field : w.field));
-    acc[v] = w.ok && some ? ((v == 0 || v == kMV ? cut >> 16 : cut & 0xffff) + 1) / 2 : 0;
+    acc[v] = w.ok ? mw_start(cut, v) : 0;
   }
 #pragma unroll
   for (int dir = 0; dir < 3; ++dir) {
@@ -422,7 +449,9 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
   double val[kMV + 1];
 #pragma unroll
   for (int v = 0; v <= kMV; ++v)
-    val[v] = w.ok ? fx::to_double_int(acc[v], ed + unit(v) - 60) : __longlong_as_double(acc[v]);
+    val[v] = !w.ok                       ? __longlong_as_double(acc[v])
+             : acc[v] == mw_start(cut, v) ? 0.0  // nothing but zeros
+                                          : fx::to_double_int(acc[v], ed + unit(v) - 60);
   for (int dir = 0; late && dir < 3; ++dir, late >>= 9) {
     int l, i;
     line_of<N>(dir, node, l, i);

@@ -188,3 +188,12 @@ def _check_corner(torch, eq, d, N, n, vf, sf, kind):
 @pytest.mark.parametrize("kind", ["pressure", "density", "velocity", "all", "rest"])
 def test_weak_form_far_from_a_strong_corner(d, N, n, kind):
     _check_corner(_gpu(), "euler", d, N, n, "central", "hll", kind)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,n", [(2, (3, 2, 2)), (2, (9, 9, 8)), (3, (3, 2, 2)), (3, (9, 9, 8)),
+                                 (4, (9, 9, 8)), (7, (2, 2, 2))])
+@pytest.mark.parametrize("kind", ["pressure", "density", "velocity", "field", "all", "rest",
+                                  "vacuum field"])
+def test_mhd_weak_form_far_from_a_strong_corner(N, n, kind):
+    _check_corner(_gpu(), "mhd", 3, N, n, "central", "hll", kind)

@@ -22,9 +22,9 @@ constexpr int kCSlots = 8 + 9;  // r, ln rho, e, ln e, p, v[3] and (J a^r)_n/2 b
 __device__ __forceinline__ CScale cfx_scale(const unsigned* key, const int* cb) {
   CScale s;
   s.u = fx::element_scale(key, cb);
-  s.eg = fx::exp_above(key[6]);
+  s.eg = fx::exp_above(key[8]);
   const unsigned lo = (fx::kBias - 150u) << 20, hi = (fx::kBias + 150u) << 20;
-  if (!(key[6] < hi && key[6] > lo)) s.u.ok = 0;
+  if (!(key[8] < hi && key[8] > lo)) s.u.ok = 0;
   return s;
 }
 
@@ -154,13 +154,13 @@ __global__ void __launch_bounds__((SPREAD ? 3 : 1) * CFxLaunch<N>::threads(EPB),
   __shared__ fx::Limbs s_d[kNPMax][kNPMax];
   __shared__ double s_d64[kNPMax][kNPMax];
   __shared__ CScale s_scale[EPB];
-  __shared__ unsigned s_key[EPB][7];
+  __shared__ unsigned s_key[EPB][9];  // those of FxShared, then the metric vectors'
   const int e0 = blockIdx.x * EPB;
   const int count = (int)g.nelem - e0 < EPB ? (int)g.nelem - e0 : EPB;
   const int t = threadIdx.x;
   if (t < count) {
     fx_clear_key(s_key[t]);
-    s_key[t][6] = 0u;
+    s_key[t][8] = 0u;
   }
   // |Dt[0][1]| is the largest coefficient (fx_table_exponent)
   const int ed = fx::exp_above((unsigned)__double2hiint(tb.Ds[0][1]) & 0x7fffffffu);
@@ -203,13 +203,22 @@ __global__ void __launch_bounds__((SPREAD ? 3 : 1) * CFxLaunch<N>::threads(EPB),
       const bool mine = in && el == ek;
       fx_merge_keys(k, mine, s_key[ek]);
       const unsigned m = __reduce_max_sync(0xffffffffu, mine ? kg : 0u);
-      if ((t & 31) == 0) atomicMax(&s_key[ek][6], m);
+      if ((t & 31) == 0) atomicMax(&s_key[ek][8], m);
     }
   }
   if (bad) atomicOr(err, bad);
   __syncthreads();
-  if (t < count) s_scale[t] = cfx_scale(s_key[t], cb);
-  __syncthreads();
+  bool slow = false;
+  if (t < count) {
+    s_scale[t] = cfx_scale(s_key[t], cb);
+    if (energy_far(s_scale[t].u.em, s_key[t][7])) s_scale[t].u.ok = 0;
+    slow = fx_slow(s_key[t], s_scale[t].u);
+  }
+  if (__syncthreads_or(slow)) {
+    fx_slow_elements<3, N>(count, dg_smem, ELEM, 3, s_key,
+                           [&](int el) { s_scale[el].u.ok = 0; });
+    __syncthreads();
+  }
   for (int i = t; i < count * P; i += blockDim.x) {
     const int el = i / P, pl = fx_place<3, N>(i % P);
     const CScale sc = s_scale[el];
@@ -241,7 +250,7 @@ __global__ void __launch_bounds__((SPREAD ? 3 : 1) * CFxLaunch<N>::threads(EPB),
     // the units by which truncated products fall short (fx_stage_node)
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      sx[(kCSlots + v) * P] = sc.u.ok && (sc.u.moves || (v > 0 && v < 4)) ? 3 * N : 0;
+      sx[(kCSlots + v) * P] = sc.u.ok ? 3 * N : 0;
       if (SPREAD) sx[(kCSlots + 5 + v) * P] = sx[(kCSlots + 10 + v) * P] = 0;
     }
   }
@@ -284,7 +293,7 @@ __global__ void __launch_bounds__((SPREAD ? 3 : 1) * CFxLaunch<N>::threads(EPB),
         fx::i64 a = sa[v * P];
         if (SPREAD) a += sa[(5 + v) * P] + sa[(10 + v) * P];
         const int x = v == 0 ? sc.u.er + sc.u.ev - 58 : v < 4 ? sc.u.em - 59 : sc.u.em + sc.u.ev - 58;
-        val[v] = fx::to_double_int(a, ed + sc.eg + x);
+        val[v] = a == 3 * N ? 0.0 : fx::to_double_int(a, ed + sc.eg + x);  // 3 N: only zeros
       } else {
         val[v] = __longlong_as_double(sa[v * P]);
         if (SPREAD)
@@ -332,10 +341,10 @@ __device__ __forceinline__ bool curved_face_fixed(const double* cl, const double
   unsigned bad = 0;
   const FxPrim<3> L = fx_prim<3>(cl, g, bad), R = fx_prim<3>(cr, g, bad);
   const FxKeys a = fx_keys<3>(L), b = fx_keys<3>(R);
-  unsigned key[7] = {max(a.r, b.r), min(a.r, b.r), max(a.e, b.e), min(a.e, b.e),
-                     max(a.v, b.v), max(a.p, b.p), 0u};
+  unsigned key[9] = {max(a.r, b.r), min(a.r, b.r), max(a.e, b.e), min(a.e, b.e),
+                     max(a.v, b.v), max(a.p, b.p), 0u, 0u, 0u};
 #pragma unroll
-  for (int k = 0; k < 3; ++k) key[6] = max(key[6], (unsigned)__double2hiint(gv[k]) & 0x7fffffffu);
+  for (int k = 0; k < 3; ++k) key[8] = max(key[8], (unsigned)__double2hiint(gv[k]) & 0x7fffffffu);
   int cb[2];
   fx::scale_bits(g.gm1, cb);
   const CScale sc = cfx_scale(key, cb);

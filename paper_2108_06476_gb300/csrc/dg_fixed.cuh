@@ -113,7 +113,6 @@ struct Scale {
   int er, ev, ee, em;
   int kv, km, s;  // alignments: v.v to e, mass flux to momentum flux, and
                   // the excess of the bound of rho e over em
-  int moves;      // some velocity is not zero
   int ok;         // 0: the element takes the FP64 form
 };
 
@@ -151,7 +150,6 @@ DG_FX_FN Scale element_scale(const unsigned* key, const int* c) {
   s.kv = s.ee - 2 * s.ev - 2;
   s.km = s.em - s.er - 2 * s.ev - 2;
   s.s = s.er + s.ee - s.em;
-  s.moves = vmax != 0u;
   const unsigned lo = (kBias - 150u) << 20, hi = (kBias + 150u) << 20;
   s.ok = rmax < hi && rmin > lo && emax < hi && emin > lo && vmax < hi && pmax < hi &&
          rmax - rmin < (6u << 20) && emax - emin < (6u << 20) &&

@@ -78,7 +78,7 @@ template <int D, int MAXE>
 struct FxShared {
   fx::Limbs Ds[D][kNPMax][kNPMax];  // format 62 - ed
   fx::Scale scale[MAXE];
-  unsigned key[MAXE][6];
+  unsigned key[MAXE][8];
   int left[MAXE][D];
   int ed;
 };
@@ -181,6 +181,7 @@ __device__ __forceinline__ int fx_table_exponent(const Tables<double>& tb) {
 template <int D>
 struct FxPrim {
   double rho, e, p, v[D];
+  unsigned E;  // high word of the total energy
 };
 template <int D>
 __device__ __forceinline__ FxPrim<D> fx_prim(const double* c, const Geom& g, unsigned& bad) {
@@ -197,12 +198,13 @@ __device__ __forceinline__ FxPrim<D> fx_prim(const double* c, const Geom& g, uns
   const double i = fma(-0.5, mv, c[D + 1]);  // rho e
   q.p = r.p = g.gm1 * i;
   r.e = i * rr;
+  r.E = (unsigned)__double2hiint(c[D + 1]);
   bad |= prim_check(q);
   return r;
 }
 
 struct FxKeys {
-  unsigned r, e, v, p;
+  unsigned r, e, v, p, E;
 };
 template <int D>
 __device__ __forceinline__ FxKeys fx_keys(const FxPrim<D>& q) {
@@ -210,6 +212,7 @@ __device__ __forceinline__ FxKeys fx_keys(const FxPrim<D>& q) {
   k.r = (unsigned)__double2hiint(q.rho);
   k.e = (unsigned)__double2hiint(q.e);
   k.p = (unsigned)__double2hiint(q.p);
+  k.E = q.E;
   k.v = 0;
 #pragma unroll
   for (int j = 0; j < D; ++j) {
@@ -219,6 +222,8 @@ __device__ __forceinline__ FxKeys fx_keys(const FxPrim<D>& q) {
   return k;
 }
 // the keys of one element over the warp's lanes `mine`, by lane 0 into key
+// (LEAST: the least velocity and energy too)
+template <bool LEAST = true>
 __device__ __forceinline__ void fx_merge_keys(const FxKeys& k, bool mine, unsigned* key) {
   const unsigned a = __reduce_max_sync(0xffffffffu, mine ? k.r : 0u);
   const unsigned b = __reduce_min_sync(0xffffffffu, mine ? k.r : 0xffffffffu);
@@ -226,6 +231,11 @@ __device__ __forceinline__ void fx_merge_keys(const FxKeys& k, bool mine, unsign
   const unsigned d = __reduce_min_sync(0xffffffffu, mine ? k.e : 0xffffffffu);
   const unsigned v = __reduce_max_sync(0xffffffffu, mine ? k.v : 0u);
   const unsigned p = __reduce_max_sync(0xffffffffu, mine ? k.p : 0u);
+  unsigned lv, le;
+  if (LEAST) {
+    lv = __reduce_min_sync(0xffffffffu, mine ? k.v : 0xffffffffu);
+    le = __reduce_min_sync(0xffffffffu, mine ? k.E : 0xffffffffu);
+  }
   if ((threadIdx.x & 31) == 0) {
     atomicMax(&key[0], a);
     atomicMin(&key[1], b);
@@ -233,6 +243,10 @@ __device__ __forceinline__ void fx_merge_keys(const FxKeys& k, bool mine, unsign
     atomicMin(&key[3], d);
     atomicMax(&key[4], v);
     atomicMax(&key[5], p);
+    if (LEAST) {
+      atomicMin(&key[6], lv);
+      atomicMin(&key[7], le);
+    }
   }
 }
 
@@ -258,11 +272,44 @@ __device__ __forceinline__ void fx_stage_node(const FxPrim<D>& q, const fx::Scal
     for (int k = 0; k < D; ++k) sp[(3 + k) * P + pl] = q.v[k];
   }
   // the sums start at +0.0, or at the D N units by which the truncated
-  // products fall short on average; where nothing moves, mass and energy
-  // fluxes are zeros and so are their sums
+  // products fall short on average
 #pragma unroll
-  for (int v = 0; v < NV; ++v)
-    sx[(SL + v) * P + pl] = sc.ok && (sc.moves || (v > 0 && v <= D)) ? D * N : 0;
+  for (int v = 0; v < NV; ++v) sx[(SL + v) * P + pl] = sc.ok ? D * N : 0;
+}
+
+// whether some node of the element is so slow that its lines have to be looked
+// at (fx_slow_node)
+__device__ __forceinline__ bool fx_slow(const unsigned* key, const fx::Scale& sc) {
+  return sc.ok && key[4] - key[6] > (kCrossBits << 20);
+}
+// whether the velocities on the node's lines lie too far below the element's
+// units; at(n): the key of node n's largest component
+template <int D, int N, typename F>
+__device__ __forceinline__ bool fx_slow_node(const unsigned* key, int node, const F& at) {
+  return key[4] - at(node) > (kCrossBits << 20) && cross_far(key[4], cross_max<D, N>(node, at));
+}
+
+// clears the integer form (drop(el)) of elements with a node whose velocities
+// lie too far below the units; v: FP64 slots `at` on of the elements at smem,
+// `stride` bytes apart; by the whole block, between barriers
+template <int D, int N, int K, typename F>
+__device__ __forceinline__ void fx_slow_elements(int count, const unsigned char* smem, int stride,
+                                                 int at, unsigned (*key)[K], const F& drop) {
+  constexpr int P = Shape<D, N>::P;
+  for (int t = threadIdx.x; t < count * P; t += blockDim.x) {
+    const int el = t / P;
+    const double* sv = reinterpret_cast<const double*>(smem + el * stride) + at * P;
+    auto speed = [&](int n) {
+      unsigned k = 0;
+#pragma unroll
+      for (int j = 0; j < D; ++j) {
+        const unsigned h = (unsigned)__double2hiint(sv[j * P + fx_place<D, N>(n)]) & 0x7fffffffu;
+        k = h > k ? h : k;
+      }
+      return k;
+    };
+    if (fx_slow_node<D, N>(key[el], t % P, speed)) drop(el);
+  }
 }
 
 // primitives of the batch's nodes (rho, e, p, v in FP64 slots) and the keys of
@@ -270,7 +317,7 @@ __device__ __forceinline__ void fx_stage_node(const FxPrim<D>& q, const fx::Scal
 template <int D, int N>
 __device__ __forceinline__ unsigned fx_load(const double* __restrict__ u, const Geom& g, int e0,
                                             int count, unsigned char* smem,
-                                            unsigned (*key)[6]) {
+                                            unsigned (*key)[8]) {
   constexpr int P = Shape<D, N>::P, NV = D + 2, ELEM = FxShape<D, N>::ELEM;
   unsigned bad = 0;
   for (int t0 = threadIdx.x & ~31; t0 < count * P; t0 += blockDim.x) {
@@ -299,15 +346,15 @@ __device__ __forceinline__ unsigned fx_load(const double* __restrict__ u, const 
 
 __device__ __forceinline__ void fx_clear_key(unsigned* key) {
   key[0] = key[2] = key[4] = key[5] = 0u;
-  key[1] = key[3] = 0xffffffffu;
+  key[1] = key[3] = key[6] = 0xffffffffu;
+  key[7] = 0x7fefffffu;  // where it is not used it refuses nothing
 }
 
 __device__ __forceinline__ fx::Scale fx_scale(const unsigned* key, const int* c, int ed) {
   fx::Scale sc = fx::element_scale(key, c);
-  if (ed > 300 || ed < -300) sc.ok = 0;
+  if (ed > 300 || ed < -300 || energy_far(sc.em, key[7])) sc.ok = 0;
   return sc;
 }
-
 // the slots of each element's form, in place, by the whole block
 template <int D, int N>
 __device__ __forceinline__ void fx_stage(const Geom& g, int count, unsigned char* smem,
@@ -326,10 +373,11 @@ __device__ __forceinline__ void fx_stage(const Geom& g, int count, unsigned char
   }
 }
 
-// a sum of variable v as a double
-template <int D>
+// a sum of variable v as a double (D N: nothing but zeros)
+template <int D, int N>
 __device__ __forceinline__ double fx_value(fx::i64 a, int v, const fx::Scale& sc, int ed) {
   if (!sc.ok) return __longlong_as_double(a);
+  if (a == D * N) return 0.0;
   return fx::to_double_int(a, ed + (v == 0 ? sc.er + sc.ev - 60 : v <= D ? sc.em - 61
                                                                          : sc.em + sc.ev - 59));
 }
@@ -344,7 +392,7 @@ __device__ __forceinline__ void fx_result(const unsigned char* elem, const fx::S
                 LINES = Shape<D, N>::LINES;
   const fx::i64* sa = reinterpret_cast<const fx::i64*>(elem) + SL * P + fx_place<D, N>(node);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) val[v] = fx_value<D>(sa[v * P], v, sc, ed);
+  for (int v = 0; v < NV; ++v) val[v] = fx_value<D, N>(sa[v * P], v, sc, ed);
   const long long base = (long long)nelem * LINES;
 #pragma unroll
   for (int dir = 0; dir < D; ++dir) {
@@ -421,9 +469,26 @@ __device__ __forceinline__ void fx_batch(double* u, double* __restrict__ du,
       }
       if (bad) atomicOr(err, bad);
 #pragma unroll
-      for (int j = 0; j < NPL; ++j) fx_merge_keys(fx_keys<D>(q[j]), true, sh.key[el]);
+      for (int j = 0; j < NPL; ++j) fx_merge_keys<false>(fx_keys<D>(q[j]), true, sh.key[el]);
       __syncwarp();
-      const fx::Scale sc = fx_scale(sh.key[el], cb, ed);
+      fx::Scale sc = fx_scale(sh.key[el], cb, ed);
+      // each node against the units by itself, in place of the least keys
+      bool low = false, slow = false;
+#pragma unroll
+      for (int j = 0; j < NPL; ++j) {
+        low = low || energy_far(sc.em, q[j].E);
+        slow = slow || sh.key[el][4] - fx_keys<D>(q[j]).v > (kCrossBits << 20);
+      }
+      if (__any_sync(0xffffffffu, sc.ok && (low || slow))) {
+        unsigned* sk = reinterpret_cast<unsigned*>(elem);
+#pragma unroll
+        for (int j = 0; j < NPL; ++j) sk[lane + 32 * j] = fx_keys<D>(q[j]).v;
+        __syncwarp();
+#pragma unroll 1
+        for (int j = 0; j < NPL; ++j)
+          low = low || fx_slow_node<D, N>(sh.key[el], lane + 32 * j, [&](int n) { return sk[n]; });
+        if (__any_sync(0xffffffffu, low)) sc.ok = 0;
+      }
 #pragma unroll
       for (int j = 0; j < NPL; ++j)
         fx_stage_node<D, N>(q[j], sc, g.gm1, elem, fx_place<D, N>(lane + 32 * j));
@@ -457,9 +522,16 @@ __device__ __forceinline__ void fx_batch(double* u, double* __restrict__ du,
     const unsigned bad = fx_load<D, N>(u, g, e0, count, smem, sh.key);
     if (bad) atomicOr(err, bad);
     __syncthreads();
-    if ((int)threadIdx.x < count)
+    bool slow = false;
+    if ((int)threadIdx.x < count) {
       sh.scale[threadIdx.x] = fx_scale(sh.key[threadIdx.x], cb, ed);
-    __syncthreads();
+      slow = fx_slow(sh.key[threadIdx.x], sh.scale[threadIdx.x]);
+    }
+    if (__syncthreads_or(slow)) {
+      fx_slow_elements<D, N>(count, smem, FxShape<D, N>::ELEM, 3, sh.key,
+                             [&](int el) { sh.scale[el].ok = 0; });
+      __syncthreads();
+    }
     fx_stage<D, N>(g, count, smem, sh.scale);
     __syncthreads();
     const int lane = threadIdx.x & 31, t = lane / T::LPW;
@@ -642,8 +714,23 @@ __global__ void __launch_bounds__(FACES ? FxPairPar<D, N, EPB>::THREADS_F
     const FxKeys kk = fx_keys<D>(q);
     for (int ek = first; ek <= lastt / P; ++ek) fx_merge_keys(kk, in && el == ek, sh.key[ek]);
     vsync();
+    fx::Scale sc = fx_scale(sh.key[el], cb, ed);
+    bool slow = false;  // the same for all threads
+    for (int ek = 0; ek < count; ++ek)
+      slow = slow || sh.key[ek][4] - sh.key[ek][6] > (kCrossBits << 20);
+    if (slow) {
+      unsigned* sk = reinterpret_cast<unsigned*>(smem + el * C::ELEM);
+      if (in) sk[node] = kk.v;
+      if (in && node == 0) sh.scale[el].ok = 1;
+      vsync();
+      if (in && fx_slow(sh.key[el], sc) &&
+          fx_slow_node<D, N>(sh.key[el], node, [&](int n) { return sk[n]; }))
+        sh.scale[el].ok = 0;
+      vsync();
+      if (in && !sh.scale[el].ok) sc.ok = 0;
+      vsync();
+    }
     if (in) {
-      const fx::Scale sc = fx_scale(sh.key[el], cb, ed);
       if (node == 0) sh.scale[el] = sc;
       fx_stage_node<D, N>(q, sc, g.gm1, smem + el * C::ELEM, fx_place<D, N>(node));
     }
@@ -717,7 +804,7 @@ __global__ void __launch_bounds__(FACES ? FxPairPar<D, N, EPB>::THREADS_F
         *sa = acc;
         continue;
       }
-      double val = fx_value<D>(acc, v, sc, sh.ed);
+      double val = fx_value<D, N>(acc, v, sc, sh.ed);
       const double* fce = sfc + el * 2 * D * LINES * NV;
 #pragma unroll
       for (int dir = 0; dir < D; ++dir) {

@@ -82,6 +82,7 @@ struct VScale {
   int pg, pe;          // g_n, g_E v to p
   int sa, sb;          // to A1, B1
   int np, nb;          // some cotangent of p, of e
+  int moves;           // some velocity is not zero
 };
 __device__ __forceinline__ int exp_of(double x) {
   return x > 0.0 ? exp_above((unsigned)__double2hiint(x)) : kNone;
@@ -91,12 +92,13 @@ __device__ __forceinline__ VScale vjp_scale(const unsigned* key, const int* c, i
                                             double dmax) {
   VScale s;
   s.u = element_scale(key, c);
+  s.moves = key[4] != 0u;
   const unsigned lo = (kBias - 150u) << 20, hi = (kBias + 150u) << 20;
   auto up = [](unsigned k) { return k ? __hiloint2double((int)k + 1, 0) : 0.0; };
   double W[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const unsigned w = key[6 + k];
+    const unsigned w = key[8 + k];
     s.x[k] = w ? exp_above(w) : kNone;
     W[k] = up(w);
     if (w && !(w > lo && w < hi)) s.u.ok = 0;
@@ -323,13 +325,13 @@ __global__ void __launch_bounds__(VjpFx<D, N>::threads(VjpFx<D, N>::EPB),
   __shared__ fx::Limbs s_d[D][kNPMax][kNPMax];  // 63 - ed
   __shared__ double s_d64[D][kNPMax][kNPMax];
   __shared__ fx::VScale s_scale[EPB];
-  __shared__ unsigned s_key[EPB][9];
+  __shared__ unsigned s_key[EPB][11];  // those of FxShared, then the cotangents'
   const int e0 = blockIdx.x * EPB;
   const int count = (int)g.nelem - e0 < EPB ? (int)g.nelem - e0 : EPB;
   const int t = threadIdx.x;
   if (t < count) {
     fx_clear_key(s_key[t]);
-    s_key[t][6] = s_key[t][7] = s_key[t][8] = 0u;
+    s_key[t][8] = s_key[t][9] = s_key[t][10] = 0u;
   }
   const int ed = fx_table_exponent<D>(tb) + (N == 1);
   for (int i = t; i < D * NP * NP; i += blockDim.x) {
@@ -374,7 +376,7 @@ __global__ void __launch_bounds__(VjpFx<D, N>::threads(VjpFx<D, N>::EPB),
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
         const unsigned m = __reduce_max_sync(0xffffffffu, mine ? kw[j] : 0u);
-        if ((t & 31) == 0) atomicMax(&s_key[ek][6 + j], m);
+        if ((t & 31) == 0) atomicMax(&s_key[ek][8 + j], m);
       }
     }
   }
@@ -413,9 +415,9 @@ __global__ void __launch_bounds__(VjpFx<D, N>::threads(VjpFx<D, N>::EPB),
     // short on average
     constexpr int DN = D * N;
     fx::i64* sa = sx + V::SL * P;
-    sa[0] = sc.u.ok && sc.u.moves ? 3 * DN / 2 : 0;
+    sa[0] = sc.u.ok && sc.moves ? 3 * DN / 2 : 0;
     sa[P] = sa[3 * P] = 0;
-    sa[2 * P] = sc.u.ok && sc.u.moves && sc.nb ? 3 * DN / 2 : 0;
+    sa[2 * P] = sc.u.ok && sc.moves && sc.nb ? 3 * DN / 2 : 0;
     sa[4 * P] = sc.u.ok && sc.np ? 3 * DN / 2 : 0;
 #pragma unroll
     for (int j = 0; j < D; ++j) sa[(5 + j) * P] = sc.u.ok ? (2 * D + 3) * N / 2 : 0;

@@ -197,3 +197,48 @@ def test_weak_form_far_from_a_strong_corner(d, N, n, kind):
                                   "vacuum field"])
 def test_mhd_weak_form_far_from_a_strong_corner(N, n, kind):
     _check_corner(_gpu(), "mhd", 3, N, n, "central", "hll", kind)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,N,n", [(2, 2, (3, 4)), (2, 2, (26, 25)), (2, 3, (4, 4)), (2, 3, (26, 25)),
+                                   (2, 6, (25, 26)), (3, 2, (3, 2, 3)), (3, 2, (9, 9, 8)),
+                                   (3, 3, (4, 3, 3)), (3, 3, (9, 9, 8)), (3, 4, (9, 9, 8)),
+                                   (3, 5, (3, 2, 2)), (3, 7, (2, 2, 2)), (3, 7, (9, 9, 8))])
+@pytest.mark.parametrize("kind", ["pressure", "velocity", "rest", "both ratios"])
+def test_two_point_flux_far_from_a_strong_corner(d, N, n, kind):
+    torch = _gpu()
+    if kind != "both ratios":
+        return _check_corner(torch, "euler", d, N, n, "ranocha", "llf", kind)
+    # density and internal energy both 2^5.9 higher at the corner: the pressure
+    # 2^11.8 times, inside the limits of the first two. The other nodes' rows of
+    # momentum are sums of their pressure's rounding, 2^-53 to 2^-52 times the
+    # coefficients' row sums (up to 60 in units of 2/h)
+    ne, P = int(np.prod(n)), (N + 1) ** d
+    rng = np.random.default_rng([d, N, 4])
+    rho, p = np.ones((ne, P)), np.ones((ne, P))
+    rho[:, P - 1], p[:, P - 1] = 2.0 ** 5.9, 2.0 ** 11.8
+    u = _euler(rho, 1e-3 * rng.uniform(-1, 1, (d, ne, P)), p)
+    inner = _corner("euler", d, N, ne, "none", rng)[1]
+    got, ref = _rhs(torch, "euler", d, N, n, "ranocha", "llf", u)
+    err = np.abs(got - ref)[:, 1:d + 1, inner].max()
+    assert err <= 2.0 ** -51 * 60 * max(n), err
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,n", [(2, (3, 2, 2)), (3, (9, 9, 8)), (4, (9, 9, 8)), (5, (2, 3, 2))])
+@pytest.mark.parametrize("kind", ["pressure", "velocity", "rest"])
+def test_warped_box_far_from_a_strong_corner(N, n, kind):
+    torch = _gpu()
+    import oracle
+    from paper_2108_06476_gb300 import Mesh
+    ne = int(np.prod(n))
+    u, inner = _corner("euler", 3, N, ne, kind, np.random.default_rng([N, 6]))
+    m = Mesh(3, N, n, warp=0.02, surface_flux="ranocha")
+    geom = oracle.CurvedGeometry(N, n, 0.02)
+    m.set_nodes(torch.from_numpy(geom.X).cuda())
+    m.set_metric(torch.from_numpy(geom.Ja).cuda(), torch.from_numpy(geom.J).cuda())
+    got = m.rhs(torch.from_numpy(u.reshape(-1)).cuda()).cpu().numpy().reshape(u.shape)
+    ref = oracle.curved_rhs(geom, u.reshape(-1), sflux=1).reshape(u.shape)
+    size = np.abs(ref[:, :, inner]).max(axis=(0, 2))
+    err = np.abs(got - ref)[:, :, inner].max(axis=(0, 2))
+    assert (err <= BAR * size).all(), err / np.where(size > 0, size, 1.0)

@@ -19,7 +19,7 @@
 // momentum fluxes by em, energy fluxes by em + ev
 struct MEScale {
   int er, ev, eb, ee, em;
-  int moves, field, ok;
+  int ok;
 };
 
 // node values: r = rho/2 (63 - er), e/2 (63 - ee), pt/2 (63 - em), v/2 (63 -
@@ -32,6 +32,7 @@ constexpr int kMESlots = 14;
 
 struct MEPrim {
   double rho, e, p, v[3], B[3];
+  unsigned E;  // high word of the total energy
 };
 
 __device__ __forceinline__ MEPrim me_prim(const double* c, double gm1, double gm1inv,
@@ -49,6 +50,7 @@ __device__ __forceinline__ MEPrim me_prim(const double* c, double gm1, double gm
   }
   q.p = gm1 * fma(-0.5, mv, c[4]);
   q.e = q.p * rr * gm1inv;
+  q.E = (unsigned)__double2hiint(c[4]);
   Prim<double, 3> t;
   t.rho = q.rho;
   t.p = q.p;
@@ -56,7 +58,8 @@ __device__ __forceinline__ MEPrim me_prim(const double* c, double gm1, double gm
   return q;
 }
 
-// keys: rho max and min, e max and min, |v| max, p max, |B| max
+// keys: rho max and min, e max and min, |v| max, p max, |B| max (then, not used
+// here, |v| min, |B| min, total energy min)
 __device__ __forceinline__ MEScale me_scale(const unsigned* key, const int* c, bool usable) {
   const unsigned rmax = key[0], rmin = key[1], emax = key[2], emin = key[3], vmax = key[4],
                  pmax = key[5], bmax = key[6];
@@ -74,8 +77,6 @@ __device__ __forceinline__ MEScale me_scale(const unsigned* key, const int* c, b
   s.ee = ee + 1;
   if (s.ee < 2 * s.ev + 2) s.ee = 2 * s.ev + 2;
   if (s.ee < s.em - s.er) s.ee = s.em - s.er;
-  s.moves = vmax != 0u;
-  s.field = bmax != 0u;
   const unsigned lo = (fx::kBias - 150u) << 20, hi = (fx::kBias + 150u) << 20;
   s.ok = usable && rmax < hi && rmin > lo && emax < hi && emin > lo && vmax < hi && pmax < hi &&
          bmax < hi && rmax - rmin < (6u << 20) && emax - emin < (6u << 20) &&
@@ -161,6 +162,10 @@ __device__ __forceinline__ int me_exponent(int v, const MEScale& s) {
                                                                           : s.eb - 60;
 }
 
+constexpr int kMEKeys = 10;
+__device__ __forceinline__ constexpr bool me_key_is_min(int j) {
+  return j == 1 || j == 3 || j > 6;
+}
 __device__ __forceinline__ void me_keys(const MEPrim& q, unsigned* k) {
   auto hw = [](double x) { return (unsigned)__double2hiint(x); };
   k[0] = k[1] = hw(q.rho);
@@ -172,6 +177,9 @@ __device__ __forceinline__ void me_keys(const MEPrim& q, unsigned* k) {
     k[4] = max(k[4], hw(q.v[j]) & 0x7fffffffu);
     k[6] = max(k[6], hw(q.B[j]) & 0x7fffffffu);
   }
+  k[7] = k[4];
+  k[8] = k[6];
+  k[9] = q.E;
 }
 
 // the EC face flux (normal component first) from the conserved traces; false
@@ -179,11 +187,11 @@ __device__ __forceinline__ void me_keys(const MEPrim& q, unsigned* k) {
 __device__ __forceinline__ bool mhd_ec_face_fixed(const double* cl, const double* cr, const Geom& g,
                                                   unsigned& bad, double* f) {
   const MEPrim L = me_prim(cl, g.gm1, g.gm1inv, bad), R = me_prim(cr, g.gm1, g.gm1inv, bad);
-  unsigned kl[7], kr[7];
+  unsigned kl[kMEKeys], kr[kMEKeys];
   me_keys(L, kl);
   me_keys(R, kr);
 #pragma unroll
-  for (int j = 0; j < 7; ++j) kl[j] = j == 1 || j == 3 ? min(kl[j], kr[j]) : max(kl[j], kr[j]);
+  for (int j = 0; j < 7; ++j) kl[j] = me_key_is_min(j) ? min(kl[j], kr[j]) : max(kl[j], kr[j]);
   int c[2];
   fx::scale_bits(g.gm1, c);
   const MEScale s = me_scale(kl, c, true);
@@ -288,6 +296,12 @@ __device__ __forceinline__ void me_pair(unsigned char* elem, const MEScale& sc,
   }
 }
 
+// the units by which a sum's truncated products fall short (fx_stage_node)
+template <int N>
+__device__ __forceinline__ constexpr int me_start(int v) {
+  return v >= 5 && v < kMV ? 2 * N : 3 * N;
+}
+
 // stage a node's slots in its element's form and start its sums
 // (uc: the node's first conserved value, the others P apart)
 template <int N, bool SPREAD>
@@ -329,16 +343,9 @@ __device__ __forceinline__ void me_stage(const MEPrim& q, const double* uc, cons
     sp[10 * P + pl] = n.qB2;
     sp[11 * P + pl] = n.hvB;
   }
-  // the units by which truncated products fall short (fx_stage_node); sums of
-  // zero fluxes start from zero
 #pragma unroll
   for (int v = 0; v < kMQ; ++v) {
-    const bool some = v == 0 || v == 4 ? sc.moves
-                      : v <= 3         ? true
-                      : v < kMV        ? sc.moves && sc.field
-                                       : sc.field;
-    const int terms = v >= 5 && v < kMV ? 2 * N : 3 * N;
-    sx[(kMESlots + v) * P + pl] = sc.ok && some ? terms : 0;
+    sx[(kMESlots + v) * P + pl] = sc.ok ? me_start<N>(v) : 0;
     if (SPREAD) {
       sx[(kMESlots + kMQ + v) * P + pl] = 0;
       sx[(kMESlots + 2 * kMQ + v) * P + pl] = 0;
@@ -363,13 +370,13 @@ __global__ void __launch_bounds__((SPREAD ? 3 : 1) * MELaunch<N>::threads(EPB),
   __shared__ Tables<double> tb;
   __shared__ fx::Limbs s_d[3][kNPMax][kNPMax];
   __shared__ MEScale s_scale[EPB];
-  __shared__ unsigned s_key[EPB][7];
+  __shared__ unsigned s_key[EPB][kMEKeys];
   const int e0 = blockIdx.x * EPB;
   const int count = (int)g.nelem - e0 < EPB ? (int)g.nelem - e0 : EPB;
   const int t = threadIdx.x;
   if (t < count) {
 #pragma unroll
-    for (int j = 0; j < 7; ++j) s_key[t][j] = j == 1 || j == 3 ? 0xffffffffu : 0u;
+    for (int j = 0; j < kMEKeys; ++j) s_key[t][j] = me_key_is_min(j) ? 0xffffffffu : 0u;
   }
   stage_tables<3, N, double>(tb, tbg, fz.k ? *fz.dt : 1.0);
   __syncthreads();
@@ -387,7 +394,7 @@ __global__ void __launch_bounds__((SPREAD ? 3 : 1) * MELaunch<N>::threads(EPB),
     const int i = t0 + (t & 31);
     const bool in = i < count * P;
     const int el = i / P, node = i % P;
-    unsigned k[7] = {};
+    unsigned k[kMEKeys] = {};
     if (in) {
       double c[kMV];
 #pragma unroll
@@ -408,8 +415,8 @@ __global__ void __launch_bounds__((SPREAD ? 3 : 1) * MELaunch<N>::threads(EPB),
     for (int ek = t0 / P; ek <= last; ++ek) {
       const bool mine = in && el == ek;
 #pragma unroll
-      for (int j = 0; j < 7; ++j) {
-        if (j == 1 || j == 3) {
+      for (int j = 0; j < kMEKeys; ++j) {
+        if (me_key_is_min(j)) {
           const unsigned m = __reduce_min_sync(0xffffffffu, mine ? k[j] : 0xffffffffu);
           if ((t & 31) == 0) atomicMin(&s_key[ek][j], m);
         } else {
@@ -421,8 +428,34 @@ __global__ void __launch_bounds__((SPREAD ? 3 : 1) * MELaunch<N>::threads(EPB),
   }
   if (bad) atomicOr(err, bad);
   __syncthreads();
-  if (t < count) s_scale[t] = me_scale(s_key[t], cb, usable);
-  __syncthreads();
+  bool weak = false;
+  if (t < count) {
+    const unsigned* k = s_key[t];
+    s_scale[t] = me_scale(k, cb, usable);
+    if (energy_far(s_scale[t].em, k[9])) s_scale[t].ok = 0;
+    weak = s_scale[t].ok && (k[4] - k[7]) + (k[6] - k[8]) > (kCrossBits << 20);
+  }
+  if (__syncthreads_or(weak)) {  // some node may lie too far below
+    for (int i = t; i < count * P; i += blockDim.x) {
+      const int el = i / P;
+      const double* sp = reinterpret_cast<const double*>(dg_smem + el * ELEM);
+      auto size = [&](int at, int n) {
+        unsigned m = 0;
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          m = max(m, (unsigned)__double2hiint(sp[(at + j) * P + fx_place<3, N>(n)]) & 0x7fffffffu);
+        return m;
+      };
+      const unsigned mv = s_key[el][4], mb = s_key[el][6];
+      if ((mv - size(3, i % P)) + (mb - size(6, i % P)) <= (kCrossBits << 20)) continue;
+      const unsigned cv = cross_max<3, N>(i % P, [&](int n) { return size(3, n); });
+      const unsigned cb2 = cross_max<3, N>(i % P, [&](int n) { return size(6, n); });
+      // the induction rows hold products of v and B
+      if (cross_far(mv, cv) || (cv && cb2 && (mv - cv) + (mb - cb2) > (kCrossBits << 20)))
+        s_scale[el].ok = 0;
+    }
+    __syncthreads();
+  }
   for (int i = t; i < count * P; i += blockDim.x) {
     const int el = i / P, node = i % P, pl = fx_place<3, N>(node);
     const double* sp = reinterpret_cast<const double*>(dg_smem + el * ELEM) + pl;
@@ -475,7 +508,8 @@ __global__ void __launch_bounds__((SPREAD ? 3 : 1) * MELaunch<N>::threads(EPB),
       if (sc.ok) {
         fx::i64 a = sa[v * P];
         if (SPREAD) a += sa[(kMQ + v) * P] + sa[(2 * kMQ + v) * P];
-        val[v] = fx::to_double_int(a, ed + me_exponent(v, sc));
+        val[v] = a == me_start<N>(v) ? 0.0  // nothing but zeros
+                                     : fx::to_double_int(a, ed + me_exponent(v, sc));
       } else {
         val[v] = __longlong_as_double(sa[v * P]);
         if (SPREAD)

@@ -242,3 +242,11 @@ def test_warped_box_far_from_a_strong_corner(N, n, kind):
     size = np.abs(ref[:, :, inner]).max(axis=(0, 2))
     err = np.abs(got - ref)[:, :, inner].max(axis=(0, 2))
     assert (err <= BAR * size).all(), err / np.where(size > 0, size, 1.0)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,n", [(2, (3, 2, 2)), (2, (9, 9, 8)), (3, (3, 2, 2)), (3, (9, 9, 8)),
+                                 (4, (9, 9, 8)), (5, (3, 2, 2)), (7, (2, 2, 2))])
+@pytest.mark.parametrize("kind", ["pressure", "velocity", "field", "rest", "vacuum field"])
+def test_mhd_two_point_flux_far_from_a_strong_corner(N, n, kind):
+    _check_corner(_gpu(), "mhd", 3, N, n, "ec", "ec", kind)

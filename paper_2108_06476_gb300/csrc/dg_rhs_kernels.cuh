@@ -139,8 +139,9 @@ __device__ __forceinline__ void pp_line_of(int dir, int node, int& l, int& i) {
 // sums comes from these lines); elements with other nodes take the FP64 form.
 // Lines of zeros are exact: sums that saw nothing but zeros are set to zero.
 constexpr unsigned kCrossBits = 6;
+// (top != 0: the first that is near enough to top, zero if there is none)
 template <int D, int N, typename F>
-__device__ __forceinline__ unsigned cross_max(int node, const F& at) {
+__device__ __forceinline__ unsigned cross_max(int node, const F& at, unsigned top = 0u) {
   unsigned m = 0;
 #pragma unroll 1
   for (int dir = 0; dir < D; ++dir) {
@@ -150,9 +151,10 @@ __device__ __forceinline__ unsigned cross_max(int node, const F& at) {
     for (int b = 0; b <= N; ++b) {
       const unsigned k = at(line_node_rt<D, N>(dir, l, b));
       m = k > m ? k : m;
+      if (top && top - m <= (kCrossBits << 20)) return m;
     }
   }
-  return m;
+  return top ? 0u : m;
 }
 // whether the key (high word) `most` of an element leaves one of `some` too far
 // below

@@ -81,8 +81,7 @@ struct VScale {
   int vF, vg, ve, vp;  // F R, g_k f_0, g_E f_0 v, g_E p to v
   int pg, pe;          // g_n, g_E v to p
   int sa, sb;          // to A1, B1
-  int np, nb;          // some cotangent of p, of e
-  int moves;           // some velocity is not zero
+  int zero;            // no cotangent: nothing to sum
 };
 __device__ __forceinline__ int exp_of(double x) {
   return x > 0.0 ? exp_above((unsigned)__double2hiint(x)) : kNone;
@@ -92,7 +91,6 @@ __device__ __forceinline__ VScale vjp_scale(const unsigned* key, const int* c, i
                                             double dmax) {
   VScale s;
   s.u = element_scale(key, c);
-  s.moves = key[4] != 0u;
   const unsigned lo = (kBias - 150u) << 20, hi = (kBias + 150u) << 20;
   auto up = [](unsigned k) { return k ? __hiloint2double((int)k + 1, 0) : 0.0; };
   double W[3];
@@ -103,10 +101,9 @@ __device__ __forceinline__ VScale vjp_scale(const unsigned* key, const int* c, i
     W[k] = up(w);
     if (w && !(w > lo && w < hi)) s.u.ok = 0;
   }
-  s.np = s.x[1] != kNone || s.x[2] != kNone;
-  s.nb = s.x[2] != kNone;
-  if (ed > 300 || ed < -300 || !(s.x[0] != kNone || s.np)) s.u.ok = 0;
-  if (!s.u.ok) return s;
+  s.zero = s.x[0] == kNone && s.x[1] == kNone && s.x[2] == kNone;
+  if (ed > 300 || ed < -300 || energy_far(s.u.em, key[7])) s.u.ok = 0;
+  if (!s.u.ok || s.zero) return s;
   // pressures and energies by themselves (the scales that momentum and energy
   // fluxes need would cost them bits). Where kinetic energies exceed the
   // internal ones, from a Mach number between 1.3 and 2.6, the common exponents
@@ -173,7 +170,11 @@ __device__ __forceinline__ PairAdj<D> pair_adjoint(const Node<D>& a, const Node<
   const Limbs vn = limbs(vm0), gE = limbs(g[D + 1]);
   const Limbs f0 = limbs(mul(R, vn) << 1);  // 63 - er - ev
   Limbs xa[D], xb[D];
-  i64 vv = 0, F = (g[0] >> s.sm) + D;  // D: the shifted products' mean loss
+  i64 some = g[0] | g[D + 1];
+#pragma unroll
+  for (int k = 0; k < D; ++k) some |= g[1 + k];
+  // D: the shifted products' mean loss (where there is nothing but zeros, zero)
+  i64 vv = 0, F = (g[0] >> s.sm) + (some ? D : 0);
 #pragma unroll
   for (int k = 0; k < D; ++k) {
     xa[k] = limbs(a.v[k]);
@@ -233,7 +234,50 @@ struct VjpFx {
     return b;
   }
   static constexpr int EPB = best();
+  // where sum j starts: the units by which its truncated products and shifts
+  // fall short on average (A2 and B2: none on average)
+  __device__ __forceinline__ static constexpr int start(int j) {
+    return j == 1 || j == 3 ? 0 : j < 5 ? 3 * D * N / 2 : (2 * D + 3) * N / 2;
+  }
 };
+
+// Whether what a node's sums come from lies too far below the units of its
+// element (at sp; cross_far): its velocities, or any class of cotangents while
+// another one on its lines is not zero (the classes' terms share exponents)
+template <int D, int N>
+__device__ __forceinline__ bool vjp_far_node(const double* sp, const unsigned* key, int node) {
+  using V = VjpFx<D, N>;
+  auto most = [&](int at, int n, int cnt) {
+    unsigned m = 0;
+    for (int j = 0; j < cnt; ++j)
+      m = max(m, (unsigned)__double2hiint(sp[(at + j) * V::P + n]) & 0x7fffffffu);
+    return m;
+  };
+  const int at[4] = {3, V::W, V::W + 1, V::W + 1 + D}, cnt[4] = {D, 1, D, 1};
+  // most nodes, or one of the first on their lines, are near enough themselves
+  bool near = true;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const unsigned top = key[c ? 7 + c : 4];
+    near = near &&
+           (top - most(at[c], node, cnt[c]) <= (kCrossBits << 20) ||
+            cross_max<D, N>(node, [&](int n) { return most(at[c], n, cnt[c]); }, top) != 0u);
+  }
+  if (near) return false;
+  bool some = false, far = false;
+#pragma unroll 1
+  for (int c = 0; c < 4; ++c) {
+    const unsigned top = key[c ? 7 + c : 4];
+    const unsigned m = cross_max<D, N>(node, [&](int n) { return most(at[c], n, cnt[c]); });
+    if (c == 0) {
+      if (cross_far(top, m)) return true;
+    } else {
+      some = some || m != 0u;
+      far = far || top - m > (kCrossBits << 20);
+    }
+  }
+  return some && far;
+}
 
 template <int D, int N>
 __device__ __forceinline__ void vjp_fx_pair(unsigned char* elem, const fx::VScale& sc,
@@ -390,6 +434,13 @@ __global__ void __launch_bounds__(VjpFx<D, N>::threads(VjpFx<D, N>::EPB),
   __syncthreads();
   for (int i = t; i < count * P; i += blockDim.x) {
     const int el = i / P;
+    if (vjp_far_node<D, N>(reinterpret_cast<const double*>(dg_smem + el * V::ELEM), s_key[el],
+                           i % P))
+      s_scale[el].u.ok = 0;
+  }
+  __syncthreads();
+  for (int i = t; i < count * P; i += blockDim.x) {
+    const int el = i / P;
     const fx::VScale& sc = s_scale[el];
     double* sp = reinterpret_cast<double*>(dg_smem + el * V::ELEM) + i % P;
     fx::i64* sx = reinterpret_cast<fx::i64*>(sp);
@@ -411,16 +462,9 @@ __global__ void __launch_bounds__(VjpFx<D, N>::threads(VjpFx<D, N>::EPB),
         sx[(V::W + j) * P] = x == fx::kNone ? 0 : fx::half_fixed(sp[(V::W + j) * P], x) << 1;
       }
     }
-    // the sums start at the units by which truncated products and shifts fall
-    // short on average
-    constexpr int DN = D * N;
     fx::i64* sa = sx + V::SL * P;
-    sa[0] = sc.u.ok && sc.moves ? 3 * DN / 2 : 0;
-    sa[P] = sa[3 * P] = 0;
-    sa[2 * P] = sc.u.ok && sc.moves && sc.nb ? 3 * DN / 2 : 0;
-    sa[4 * P] = sc.u.ok && sc.np ? 3 * DN / 2 : 0;
 #pragma unroll
-    for (int j = 0; j < D; ++j) sa[(5 + j) * P] = sc.u.ok ? (2 * D + 3) * N / 2 : 0;
+    for (int j = 0; j < 5 + D; ++j) sa[j * P] = sc.u.ok ? V::start(j) : 0;
   }
   __syncthreads();
   const int lane = t & 31, slot = lane / T::LPW;
@@ -431,7 +475,7 @@ __global__ void __launch_bounds__(VjpFx<D, N>::threads(VjpFx<D, N>::EPB),
   for (int dir = 0; dir < D; ++dir) {
 #pragma unroll 1
     for (int m = 0; m < T::ROUNDS; ++m) {
-      if (in) {
+      if (in && !(s_scale[el].u.ok && s_scale[el].zero)) {
         int a, b;
         tourney_pair<N>(m, slot, a, b);
         vjp_fx_pair<D, N>(dg_smem + el * V::ELEM, s_scale[el], s_d[dir], s_d64[dir], g.gm1inv,
@@ -454,16 +498,18 @@ __global__ void __launch_bounds__(VjpFx<D, N>::threads(VjpFx<D, N>::EPB),
       const int er = sc.u.er, ev = sc.u.ev, ee = sc.u.ee;
       const double en = fx::to_double_int(sx[2 * P], ee - 62);
       irho = rcp(fx::to_double_int(sx[0], er - 62));
-      const double eb = fx::to_double_int(sa[2 * P], sc.b - 63) +
-                        fx::to_double_int(sa[3 * P], sc.e2 - 61) * rcp(en);
+      // (a sum still at its start saw nothing but zeros)
+      auto sum = [&](int j, int x) {
+        return sa[j * P] == V::start(j) ? 0.0 : fx::to_double_int(sa[j * P], x);
+      };
+      const double eb = sum(2, sc.b - 63) + sum(3, sc.e2 - 61) * rcp(en);
       const double eir = eb * irho;
-      pb = fx::to_double_int(sa[4 * P], sc.p - 63) + eir * g.gm1inv;
-      rb = fx::to_double_int(sa[0], sc.a - 63) +
-           fx::to_double_int(sa[P], sc.F + ev + er - 62) * irho - eir * en;
+      pb = sum(4, sc.p - 63) + eir * g.gm1inv;
+      rb = sum(0, sc.a - 63) + sum(1, sc.F + ev + er - 62) * irho - eir * en;
 #pragma unroll
       for (int k = 0; k < D; ++k) {
         v[k] = fx::to_double_int(sx[(5 + k) * P], ev - 62);
-        vb[k] = fx::to_double_int(sa[(5 + k) * P], sc.v - 63);
+        vb[k] = sum(5 + k, sc.v - 63);
       }
     } else {
       irho = 1.0 / sp[0];

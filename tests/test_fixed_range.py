@@ -250,3 +250,47 @@ def test_warped_box_far_from_a_strong_corner(N, n, kind):
 @pytest.mark.parametrize("kind", ["pressure", "velocity", "field", "rest", "vacuum field"])
 def test_mhd_two_point_flux_far_from_a_strong_corner(N, n, kind):
     _check_corner(_gpu(), "mhd", 3, N, n, "ec", "ec", kind)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,N,n", [(2, 2, (3, 2)), (2, 5, (2, 2)), (3, 2, (2, 2, 2)), (3, 3, (2, 2, 1)),
+                                   (3, 4, (2, 1, 1)), (3, 5, (2, 1, 1)), (3, 7, (1, 2, 1))])
+@pytest.mark.parametrize("kind", ["probe", "mass probe", "spread", "momentum spread", "two probes",
+                                  "slow"])
+def test_gradient_far_from_a_strong_corner(d, N, n, kind):
+    # the entries of J^T w at nodes whose lines do not reach the corner that
+    # holds the large cotangents, each against w . (J e_j) by the oracle's exact
+    # JVP; a probe's gradient is zero there
+    torch = _gpu()
+    import oracle
+    from paper_2108_06476_gb300 import Mesh, workloads as W
+    ne, P = int(np.prod(n)), (N + 1) ** d
+    rng = np.random.default_rng([d, N, 8])
+    u, inner = _corner("euler", d, N, ne, "velocity" if kind == "slow" else "none", rng)
+    w = rng.standard_normal((ne, d + 2, P))
+    if kind in ("probe", "mass probe"):
+        w[:, :, :P - 1] = 0.0
+    if kind == "mass probe":
+        w[:, 1:] = 0.0
+    if kind == "spread":
+        w[:, :, :P - 1] *= 1e-9
+    if kind == "momentum spread":
+        w[:, 1:d + 1, :P - 1] *= 1e-9
+        w[:, [0, d + 1]] = 0.0
+    if kind == "two probes":  # energy cotangents everywhere, a large mass cotangent at the corner
+        w[:, :d + 1] = 0.0
+        w[:, 0, P - 1] = 1e9
+    m = Mesh(d, N, n, surface_flux="ranocha")
+    ub = m.rhs_vjp(torch.from_numpy(u.reshape(-1)).cuda(),
+                   torch.from_numpy(w.reshape(-1)).cuda()).cpu().numpy().reshape(w.shape)
+    if "probe" in kind and kind != "two probes":
+        assert not ub[:, :, inner].any()
+    at = np.flatnonzero(inner)
+    for _ in range(12):
+        e, v, j = rng.integers(ne), rng.integers(d + 2), rng.choice(at)
+        t = np.zeros_like(u)
+        t[e, v, j] = 1.0
+        jv = oracle.rhs_jvp(d, N, n, W.box(d), u.reshape(-1), t.reshape(-1),
+                            sflux=1).reshape(u.shape)
+        size = np.abs(w * jv).sum()
+        assert abs(ub[e, v, j] - (w * jv).sum()) <= BAR * size, (e, v, j, ub[e, v, j], size)

@@ -80,7 +80,7 @@ struct FxShared {
   fx::Scale scale[MAXE];
   unsigned key[MAXE][8];
   int left[MAXE][D];
-  int ed;
+  int ed, far;
 };
 
 template <int D, int N>
@@ -700,7 +700,10 @@ __global__ void __launch_bounds__(FACES ? FxPairPar<D, N, EPB>::THREADS_F
       fx_clear_key(sh.key[t]);
       for (int k = 0; k < D; ++k) sh.left[t][k] = neighbour32(g, e0 + t, k, -1);
     }
-    if (t == 0) sh.ed = ed;
+    if (t == 0) {
+      sh.ed = ed;
+      sh.far = 0;
+    }
     int cb[2];
     fx::scale_bits(g.gm1, cb);
     FxPrim<D> q = {};
@@ -712,29 +715,38 @@ __global__ void __launch_bounds__(FACES ? FxPairPar<D, N, EPB>::THREADS_F
     vsync();
     const int first = (t & ~31) / P, lastt = (t | 31) < count * P ? (t | 31) : count * P - 1;
     const FxKeys kk = fx_keys<D>(q);
-    for (int ek = first; ek <= lastt / P; ++ek) fx_merge_keys(kk, in && el == ek, sh.key[ek]);
+    for (int ek = first; ek <= lastt / P; ++ek)
+      fx_merge_keys<false>(kk, in && el == ek, sh.key[ek]);
     vsync();
-    fx::Scale sc = fx_scale(sh.key[el], cb, ed);
-    bool slow = false;  // the same for all threads
-    for (int ek = 0; ek < count; ++ek)
-      slow = slow || sh.key[ek][4] - sh.key[ek][6] > (kCrossBits << 20);
-    if (slow) {
-      unsigned* sk = reinterpret_cast<unsigned*>(smem + el * C::ELEM);
-      if (in) sk[node] = kk.v;
-      if (in && node == 0) sh.scale[el].ok = 1;
-      vsync();
-      if (in && fx_slow(sh.key[el], sc) &&
-          fx_slow_node<D, N>(sh.key[el], node, [&](int n) { return sk[n]; }))
-        sh.scale[el].ok = 0;
-      vsync();
-      if (in && !sh.scale[el].ok) sc.ok = 0;
-      vsync();
-    }
     if (in) {
+      const fx::Scale sc = fx_scale(sh.key[el], cb, ed);
       if (node == 0) sh.scale[el] = sc;
+      if (sc.ok && (energy_far(sc.em, q.E) || sh.key[el][4] - kk.v > (kCrossBits << 20)))
+        sh.far = 1;
       fx_stage_node<D, N>(q, sc, g.gm1, smem + el * C::ELEM, fx_place<D, N>(node));
     }
     vsync();
+    if (sh.far) {  // some node may lie too far below: staged again, maybe in FP64
+      unsigned* sk = reinterpret_cast<unsigned*>(smem + el * C::ELEM);
+      FxPrim<D> p = {};
+      if (in) {
+        double cc[NV];
+        unsigned seen = 0;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) cc[v] = u[(long long)e0 * NV * P + (el * NV + v) * P + node];
+        p = fx_prim<D>(cc, g, seen);
+        sk[node] = fx_keys<D>(p).v;
+      }
+      vsync();
+      if (in && sh.scale[el].ok &&
+          (energy_far(sh.scale[el].em, p.E) ||
+           fx_slow_node<D, N>(sh.key[el], node, [&](int n) { return sk[n]; })))
+        sh.scale[el].ok = 0;
+      vsync();
+      if (in)
+        fx_stage_node<D, N>(p, sh.scale[el], g.gm1, smem + el * C::ELEM, fx_place<D, N>(node));
+      vsync();
+    }
   }
 #pragma unroll 1
   for (int d0 = 0; d0 < D; d0 += GROUP) {

@@ -332,6 +332,10 @@ __device__ __forceinline__ bool speed_skip(bool fine, float bound, double most) 
   return __all_sync(0xffffffffu, fine && bound > 1e-30f && bound < d2f(most) * 0.999999f);
 }
 
+}  // namespace dg
+#include "dg_fixed.cuh"
+namespace dg {
+
 // ---- logarithmic mean ----
 // ln_mean(x, y) = (y - x) / ln(y / x). With s = x + y, t = (y - x)/s and
 // f2 = t^2, ln(y/x) = 2 atanh(t), so
@@ -459,10 +463,17 @@ __device__ __forceinline__ double s_long(double f2) {
 __device__ __forceinline__ double series_limit(double) { return 1.0e-2; }
 __device__ __forceinline__ float series_limit(float) { return 4.0e-2f; }
 
-// far from x = y: the direct forms (rare; kept out of line)
-static __device__ __noinline__ double ln_mean_far(double x, double y) { return (y - x) / log1p((y - x) / x); }
+// far from x = y: the direct forms (rare; kept out of line), in FP64 with
+// ln(y/x) from the integer pipe where x and y are positive and in range
+static __device__ __noinline__ double ln_mean_far(double x, double y) {
+  if (fx::ln_ratio_in_range(x, y)) return (y - x) * rcp(fx::ln_ratio(x, y));
+  return (y - x) / log1p((y - x) / x);
+}
 static __device__ __noinline__ float ln_mean_far(float x, float y) { return (y - x) / log1pf((y - x) / x); }
-static __device__ __noinline__ double inv_ln_mean_far(double x, double y) { return log1p((y - x) / x) / (y - x); }
+static __device__ __noinline__ double inv_ln_mean_far(double x, double y) {
+  if (fx::ln_ratio_in_range(x, y)) return fx::ln_ratio(x, y) * rcp(y - x);
+  return log1p((y - x) / x) / (y - x);
+}
 static __device__ __noinline__ float inv_ln_mean_far(float x, float y) { return log1pf((y - x) / x) / (y - x); }
 
 // f2 >= 0 (an FP64 value in both kernel precisions), so the range tests

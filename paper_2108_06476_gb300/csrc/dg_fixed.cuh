@@ -35,7 +35,7 @@
 #include <cmath>
 #define __align__(n) alignas(n)
 #else
-#include "dg_device.cuh"
+#include "dg_device.cuh"  // which includes this file before its log means
 #endif
 #include "dg_fixed_tables.cuh"
 
@@ -52,6 +52,7 @@ inline double bitsd(u64 b) { double x; __builtin_memcpy(&x, &b, 8); return x; }
 static const LogEntry kLog[128] = {DG_FX_LOG_ROWS};
 static const i64 kTanhFar[] = DG_FX_TanhFar, kSinhFar[] = DG_FX_SinhFar;
 inline LogEntry log_entry(int i) { return kLog[i]; }
+inline int clz64(u64 a) { return a ? __builtin_clzll(a) : 64; }
 #else
 #define DG_FX_FN __device__ __forceinline__
 __device__ __forceinline__ int mulhi32(int a, int b) { return __mulhi(a, b); }
@@ -59,6 +60,7 @@ __device__ __forceinline__ u64 dbits(double x) { return (u64)__double_as_longlon
 __device__ __forceinline__ double bitsd(u64 b) { return __longlong_as_double((i64)b); }
 static __device__ const LogEntry kLog[128] = {DG_FX_LOG_ROWS};
 static __constant__ i64 kTanhFar[] = DG_FX_TanhFar, kSinhFar[] = DG_FX_SinhFar;
+__device__ __forceinline__ int clz64(u64 a) { return __clzll((i64)a); }
 __device__ __forceinline__ LogEntry log_entry(int i) {
   const int4 v = __ldg(reinterpret_cast<const int4*>(kLog) + i);
   LogEntry e;
@@ -332,6 +334,34 @@ DG_FX_FN double to_double(i64 a, int e) {
   const double h = bitsd(((u64)0x45300000u << 32) | hi) - 19342822341709703277445120.0;
   const double r = h + bitsd(((u64)0x43300000u << 32) | lo);
   return bitsd(dbits(r) + ((u64)(i64)e << 52));
+}
+
+// a 2^e rounded to FP64 on the integer pipe (to_double's two FP64 additions
+// would double the FP64 work of a face node); ties away from zero
+DG_FX_FN double to_double_int(i64 a, int e) {
+  if (a == 0) return 0.0;
+  const u64 m0 = (u64)(a < 0 ? -a : a);
+  const int n = clz64(m0);
+  const u64 m = m0 << n;  // leading one at bit 63
+  const u64 q = (m >> 11) + ((m >> 10) & 1);
+  const u64 b = q + ((u64)(i64)((int)kBias + 62 - n + e) << 52);
+  return bitsd(b | ((u64)a & 0x8000000000000000ULL));
+}
+
+// ln(y/x) in FP64 for normal x and y in (2^-1000, 2^1000), within 2^-52 and its
+// own rounding: the log means' far range (|ln(y/x)| > 1.09) divides by it. On
+// the integer pipe: log1p((y - x)/x) costs some 50 instructions of the FP64
+// unit, and a warp runs them if only one of its lanes is in that range.
+DG_FX_FN double ln_ratio(double x, double y) {
+  const int ex = (int)(dbits(x) >> 52) - (int)kBias, ey = (int)(dbits(y) >> 52) - (int)kBias;
+  const i64 m = ln_fixed(y, ey) - ln_fixed(x, ex);  // of the significands, 2^-60
+  const i64 j = ey - ex;
+  if (j > -10 && j < 10) return to_double_int(m + j * kLn2, -60);
+  return to_double_int((m >> 8) + j * (kLn2 >> 8) + ((j * (kLn2 & 255)) >> 8), -52);
+}
+DG_FX_FN bool ln_ratio_in_range(double x, double y) {
+  const u64 lo = (u64)(kBias - 1000u) << 52, n = (u64)2000u << 52;
+  return dbits(x) - lo < n && dbits(y) - lo < n;
 }
 
 }  // namespace fx

@@ -21,18 +21,6 @@ namespace fx {
 // x in format 63 - E (|x| < 2^E (1 - 2^-21))
 __device__ __forceinline__ i64 full_fixed(double x, int E) { return half_fixed(x, E - 1); }
 
-// a 2^e rounded to FP64 on the integer pipe (to_double's two FP64 additions
-// would double the FP64 work of a face node); ties away from zero
-__device__ __forceinline__ double to_double_int(i64 a, int e) {
-  if (a == 0) return 0.0;
-  const u64 m0 = (u64)(a < 0 ? -a : a);
-  const int n = __clzll((i64)m0);
-  const u64 m = m0 << n;  // leading one at bit 63
-  const u64 q = (m >> 11) + ((m >> 10) & 1);
-  const u64 b = q + ((u64)(i64)((int)kBias + 62 - n + e) << 52);
-  return bitsd(b | ((u64)a & 0x8000000000000000ULL));
-}
-
 // d shifted up until its leading bit is at 61 or 60; n the shift
 __device__ __forceinline__ i64 normalised(i64 d, int& n) {
   n = __clzll(d < 0 ? ~d : d) - 2;

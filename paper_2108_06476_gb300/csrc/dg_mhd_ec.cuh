@@ -303,10 +303,9 @@ __device__ __forceinline__ constexpr int me_start(int v) {
 }
 
 // stage a node's slots in its element's form and start its sums
-// (uc: the node's first conserved value, the others P apart)
 template <int N, bool SPREAD>
-__device__ __forceinline__ void me_stage(const MEPrim& q, const double* uc, const MEScale& sc,
-                                         double gm1, unsigned char* elem, int pl) {
+__device__ __forceinline__ void me_stage(const MEPrim& q, const MEScale& sc, unsigned char* elem,
+                                         int pl) {
   constexpr int P = MELaunch<N>::P;
   fx::i64* sx = reinterpret_cast<fx::i64*>(elem);
   if (sc.ok) {
@@ -325,23 +324,24 @@ __device__ __forceinline__ void me_stage(const MEPrim& q, const double* uc, cons
     sx[12 * P + pl] = n.b2;
     sx[13 * P + pl] = n.vb;
   } else {
-    unsigned dummy = 0;
-    double c[kMV];
-#pragma unroll
-    for (int v = 0; v < kMV; ++v) c[v] = uc[v * P];
-    const ECq n = ec_of(mhd_state(c, gm1, dummy));
+    // as ec_of, from the primitives at hand
+    const double beta = 0.5 * q.rho * rcp(q.p);
+    double v2 = 0.0, b2 = 0.0, vb = 0.0;
     double* sp = reinterpret_cast<double*>(elem);
-    sp[pl] = n.rho;
-    sp[P + pl] = n.beta;
+    sp[pl] = q.rho;
+    sp[P + pl] = beta;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      sp[(2 + k) * P + pl] = n.hv[k];
-      sp[(5 + k) * P + pl] = n.hB[k];
+      v2 = fma(q.v[k], q.v[k], v2);
+      b2 = fma(q.B[k], q.B[k], b2);
+      vb = fma(q.v[k], q.B[k], vb);
+      sp[(2 + k) * P + pl] = half(q.v[k]);
+      sp[(5 + k) * P + pl] = half(q.B[k]);
     }
-    sp[8 * P + pl] = n.pm;
-    sp[9 * P + pl] = n.qv2;
-    sp[10 * P + pl] = n.qB2;
-    sp[11 * P + pl] = n.hvB;
+    sp[8 * P + pl] = 0.5 * fma(beta, b2, q.rho);
+    sp[9 * P + pl] = 0.25 * v2;
+    sp[10 * P + pl] = 0.25 * b2;
+    sp[11 * P + pl] = half(vb);
   }
 #pragma unroll
   for (int v = 0; v < kMQ; ++v) {
@@ -468,8 +468,7 @@ __global__ void __launch_bounds__((SPREAD ? 3 : 1) * MELaunch<N>::threads(EPB),
       q.v[j] = sp[(3 + j) * P];
       q.B[j] = sp[(6 + j) * P];
     }
-    me_stage<N, SPREAD>(q, u + (long long)(e0 + el) * kMV * P + node, s_scale[el], g.gm1,
-                        dg_smem + el * ELEM, pl);
+    me_stage<N, SPREAD>(q, s_scale[el], dg_smem + el * ELEM, pl);
   }
   __syncthreads();
   const int lane = t & 31, slot = lane / T::LPW;

@@ -215,7 +215,8 @@ struct MELaunch {
   static constexpr int BY_THREADS = 8 * T::LPW / LINES > 0 ? 8 * T::LPW / LINES : 1;
   static constexpr int BY_SMEM = 98304 / ELEM > 0 ? 98304 / ELEM : 1;
   static constexpr int MOST = BY_THREADS < BY_SMEM ? BY_THREADS : BY_SMEM;
-  static constexpr int EPB = MOST < 16 ? MOST : 16;
+  // 3D N = 4: three elements fill 94% of their warps' lanes, four 89%
+  static constexpr int EPB = N == 4 && MOST == 4 ? 3 : MOST < 16 ? MOST : 16;
   static constexpr int threads(int epb) { return 32 * ((epb * LINES + T::LPW - 1) / T::LPW); }
   // SPREAD (small meshes): one element per CTA with warps and sums of their own
   // for each direction

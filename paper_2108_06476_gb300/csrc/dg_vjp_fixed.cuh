@@ -219,18 +219,24 @@ struct VjpFx {
   static constexpr int W = 5 + D, SL = W + NV, ELEM = (SL + 5 + D) * P * 8;
   static constexpr int threads(int epb) { return 32 * ((epb * LINES + T::LPW - 1) / T::LPW); }
   // elements per CTA: the count for which the warps an SM holds (shared
-  // memory, 20 warps at 100 registers) have the most lines; the smallest of
-  // equals
+  // memory, 20 warps at 100 registers) have the most lines; of equals the one
+  // with a tenth more of its lanes in use (3D N = 4: 5 elements in 8 warps, not
+  // 2 in 4), else the smallest
   static constexpr int score(int epb) {
     const int warps = threads(epb) / 32;
     const int by_smem = 229376 / (epb * ELEM + 2048), by_warps = 20 / warps;
     const int ctas = by_smem < by_warps ? by_smem : by_warps;
     return ctas * epb * LINES;
   }
+  static constexpr bool fuller(int e, int b) {
+    return e * threads(b) * 10 > b * threads(e) * 11 && score(e) * 21 >= score(b) * 20;
+  }
   static constexpr int best() {
     int b = 1;
     for (int e = 2; e <= 16; ++e)
-      if (threads(e) <= 512 && e * ELEM <= 200000 && score(e) * 20 > score(b) * 21) b = e;
+      if (threads(e) <= 512 && e * ELEM <= 200000 &&
+          (score(e) * 20 > score(b) * 21 || fuller(e, b)))
+        b = e;
     return b;
   }
   static constexpr int EPB = best();

@@ -132,7 +132,8 @@ def _code_only(text):
     return re.sub(r"\s+", "", text)
 
 
-MHD_KERNEL_SOURCES = ("dg_device.cuh", "dg_fixed.cuh", "dg_mhd_weak.cuh", "dg_mhd.cu")
+MHD_KERNEL_SOURCES = ("dg_device.cuh", "dg_fixed.cuh", "dg_fixed_tables.cuh", "dg_fixed_face.cuh",
+                      "dg_rhs_kernels.cuh", "dg_mhd_weak.cuh", "dg_mhd.cu")
 
 
 def source_sha(files=KERNEL_SOURCES):

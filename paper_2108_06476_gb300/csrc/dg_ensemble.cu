@@ -790,8 +790,8 @@ int dg_ensemble_get_block(const dg_ensemble* E, int* threads, int* ctas_per_sm, 
 // (u is not changed) and keeps the fastest; the RK register is saved and
 // restored around the trials, and so are the time steps: the trials take 1e-8
 // (with the zeros of an ensemble that has not stepped yet the coefficients
-// times dt would be zeros and every element take the FP64 form: 30 ms a stage
-// instead of 11, and another shape the fastest).
+// times dt would be zeros and every element take the FP64 form, three times
+// slower and with another shape the fastest).
 int dg_ensemble_tune(dg_ensemble* E, const double* u, double* u_tmp, int* best_threads,
                      int* best_blocks_per_sm, float* best_ms) {
   if (!E || !u || !u_tmp || u == u_tmp) return fail(DG_ERR_ARG, "dg_ensemble_tune: bad argument");

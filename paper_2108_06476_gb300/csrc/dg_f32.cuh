@@ -48,11 +48,12 @@ namespace dg {
 // ---- the log-mean polynomials of the perturbation form ----
 // phi(f2) = 1 - t/atanh(t) = f2 R(f2). FP64 small-difference branch (both
 // log means' f2 below kSeriesLim): the Taylor series of R to first order,
-// evaluated in FP64; its truncation (the f2^2 term, 1.4e-9 relative at the
+// on 64-bit integers (series_r); its truncation (the f2^2 term, 1.4e-9 relative at the
 // limit) lies 40 times below the FP32 rounding of every result it feeds, and
 // R(0) = 1/3 is exact. FP32 range f2 < 0.25: a fitted degree-5 R
 // (gen_log_mean_poly.py); beyond, log1p. phi_r64 and phi_r32 state the
-// polynomials; phi_r64_dd and phi_r32_dd evaluate the same coefficients.
+// polynomials; phi_r64_dd and phi_r32_dd evaluate the same coefficients (the
+// FP64 pair states the series that series_r takes; no kernel calls it).
 constexpr float kSeriesLim = 1.0e-4f;
 // degree 1 on f2 in [0, 1e-4]; measured relative error 1.4e-09
 __device__ __forceinline__ double phi_r64(double f2) {

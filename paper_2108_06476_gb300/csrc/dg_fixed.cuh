@@ -8,20 +8,26 @@
 // fluxes are polynomials in values of bounded size apart from the two
 // logarithmic means, so inside one element they run on integers scaled by
 // per-element powers of two, with 62 to 63 bits below the element's largest
-// value (FP64 has 53 below each value's own): no result loses precision as
-// long as the element's densities lie within a factor 2^5 and its internal
-// energies within 2^6 of each other (less the bits by which the kinetic
-// energies exceed them, from a Mach number of about 1.5). Elements outside
-// these limits, and any that hold a non-finite or non-positive value, take the
-// FP64 form (volume_direction).
+// value (FP64 has 53 below each value's own). An element is taken if its
+// densities and its internal energies lie within a factor 2^6 of each other
+// each (the latter less the bits by which the kinetic energies exceed them: at
+// gamma = 1.4 an element of uniform energies is refused from a Mach number
+// between 5.7 and 10.6, where its powers of two fall, and one of energies 6
+// times apart between 3.0 and 5.1), its total energies within 2^10 of the units
+// and the velocities on every node's lines within 2^6 of the largest
+// (element_scale; energy_far and cross_far in dg_rhs_kernels.cuh): each node's
+// sums then keep at least 45 bits of their own size, nearly all of them more
+// than FP64's. Other elements, and any that hold a non-finite or non-positive
+// value, take the FP64 form in the same kernel (fx_pair; measured beside
+// volume_fx_kernel).
 //
 // The logarithmic means need no division: with L = ln(rho), D = L_b - L_a,
 //   ln_mean(rho_a, rho_b) = (rho_a + rho_b)/2 tanh(D/2)/(D/2),
 // and with e = p/((gamma-1) rho) the internal energy, D = ln(e_b) - ln(e_a),
 //   p_a p_b/((gamma-1) ln_mean(rho_a p_b, rho_b p_a)) = (e_a + e_b)/2 D/sinh(D)
 // (the left side is the energy term of Ranocha's flux). The logarithms are
-// per-node values; an error d in D reaches the means only as D d/6, so 2^-53
-// in the logarithms is far below the rounding of the means.
+// per-node values, each within 2^-53; an error d in D reaches the means only as
+// D d/6, far below the rounding of the means.
 //
 // Numbers: a 64-bit integer X stands for x = X 2^-q 2^E with a format q known
 // at compile time and a per-element exponent E (Scale). mul() returns the
@@ -299,7 +305,8 @@ struct Node {
 };
 
 // f[0] mass (62 - er - ev), f[1..D] momenta, normal first (63 - em),
-// f[D + 1] energy (61 - em - ev); all below 2^62 in magnitude
+// f[D + 1] energy (61 - em - ev); all below 2^62 in magnitude, but for the
+// normal momentum where gamma > 3 (c = 1 in scale_bits): below 1.25 2^62
 template <int D>
 DG_FX_FN void pair_flux(const Node<D>& a, const Node<D>& b, const Scale& sc, i64 f[D + 2]) {
   i64 rho, ee;

@@ -12,7 +12,11 @@
 // 37% waiting for dependent results; this layout runs 24 warps per SM. Measured
 // at 64^3 N = 3, a fused stage's volume kernel: FP64 8.47 ms, fixed point with
 // one thread per line 3.87, this layout 2.49; rhs at 24^3 N = 7: 8.14 ms to
-// 2.0. About 40 FP64 instructions per node are left (prologue, lifting, stage
+// 2.0. Meshes all of whose elements take the FP64 form, against the FP64 kernels
+// with one thread per line: 32^3 N = 3 supersonic 1.42 and 1.50 ms, with a node
+// 150 times denser in every element 1.71 and 2.32; 24^3 N = 4 1.60 and 1.72,
+// 16^3 N = 7 3.00 and 3.14, 2D 256^2 N = 3 0.48 and 0.49; a stage of 18 members
+// of degree 3 to 5 6.48 and 6.28 ms. About 40 FP64 instructions per node are left (prologue, lifting, stage
 // update); the sums become doubles on the integer pipe (to_double's two
 // additions per value cost the step 4%: 14.98 and 14.30 ms). The threads of a line share a warp
 // (32/T lines per warp), so rounds are separated by a warp barrier. At N = 3
@@ -165,7 +169,7 @@ __device__ __forceinline__ void fx_pair(unsigned char* elem, const fx::Scale& sc
 // the exponent of the coefficients' format: |Dt[0][1]| is the largest
 // coefficient of every degree, and the absolute row sums over the three
 // directions stay below 6 times it, so that a node's sum of products with
-// fluxes below 2^62 stays below 2^63
+// fluxes below 2^62 (or 1.25 2^62, pair_flux) stays below 2^63
 template <int D>
 __device__ __forceinline__ int fx_table_exponent(const Tables<double>& tb) {
   unsigned m = 0;

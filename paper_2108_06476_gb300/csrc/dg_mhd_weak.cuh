@@ -9,11 +9,12 @@
 // summing to zero), and + lift F* is added before the sum is rounded to FP64:
 // the two cancel (added afterwards in FP64, the error of smooth data was up to
 // 2.2 times that of lift (F* - f(u_i)), at a supersonic outflow 25 times). A
-// face value beyond the element's units is added in FP64. Elements with non-finite
-// values, non-positive densities, densities spread over more than 2^6, nodes
-// whose energy lies far below the element's units, or whose lines hold far
-// smaller momenta, velocities or fields than the element (energy_far,
-// cross_far), take the same steps in FP64.
+// face value beyond the element's units (a strong jump's dissipation) is added
+// in FP64, which costs a tenth of the rhs where most are. The same steps run in
+// FP64 in elements with non-finite values, non-positive densities or densities
+// spread over more than 2^6, and with nodes whose energy lies far below the
+// element's units or whose lines hold far smaller momenta, velocities or fields
+// than the element (energy_far, cross_far).
 //
 // Included by dg_mhd.cu. 48^3 N = 3, rhs only: 2.68 ms in FP64, 0.98 here; HLL
 // faces 1.81 and 0.57 ms, LLF 1.55 and 0.51.

@@ -9,7 +9,10 @@
 //    meshes, the pair fluxes in 64-bit fixed point with the threads of a line
 //    taking disjoint node pairs in turn.
 //
-//  volume_kernel (Chandrashekar's and the central flux): one CTA per EPB
+//  volume_weak_kernel (dg_weak.cuh): the central flux on FP64 meshes of
+//    kPairParallelElems elements and more.
+//
+//  volume_kernel (Chandrashekar's flux on such meshes): one CTA per EPB
 //    elements, one thread per element line.
 //    Prologue: conserved -> primitive at every node into shared memory.
 //    Per direction (a runtime loop; the flux is written with the direction's
@@ -1019,7 +1022,7 @@ cudaError_t launch_volume_fx(const double* u, double* du, const double* fs, cons
   return cudaGetLastError();
 }
 
-// meshes of fewer elements than this run the pair-parallel FP64 volume kernel
+// the weak form's volume kernel (kPairParallelElems elements and more)
 template <int D, int N, int EPB>
 cudaError_t launch_volume_weak(const double* u, double* du, const double* fs, const Geom& g,
                                const Tables<double>& tb, unsigned* err, cudaStream_t st,

@@ -294,3 +294,35 @@ def test_gradient_far_from_a_strong_corner(d, N, n, kind):
                             sflux=1).reshape(u.shape)
         size = np.abs(w * jv).sum()
         assert abs(ub[e, v, j] - (w * jv).sum()) <= BAR * size, (e, v, j, ub[e, v, j], size)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("eq,d,N,n,vf,sf", [("euler", 2, 3, (4, 4), "ranocha", "llf"),
+                                            ("euler", 3, 2, (9, 9, 8), "ranocha", "ranocha"),
+                                            ("euler", 3, 3, (4, 3, 3), "ranocha", "hll"),
+                                            ("euler", 3, 3, (9, 9, 8), "ranocha", "llf"),
+                                            ("euler", 3, 5, (9, 9, 8), "ranocha", "llf"),
+                                            ("euler", 2, 4, (26, 25), "central", "hll"),
+                                            ("euler", 3, 4, (9, 9, 8), "central", "llf"),
+                                            ("mhd", 3, 2, (3, 3, 2), "central", "hll"),
+                                            ("mhd", 3, 3, (9, 9, 8), "central", "llf"),
+                                            ("mhd", 3, 4, (9, 9, 8), "ec", "ec"),
+                                            ("mhd", 3, 5, (2, 3, 2), "ec", "ec")])
+@pytest.mark.parametrize("units", [(1.0, 1.0), (1e-20, 1e6), (1e18, 1e-4), (1.0, 1e9)])
+def test_each_variable_by_itself_in_any_units(eq, d, N, n, vf, sf, units):
+    # density and velocity units: the variables' sizes lie up to 18 orders of
+    # magnitude apart, and every one has exponents of its own
+    torch = _gpu()
+    ne, P = int(np.prod(n)), (N + 1) ** d
+    rng = np.random.default_rng([d, N, 11])
+    r, c = units
+    rho = r * np.exp(rng.uniform(-0.5, 0.5, (ne, P)))
+    p = r * c * c * np.exp(rng.uniform(-0.5, 0.5, (ne, P)))
+    v = c * rng.uniform(-0.8, 0.8, (d, ne, P))
+    if eq == "mhd":
+        u = _mhd(rho, v, p, np.sqrt(r) * c * rng.uniform(-0.8, 0.8, (3, ne, P)))
+    else:
+        u = _euler(rho, v, p)
+    got, ref = _rhs(torch, eq, d, N, n, vf, sf, u)
+    err = np.abs(got - ref).max(axis=2) / np.abs(ref).max(axis=2)
+    assert err.max() <= BAR, err.max(axis=0)

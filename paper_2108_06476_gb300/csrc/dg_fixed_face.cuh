@@ -11,7 +11,8 @@
 // FP64 form (surface_nf): beyond that the weaker trace would keep fewer bits
 // than FP64 has. Where HLL takes one trace's own flux, that is evaluated in
 // FP64 from this trace, whatever the other one's size. Measured at 64^3 N = 3 (12.6 M face nodes, LLF): 1.38 ms
-// in FP64, 0.64 ms here (80 registers, 24 warps per SM; 0.72 at 96 registers).
+// in FP64, 0.66 ms here (80 registers, 24 warps per SM; 96 registers were an
+// eighth slower).
 #pragma once
 #include "dg_fixed.cuh"
 

@@ -787,7 +787,7 @@ cudaError_t mhd_volume_epb(const double* u, double* du, const double* fs, const 
                            const Tables<double>& tb, int powell, unsigned* err, cudaStream_t st,
                            const StageFuse& fz) {
   constexpr int P = MLaunch<N>::P;
-  constexpr int SMEM = EPB * kMV * P * (int)sizeof(double);
+  constexpr int SMEM = EPB * MWElem<N>::SLOTS * (int)sizeof(double);
   constexpr int THREADS = 32 * ((EPB * P + 31) / 32);
   auto kern = mhd_volume_weak_kernel<N, EPB>;
   if (SMEM > 48 * 1024) {

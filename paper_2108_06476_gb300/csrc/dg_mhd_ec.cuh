@@ -10,7 +10,7 @@
 // p_t = p + |B|^2/2, [[a]] = a_b - a_a (beta_a/(beta_a + beta_b) = (1 +
 // tanh(D/2))/2), and 1/(2 (gamma-1) beta_ln) = {e} D/sinh(D).
 //
-// Included by dg_mhd.cu. 20^3 N = 4: volume kernel 1.13 ms in FP64, 0.37 here,
+// Included by dg_mhd.cu. 20^3 N = 4: volume kernel 1.13 ms in FP64, 0.33 here,
 // faces 0.18 and 0.07 ms; 4^3 N = 7 (directions on warps of their own): 144 and
 // 42 us.
 #pragma once

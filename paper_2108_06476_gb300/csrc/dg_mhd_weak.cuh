@@ -16,8 +16,8 @@
 // element's units or whose lines hold far smaller momenta, velocities or fields
 // than the element (energy_far, cross_far).
 //
-// Included by dg_mhd.cu. 48^3 N = 3, rhs only: 2.68 ms in FP64, 0.98 here; HLL
-// faces 1.81 and 0.57 ms, LLF 1.55 and 0.51.
+// Included by dg_mhd.cu. 48^3 N = 3, rhs only: 2.68 ms in FP64, 1.11 here (0.98
+// with the lifting in FP64); HLL faces 1.81 and 0.61 ms, LLF 1.55 and 0.55.
 #pragma once
 
 // |m_k| < 2^em, |v_k| < 2^ev, |B_k| < 2^eb, energies below 2^(ee - 1), 1/rho < 2^e1
@@ -211,6 +211,14 @@ __device__ __forceinline__ bool mhd_face_fixed(bool hll, const double* cl, const
   return true;
 }
 
+// shared slots of an element: its fluxes, then the lifting of its face nodes
+template <int N>
+struct MWElem {
+  static constexpr int LINES = (N + 1) * (N + 1);
+  static constexpr int SLOTS =
+      kMV * LINES * (N + 1) > 6 * (kMV + 1) * LINES ? kMV * LINES * (N + 1) : 6 * (kMV + 1) * LINES;
+};
+
 template <int N, int EPB>
 __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31) / 32),
                                   (EPB * (N + 1) * (N + 1) * (N + 1) <= kMhdThreads) ? kMhdMinBlocks
@@ -220,7 +228,7 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
                            StageFuse fz) {
   constexpr int NP = N + 1, P = NP * NP * NP, LINES = NP * NP;
   extern __shared__ __align__(16) unsigned char dg_smem[];
-  fx::i64* sf = reinterpret_cast<fx::i64*>(dg_smem);  // [el][8][P]
+  fx::i64* sf = reinterpret_cast<fx::i64*>(dg_smem);  // [el][8][P] (MWElem)
   __shared__ fx::Limbs s_m[3][NP][NP + 1];            // M, format 62 - ed
   __shared__ double s_m64[3][NP][NP + 1];
   __shared__ double s_lift[2][3];
@@ -323,7 +331,7 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
     const bool weak = in && w.ok && (mm - km > (kCrossBits << 20) ||
                                      (mv - kv) + (mb - kb) > (kCrossBits << 20));
     if (__syncthreads_or(low || weak)) {  // some node may lie too far below
-      uint3* sk = reinterpret_cast<uint3*>(sf + el * kMV * P);
+      uint3* sk = reinterpret_cast<uint3*>(sf + el * MWElem<N>::SLOTS);
       if (in) sk[node] = make_uint3(km, kv, kb);
       __syncthreads();
       bool far = low;
@@ -368,7 +376,7 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
     int l, a;
     line_of<N>(dir, node, l, a);
     if (in) {
-      fx::i64* f = sf + el * kMV * P + node;
+      fx::i64* f = sf + el * MWElem<N>::SLOTS + node;
       if (w.ok) {
         fx::i64 d[kMV];
         mw_flux(q, w, dir, d);
@@ -388,7 +396,7 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
     __syncthreads();
     if (in) {
       const int ns = dir == 0 ? 1 : (dir == 1 ? NP : LINES);
-      const fx::i64* f = sf + el * kMV * P + line_node_rt<3, N>(dir, l, 0);
+      const fx::i64* f = sf + el * MWElem<N>::SLOTS + line_node_rt<3, N>(dir, l, 0);
       if (w.ok) {
 #pragma unroll
         for (int b = 0; b < NP; ++b) {
@@ -413,7 +421,6 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
     }
     if (dir < 2) __syncthreads();
   }
-  if (!in) return;
   // exponents of the fluxes' units: below 2^62 for values below 2^x
   auto unit = [&](int v) {
     return v == 0 ? w.em : v <= 3 ? w.ee + 1 : v == 4 ? w.ev + w.ee + 1
@@ -421,9 +428,35 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
   };
   const long long base = g.nelem * LINES;
   auto face = [&](int dir, int i, int l) {
-    const long long ef = i == N ? e : neighbour(g, e, dir, -1);
+    const long long ef = i == N ? e : neighbour32(g, e, dir, -1);
     return fs + (long long)dir * kMQ * base + ef * LINES + l;
   };
+  // lift F*: a thread takes every P-th of its element's face nodes; the products
+  // go to shared memory by variable. (By nodes, nearly every warp ran all three
+  // directions for a part of its lanes: 64^3 N = 3 2.75 ms, now 2.62; 16^3 N = 5
+  // with faces 0.29 and 0.23)
+  constexpr int FACES = 6 * LINES;
+  constexpr fx::i64 kTooLarge = (fx::i64)(1ULL << 63);
+  fx::i64* sl = sf + el * MWElem<N>::SLOTS;
+  __syncthreads();
+  if (in && w.ok) {
+#pragma unroll 1
+    for (int m = node; m < FACES; m += P) {
+      const int dir = m / (2 * LINES), right = m / LINES % 2, l = m % LINES;
+      const double* src = face(dir, right ? N : 0, l);
+      const fx::Limbs lift = s_liftx[right][dir];
+#pragma unroll
+      for (int v = 0; v <= kMV; ++v) {
+        const double f = src[v * base];
+        const unsigned most = (unsigned)(unit(v) + (int)fx::kBias) << 20;
+        sl[v * FACES + m] = ((unsigned)__double2hiint(f) & 0x7fffffffu) < most
+                                ? fx::mul(lift, fx::limbs(fx::half_fixed(f, unit(v))))
+                                : kTooLarge;
+      }
+    }
+  }
+  __syncthreads();
+  if (!in) return;
   // face values that are added in FP64: bit 9 dir + variable
   static_assert(kMV + 1 == 9, "");
   unsigned late = w.ok ? 0u : 0x7ffffffu;
@@ -433,16 +466,12 @@ __global__ void __launch_bounds__(32 * ((EPB * (N + 1) * (N + 1) * (N + 1) + 31)
       int l, i;
       line_of<N>(dir, node, l, i);
       if (i == N || i == 0) {
-        const double* src = face(dir, i, l);
-        const fx::Limbs lift = s_liftx[i == N][dir];
+        const fx::i64* x = sl + (2 * dir + (i == N)) * LINES + l;
 #pragma unroll
         for (int v = 0; v <= kMV; ++v) {
-          const double f = src[v * base];
-          const unsigned most = (unsigned)(unit(v) + (int)fx::kBias) << 20;
-          if (((unsigned)__double2hiint(f) & 0x7fffffffu) < most)
-            acc[v] = fx::fma64(lift, fx::limbs(fx::half_fixed(f, unit(v))), acc[v]);
-          else
-            late |= 1u << (9 * dir + v);
+          const fx::i64 p = x[v * FACES];
+          if (p != kTooLarge) acc[v] += p;
+          else late |= 1u << (9 * dir + v);
         }
       }
     }

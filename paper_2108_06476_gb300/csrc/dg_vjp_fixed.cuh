@@ -1,8 +1,8 @@
 // The adjoint of Ranocha's volume flux in 64-bit fixed point (FP64 meshes), in
 // the layout and with the scales of dg_fixed_volume.cuh. In FP64 a pair costs
 // 376 instructions of the FP64 unit (64 cycles each): 1.98 ms of the 2.07 ms
-// that one call takes at 16^3 N = 4. Here it costs none: 0.245 ms, the warps'
-// issue slots half busy (20 warps per SM by registers and shared memory). The
+// that one call takes at 16^3 N = 4. Here it costs none: 0.244 ms, the warps'
+// issue slots 44% busy (16 warps per SM by registers and shared memory). The
 // gradient of one rhs there (rhs, face adjoints, this) went from 2.07 to 0.46
 // ms.
 //

@@ -10,9 +10,9 @@
 // differ by more than 2^6, or with non-finite or non-positive values, take the
 // FP64 form (surface_nf): beyond that the weaker trace would keep fewer bits
 // than FP64 has. Where HLL takes one trace's own flux, that is evaluated in
-// FP64 from this trace, whatever the other one's size. Measured at 64^3 N = 3 (12.6 M face nodes, LLF): 1.38 ms
-// in FP64, 0.66 ms here (80 registers, 24 warps per SM; 96 registers were an
-// eighth slower).
+// FP64 from this trace, whatever the other one's size. Measured at 64^3 N = 3
+// (12.6 M face nodes, LLF): 1.38 ms in FP64, 0.66 ms here (80 registers, 24
+// warps per SM; 96 registers were an eighth slower).
 #pragma once
 #include "dg_fixed.cuh"
 
@@ -126,6 +126,21 @@ struct FaceSide {
   i64 vn, p, c2, fm[D], fe;
 };
 
+// The physical flux of a 2D trace (normal component first) in FP64. Out of
+// line, the compiler else issues its few FP64 instructions under predicates in
+// every warp (HLL faces of 185 x 225 elements of degree 3 33 us, 27 so); in 3D
+// it branches, and a call would cost registers (3%).
+struct SideFlux2 {
+  double f[4];
+};
+static __device__ __noinline__ SideFlux2 side_flux_2d(double rho, double mn, double mt, double E,
+                                                      double gm1) {
+  const double c[4] = {rho, mn, mt, E};
+  double rr;
+  const Prim<double, 2> q = prim_rcp<2>(c, gm1, rr);
+  return {{mn, fma(mn, q.v[0], q.p), mn * q.v[1], (E + q.p) * q.v[0]}};
+}
+
 // LLF or HLL from the conserved traces, normal component first. Returns false
 // (f not written) if the FP64 form is due.
 template <int D>
@@ -217,12 +232,18 @@ __device__ __forceinline__ bool face_fixed(bool hll, const double* cl, const dou
     double cc[D + 2];
 #pragma unroll
     for (int v = 0; v < D + 2; ++v) cc[v] = c[v];
-    double rr;
-    const Prim<double, D> q = prim_rcp<D>(cc, gm1, rr);
-    f[0] = cc[1];
+    if constexpr (D == 2) {
+      const SideFlux2 o = side_flux_2d(cc[0], cc[1], cc[2], cc[3], gm1);
 #pragma unroll
-    for (int k = 0; k < D; ++k) f[1 + k] = fma(cc[1], q.v[k], k == 0 ? q.p : 0.0);
-    f[D + 1] = (cc[D + 1] + q.p) * q.v[0];
+      for (int v = 0; v < 4; ++v) f[v] = o.f[v];
+    } else {
+      double rr;
+      const Prim<double, D> q = prim_rcp<D>(cc, gm1, rr);
+      f[0] = cc[1];
+#pragma unroll
+      for (int k = 0; k < D; ++k) f[1 + k] = fma(cc[1], q.v[k], k == 0 ? q.p : 0.0);
+      f[D + 1] = (cc[D + 1] + q.p) * q.v[0];
+    }
     return true;
   }
   const i64 drho = full_fixed(cr[0], er) - full_fixed(cl[0], er);
